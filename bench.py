@@ -49,27 +49,34 @@ PROFILES = os.path.join(ROOT, "profiles")
 
 
 def conv_pairs_per_cell(n):
-    """Unordered (zeta, {xi, zeta - xi}) pairs the FP32 kernel evaluates per cell."""
+    """Unordered (zeta, {xi, zeta - xi}) pairs the FP32 kernel evaluates per cell: one pencil
+    (k1, k2) of each mirror pair, blocks (m1, m2) <= (n1, n2) of the pencil's and its mirror's box,
+    partner indices mod n."""
     h = n // 2
 
-    def lo(k):
-        return max(0, k - h + 1)
+    def mirror(i):
+        return (n - i) % n
 
-    def hi(k):
-        return min(n - 1, k + h)
+    def on(k, m):
+        return 0 <= k - m + h < n
 
-    row = sum(hi(k) - lo(k) + 1 for k in range(n))
+    def onm(k, m):
+        return on(mirror(k), mirror(m))
+
+    row = sum(on(k, m) or onm(k, m) for k in range(n) for m in range(n))
     blocks = 0
     for k1 in range(n):
         for k2 in range(n):
-            for m1 in range(lo(k1), hi(k1) + 1):
-                n1 = k1 - m1 + h
+            if not (k1 > h or (k1 in (0, h) and (k2 == 0 or k2 >= h))):
+                continue
+            for m1 in range(n):
+                n1 = (k1 - m1 + h) % n
                 if m1 > n1:
                     continue
-                for m2 in range(lo(k2), hi(k2) + 1):
-                    if m1 == n1 and m2 > k2 - m2 + h:
+                for m2 in range(n):
+                    if m1 == n1 and m2 > (k2 - m2 + h) % n:
                         continue
-                    blocks += 1
+                    blocks += (on(k1, m1) and on(k2, m2)) or (onm(k1, m1) and onm(k2, m2))
     return blocks * row
 
 

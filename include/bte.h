@@ -136,7 +136,7 @@ const char *bte_last_error(const bte_ctx *ctx);
 /* Tabulate the convolution weights Ghat(xi_m, zeta_k) of Sec. 2.2,
  * Eq. GHat_calc (isotropic b, radial integral cut off at r0 = L, Sec. 3.1) in
  * FP64 on the host for each grid, and store them on the device: the FP32
- * pair-symmetrised table of the fast path and the moment/projection constants
+ * half-spectrum pair table of the fast path and the moment/projection constants
  * of Sec. 3.3. lambda = 0, 1: closed forms of the radial integrals; other
  * lambda in (-3, 1), as Sec. 2.2 prescribes, by quadrature: the power series of
  * the integrand integrated term by term on [0, 1/omega] (exact for the factor
@@ -279,7 +279,7 @@ bte_status bte_graph_count(const bte_ctx *ctx, int64_t *count);
  *                      registers (the b-row stays in registers as packed
  *                      operands for the whole block), 5 = as 4 with the weights
  *                      built on the fly: each warp computes its block's
- *                      pair-symmetrised weights from the radial integrals
+ *                      half-spectrum pair weights from the radial integrals
  *                      I(|k'|^2, |2m' - k'|^2) and J(|m'|^2) (FP32 tables of
  *                      0.5 MB at N = 16, 9 MB at N = 32) instead of streaming
  *                      the stored weight table (elastic tables only). Kinds of
@@ -431,8 +431,8 @@ bte_status bte_learned_stats(bte_ctx *ctx, int64_t *cells, int64_t *fallbacks, d
  *   each), writes per cell (DEVICE, ncells doubles)
  *     ind = ||F[Q](zeta_s) - Qhat(zeta_s)|| / ||Qhat_loss(zeta_s)||
  *   over the sampled modes: F is the forward transform of Sec. 3.2 in FP32,
- *   Qhat the weighted convolution of Sec. 3.2 at those modes (FP32, the fast
- *   path's pair-symmetrised weights) and Qhat_loss the same sum with the loss
+ *   Qhat the weighted convolution of Sec. 3.2 at those modes (FP32, the
+ *   pair-symmetrised weights of those modes) and Qhat_loss the same sum with the loss
  *   term of Ghat only. This is the quantity BTE_LEARNED compares with the
  *   threshold. Asynchronous. Errors: BTE_EINVAL, BTE_ESTATE, BTE_ENOMEM, BTE_ECUDA. */
 bte_status bte_learned_sample(bte_ctx *ctx, int *kk, int cap, int *S);

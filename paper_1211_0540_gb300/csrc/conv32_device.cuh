@@ -1,6 +1,7 @@
 // FP32 weighted convolution of Sec. 3.2 (the O(N^6) hot loop):
 //   Qhat(zeta_k) = dz^3 sum_m Ghat(xi_m, zeta_k) fhat(xi_m) fhat(zeta_k - xi_m),
-// zero extension: only m with n = k - m + N/2 on the grid.
+// zero extension: only m with n = k - m + N/2 on the grid. Q is the real part of
+// its inverse transform, and the kernels evaluate half of the modes zeta_k.
 //
 // Design (GB300, sm_103a):
 // - One warp lane per spatial cell: a warp evaluates the same (zeta, xi) pairs
@@ -9,12 +10,15 @@
 // - Pair symmetry: fhat_m fhat_n serves both m and its partner n, so every
 //   unordered pair is evaluated once with the weight Ghat(k,m) + Ghat(k,n)
 //   (host-packed, see tables.cpp). Half the products, half the weight bytes.
+// - Half spectrum: of the pencils (k1, k2) and (-k1', -k2') only one is
+//   evaluated, with the weights of both (bte_internal.h); partner indices are
+//   then taken mod N.
 // - Work item = (32-cell group, pencil (k1, k2), k3 tile of T outputs). The
 //   item loops over the kept (m1, m2) blocks of the pencil. For each block the
 //   row fhat[m1][m2][:] ("a"), the partner row fhat[n1][n2][:] ("b") and the
 //   block's weights are brought into a per-warp shared-memory ring by TMA bulk
 //   copies (cp.async.bulk, mbarrier transaction counts). The block is then a
-//   fully unrolled (m3, k3) loop: each a-value is reused for all T outputs of
+//   fully unrolled (m3, k3) loop (pair_visit): each a-value is reused for all T outputs of
 //   the tile, each b-value by T pairs along the diagonal k3 - m3, weights are
 //   read as warp-uniform 16-byte shared loads.
 // - Accumulation: plain FP32 FMAs inside `merge` blocks, then Knuth's TwoSum
@@ -28,6 +32,8 @@
 // the common kind sets and holds the host-side configuration, conv32_wide.cu
 // the kernels over the N = 48 kinds (compiled in parallel).
 #pragma once
+
+#include <type_traits>
 
 #include "kernels.h"
 
@@ -87,11 +93,16 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity)
 template <int N_, int T_, int K0_>
 struct Kind {
     static constexpr int N = N_, T = T_, K0 = K0_, H = N_ / 2;
-    static constexpr int lo(int k) { return k - H + 1 > 0 ? k - H + 1 : 0; }
-    static constexpr int hi(int k) { return k + H < N - 1 ? k + H : N - 1; }
     static constexpr int count() {
         int c = 0;
-        for (int j = 0; j < T; ++j) c += hi(K0 + j) - lo(K0 + j) + 1;
+        for (int j = 0; j < T; ++j)
+            for (int m = 0; m < N; ++m) c += pair_kept(K0 + j, m, N);
+        return c;
+    }
+    static constexpr int rank(int i, int j) {  // of the pair of visit i and output j among the block's pairs
+        int c = 0;
+        for (int v = 0; v <= i; ++v)
+            for (int t = 0; t < (v == i ? j : T); ++t) c += pair_visit(K0 + t, v, N, T);
         return c;
     }
     static constexpr int cpad = (count() + 3) & ~3;
@@ -110,33 +121,75 @@ using K48a = Kind<48, 16, 0>;
 using K48b = Kind<48, 16, 16>;
 using K48c = Kind<48, 16, 32>;
 
+// Calls f(integral_constant<int, i>) for i = I .. E - 1, unrolled.
+template <int I, int E, class F>
+__device__ __forceinline__ void static_for(F &&f) {
+    if constexpr (I < E) {
+        f(std::integral_constant<int, I>{});
+        static_for<I + 1, E>(f);
+    }
+}
+
+// The pairs of a block in the order of its weights: begin(m3) at each visit,
+// then pair(j, n3, w) for every output j of the tile that has one. All indices
+// are compile-time constants; the weights are read four at a time. Plain
+// unrolled loops where the tile holds every output (N <= 16); wider grids
+// unroll by recursion, since the compiler leaves loops of that size rolled
+// (N = 32: 14.6 against 2.6 ms on 64 cells).
+// Half way through the visits of a tile narrower than N the partners' indices
+// come round to those of the first visits (for k3 = 0 only): the memory clobber
+// has their values read again instead of kept in registers all the way.
+template <class K, class Begin, class Pair>
+__device__ __forceinline__ void for_pairs(const float4 *W4, Begin &&begin, Pair &&pair) {
+    float4 w4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    if constexpr (K::T == K::N) {
+        int wi = 0;
+#pragma unroll
+        for (int m3 = 0; m3 < K::N; ++m3) {
+            begin(m3);
+#pragma unroll
+            for (int j = 0; j < K::T; ++j)
+                if (pair_kept(j, m3, K::N)) {
+                    if ((wi & 3) == 0) w4 = W4[wi >> 2];
+                    const float w = (wi & 3) == 0 ? w4.x : (wi & 3) == 1 ? w4.y : (wi & 3) == 2 ? w4.z : w4.w;
+                    ++wi;
+                    pair(j, pair_partner(j, m3, K::N), w);
+                }
+        }
+    } else {
+        static_for<0, pair_visits(K::N, K::T)>([&](auto ic) {
+            constexpr int i = decltype(ic)::value, m3 = i % K::N;
+            if (i == K::H) asm volatile("" ::: "memory");
+            begin(m3);
+            static_for<0, K::T>([&](auto jc) {
+                constexpr int j = decltype(jc)::value;
+                if constexpr (pair_visit(K::K0 + j, i, K::N, K::T)) {
+                    constexpr int wi = K::rank(i, j);
+                    if constexpr ((wi & 3) == 0) w4 = W4[wi >> 2];
+                    pair(j, pair_partner(K::K0 + j, m3, K::N),
+                         (wi & 3) == 0 ? w4.x : (wi & 3) == 1 ? w4.y : (wi & 3) == 2 ? w4.z : w4.w);
+                }
+            });
+        });
+    }
+}
+
 // One block: a-row, b-row and weights of stage `st` into the part accumulators.
 template <class K>
 __device__ __forceinline__ void conv_block(const char *st, int lane, float (&part)[2 * K::T]) {
     const float2 *A = reinterpret_cast<const float2 *>(st);
     const float2 *B = A + K::N * kLanes;
-    const float4 *W4 = reinterpret_cast<const float4 *>(B + K::N * kLanes);
-    float4 w4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    int wi = 0;
-#pragma unroll
-    for (int m3 = 0; m3 < K::N; ++m3) {
-        const float2 a = A[m3 * kLanes + lane];
-#pragma unroll
-        for (int j = 0; j < K::T; ++j) {
-            const int n3 = K::K0 + j - m3 + K::H;
-            if (n3 >= 0 && n3 < K::N) {
-                if ((wi & 3) == 0) w4 = W4[wi >> 2];
-                const float w = (wi & 3) == 0 ? w4.x : (wi & 3) == 1 ? w4.y : (wi & 3) == 2 ? w4.z : w4.w;
-                ++wi;
-                const float2 b = B[n3 * kLanes + lane];
-                const float tr = w * a.x, ti = w * a.y;
-                part[2 * j] = fmaf(tr, b.x, part[2 * j]);
-                part[2 * j] = fmaf(-ti, b.y, part[2 * j]);
-                part[2 * j + 1] = fmaf(tr, b.y, part[2 * j + 1]);
-                part[2 * j + 1] = fmaf(ti, b.x, part[2 * j + 1]);
-            }
-        }
-    }
+    float2 a;
+    for_pairs<K>(
+        reinterpret_cast<const float4 *>(B + K::N * kLanes), [&](int m3) { a = A[m3 * kLanes + lane]; },
+        [&](int j, int n3, float w) {
+            const float2 b = B[n3 * kLanes + lane];
+            const float tr = w * a.x, ti = w * a.y;
+            part[2 * j] = fmaf(tr, b.x, part[2 * j]);
+            part[2 * j] = fmaf(-ti, b.y, part[2 * j]);
+            part[2 * j + 1] = fmaf(tr, b.y, part[2 * j + 1]);
+            part[2 * j + 1] = fmaf(ti, b.x, part[2 * j + 1]);
+        });
 }
 
 struct WarpRing {
@@ -153,8 +206,8 @@ __device__ __forceinline__ void issue_block(const WarpRing &r, int s, const Conv
                                             const ConvParams &p, int j) {
     const uint32_t d = p.D[it.table][it.desc_off + j];
     int m1 = (int)(d & 0xffffu), m2 = (int)(d >> 16);
-    int n1 = (int)it.k1 - m1 + K::H, n2 = (int)it.k2 - m2 + K::H;
-    if (m1 >= K::N || m2 >= K::N || n1 < 0 || n1 >= K::N || n2 < 0 || n2 >= K::N) {
+    int n1 = pair_partner((int)it.k1, m1, K::N), n2 = pair_partner((int)it.k2, m2, K::N);
+    if (m1 >= K::N || m2 >= K::N) {
         atomicOr(p.status, ST_BADDESC);
         m1 = m2 = n1 = n2 = 0;  // stay in bounds; the result is flagged as invalid
     }
@@ -173,13 +226,17 @@ __device__ __forceinline__ void issue_block(const WarpRing &r, int s, const Conv
 // The weights of block j of the item, built by the whole warp into the weight
 // slot of stage s from the radial integrals (conv_impl 5, the weights computed
 // on the fly instead of streamed, Sec. 5's remark on storing Ghat). With
-// k' = k - N/2 (likewise m', n' = k' - m') the block's pair weight is
-//   Ghat(k, m) + Ghat(k, n) = [I(|k'|^2, |2m' - k'|^2) - J(|m'|^2)] + [I(..) - J(|n'|^2)],
+// k' = k - N/2 (likewise m', n' = k' - m') Ghat(k, m) + Ghat(k, n) is
+//   [I(|k'|^2, |2m' - k'|^2) - J(|m'|^2)] + [I(..) - J(|n'|^2)],
 // the gain arguments of m and n being equal (|2n' - k'| = |k' - 2m'|); a block
-// that pairs with itself keeps Ghat(k, m). I and J carry sqrt(2/pi) dz^3.
-// Entry e of the tile has the third-component parts of the four invariants
-// precomputed, C[e] = (k3'^2 | (2m3' - k3')^2 << 16, m3'^2 | n3'^2 << 16); the
-// padding up to cpad is 0. Lane l builds entries l, l + 32, ...: all its
+// that pairs with itself keeps Ghat(k, m). I and J carry sqrt(2/pi) dz^3. The
+// half-spectrum weight is that value times the number of on-grid sums the pair
+// belongs to, (k, m) and (k*, m*), times 1/2 on a self-mirrored pencil: where
+// both are on the grid their invariants are equal, and where one is, that one's
+// are taken. Entry e of the tile has the third-component parts of the four
+// invariants precomputed, C[e] = (k3'^2 + 0x4000 if (k, m) + 0x8000 if (k*, m*) is
+// on the grid in the third component | (2m3' - k3')^2 << 16, m3'^2 | n3'^2 << 16);
+// the padding up to cpad is 0. Lane l builds entries l, l + 32, ...: all its
 // table reads are issued before the first weight is formed (one memory
 // latency per block instead of one per entry).
 template <class K>
@@ -187,30 +244,45 @@ __device__ __forceinline__ void gen_weights(const WarpRing &r, int s, const Conv
                                             int lane) {
     constexpr int NE = (K::cpad + kLanes - 1) / kLanes;
     const uint32_t d = p.D[it.table][it.desc_off + jb];
-    const int m1 = (int)(d & 0xffffu), m2 = (int)(d >> 16);
-    const int n1 = (int)it.k1 - m1 + K::H, n2 = (int)it.k2 - m2 + K::H;
-    const bool valid = m1 < K::N && m2 < K::N && n1 >= 0 && n1 < K::N && n2 >= 0 && n2 < K::N;
-    const int k1 = (int)it.k1 - K::H, k2 = (int)it.k2 - K::H, a1 = m1 - K::H, a2 = m2 - K::H;
+    int m1 = (int)(d & 0xffffu), m2 = (int)(d >> 16);
+    int k1 = (int)it.k1, k2 = (int)it.k2;
+    const bool valid = m1 < K::N && m2 < K::N;
+    const bool pair = !(m1 == pair_partner(k1, m1, K::N) && m2 == pair_partner(k2, m2, K::N));
+    const bool on = pair_on_grid(k1, m1, K::N) && pair_on_grid(k2, m2, K::N);
+    const bool onm = pair_on_grid_mirrored(k1, m1, K::N) && pair_on_grid_mirrored(k2, m2, K::N);
+    const float half = pencil_self_mirrored(k1, k2, K::N) ? 0.5f : 1.f;
+    if (!on) {  // the mirrored sum's invariants
+        k1 = mode_mirror(k1, K::N);
+        k2 = mode_mirror(k2, K::N);
+        m1 = mode_mirror(m1, K::N);
+        m2 = mode_mirror(m2, K::N);
+    }
+    k1 -= K::H;
+    k2 -= K::H;
+    const int a1 = m1 - K::H, a2 = m2 - K::H;
     const int p12 = k1 * k1 + k2 * k2;
     const int q12 = (2 * a1 - k1) * (2 * a1 - k1) + (2 * a2 - k2) * (2 * a2 - k2);
     const int sm12 = a1 * a1 + a2 * a2, sn12 = (k1 - a1) * (k1 - a1) + (k2 - a2) * (k2 - a2);
-    const bool pair = !(m1 == n1 && m2 == n2);
     const float *__restrict__ I = p.I32[it.table];
     const float *__restrict__ J = p.J32[it.table];
     const int nq = p.nq[it.table];
     const uint2 *__restrict__ C =
         reinterpret_cast<const uint2 *>(p.E[it.table]) + (K::K0 / K::T) * p.estride[it.table];
-    float g[NE], gm[NE], gn[NE];
+    float g[NE], gm[NE], gn[NE], mult[NE];
 #pragma unroll
     for (int t = 0; t < NE; ++t) {
         const int e = lane + t * kLanes;
-        g[t] = gm[t] = gn[t] = 0.f;
+        g[t] = gm[t] = gn[t] = mult[t] = 0.f;
         if (valid && e < K::count()) {
             const uint2 c = __ldg(C + e);
-            const int pp = p12 + (int)(c.x & 0xffffu), q = q12 + (int)(c.x >> 16);
-            g[t] = __ldg(I + (size_t)pp * nq + q);
-            gm[t] = __ldg(J + sm12 + (int)(c.y & 0xffffu));
-            gn[t] = __ldg(J + sn12 + (int)(c.y >> 16));
+            const int times = (int)(on && (c.x & 0x4000u)) + (int)(onm && (c.x & 0x8000u));
+            if (times) {
+                const int pp = p12 + (int)(c.x & 0x3fffu), q = q12 + (int)(c.x >> 16);
+                mult[t] = half * (float)times;
+                g[t] = __ldg(I + (size_t)pp * nq + q);
+                gm[t] = __ldg(J + sm12 + (int)(c.y & 0xffffu));
+                gn[t] = __ldg(J + sn12 + (int)(c.y >> 16));
+            }
         }
     }
     float *w = reinterpret_cast<float *>(r.base + s * r.stage_bytes + 2 * K::row_bytes);
@@ -218,7 +290,7 @@ __device__ __forceinline__ void gen_weights(const WarpRing &r, int s, const Conv
     for (int t = 0; t < NE; ++t) {
         const int e = lane + t * kLanes;
         const float a = g[t] - gm[t];
-        if (e < K::cpad) w[e] = pair ? a + (g[t] - gn[t]) : a;
+        if (e < K::cpad) w[e] = mult[t] * (pair ? a + (g[t] - gn[t]) : a);
     }
 }
 
@@ -363,27 +435,20 @@ template <class K>
 __device__ __forceinline__ void conv_block_packed(const char *st, int lane, uint64_t (&part)[K::T]) {
     const float2 *A = reinterpret_cast<const float2 *>(st);
     const float2 *B = A + K::N * kLanes;
-    const float4 *W4 = reinterpret_cast<const float4 *>(B + K::N * kLanes);
-    float4 w4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    int wi = 0;
-#pragma unroll
-    for (int m3 = 0; m3 < K::N; ++m3) {
-        const float2 a = A[m3 * kLanes + lane];
-        const uint64_t aR = pk2(a.x, a.x), aI = pk2(a.y, a.y);
-#pragma unroll
-        for (int j = 0; j < K::T; ++j) {
-            const int n3 = K::K0 + j - m3 + K::H;
-            if (n3 >= 0 && n3 < K::N) {
-                if ((wi & 3) == 0) w4 = W4[wi >> 2];
-                const float w = (wi & 3) == 0 ? w4.x : (wi & 3) == 1 ? w4.y : (wi & 3) == 2 ? w4.z : w4.w;
-                ++wi;
-                const float2 b = B[n3 * kLanes + lane];
-                uint64_t pr = fmul2(aR, pk2(b.x, b.y));
-                pr = ffma2(aI, pk2(-b.y, b.x), pr);
-                part[j] = ffma2(pk2(w, w), pr, part[j]);
-            }
-        }
-    }
+    uint64_t aR, aI;
+    for_pairs<K>(
+        reinterpret_cast<const float4 *>(B + K::N * kLanes),
+        [&](int m3) {
+            const float2 a = A[m3 * kLanes + lane];
+            aR = pk2(a.x, a.x);
+            aI = pk2(a.y, a.y);
+        },
+        [&](int j, int n3, float w) {
+            const float2 b = B[n3 * kLanes + lane];
+            uint64_t pr = fmul2(aR, pk2(b.x, b.y));
+            pr = ffma2(aI, pk2(-b.y, b.x), pr);
+            part[j] = ffma2(pk2(w, w), pr, part[j]);
+        });
 }
 
 __device__ __forceinline__ void two_sum(float &hi, float &lo, float p) {
@@ -514,7 +579,6 @@ template <class K>
 __device__ __forceinline__ void conv_block_packed_h(const char *st, int lane, uint64_t (&part)[K::T]) {
     const float2 *A = reinterpret_cast<const float2 *>(st);
     const float2 *B = A + K::N * kLanes;
-    const float4 *W4 = reinterpret_cast<const float4 *>(B + K::N * kLanes);
     uint64_t bb[K::N], bs[K::N];
 #pragma unroll
     for (int n = 0; n < K::N; ++n) {
@@ -522,25 +586,19 @@ __device__ __forceinline__ void conv_block_packed_h(const char *st, int lane, ui
         bb[n] = pk2(b.x, b.y);
         bs[n] = pk2(-b.y, b.x);
     }
-    float4 w4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    int wi = 0;
-#pragma unroll
-    for (int m3 = 0; m3 < K::N; ++m3) {
-        const float2 a = A[m3 * kLanes + lane];
-        const uint64_t aR = pk2(a.x, a.x), aI = pk2(a.y, a.y);
-#pragma unroll
-        for (int j = 0; j < K::T; ++j) {
-            const int n3 = K::K0 + j - m3 + K::H;
-            if (n3 >= 0 && n3 < K::N) {
-                if ((wi & 3) == 0) w4 = W4[wi >> 2];
-                const float w = (wi & 3) == 0 ? w4.x : (wi & 3) == 1 ? w4.y : (wi & 3) == 2 ? w4.z : w4.w;
-                ++wi;
-                uint64_t pr = fmul2(aR, bb[n3]);
-                pr = ffma2(aI, bs[n3], pr);
-                part[j] = ffma2(pk2(w, w), pr, part[j]);
-            }
-        }
-    }
+    uint64_t aR, aI;
+    for_pairs<K>(
+        reinterpret_cast<const float4 *>(B + K::N * kLanes),
+        [&](int m3) {
+            const float2 a = A[m3 * kLanes + lane];
+            aR = pk2(a.x, a.x);
+            aI = pk2(a.y, a.y);
+        },
+        [&](int j, int n3, float w) {
+            uint64_t pr = fmul2(aR, bb[n3]);
+            pr = ffma2(aI, bs[n3], pr);
+            part[j] = ffma2(pk2(w, w), pr, part[j]);
+        });
 }
 
 // Bytes of a warp's shared (hi, lo) sums: 4T x 32 floats with T <= 16.
@@ -736,8 +794,13 @@ __device__ __forceinline__ bool coop_run_sm(WarpRing &r, const ConvItem &it, con
     return !*abort_flag;
 }
 
+// Shared memory allows 3 CTAs per SM for the kinds of N <= 16 (168 registers) and
+// 2 for the wider ones, which then take up to 255 registers (at 168 they spill:
+// 24, 64 cells: 437 against 398 us for the 255-register variant 3).
+constexpr int sums_min_ctas(unsigned mask) { return mask & ~7u ? 2 : 3; }
+
 template <unsigned MASK, bool OTF = false>
-__global__ void __launch_bounds__(128, 3) conv32_sums_kernel(ConvParams p) {
+__global__ void __launch_bounds__(128, sums_min_ctas(MASK)) conv32_sums_kernel(ConvParams p) {
     extern __shared__ __align__(128) char smem[];
     __shared__ int s_item, s_abort, s_last, s_nitems;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;

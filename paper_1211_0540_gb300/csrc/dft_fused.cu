@@ -12,7 +12,7 @@
 // FMA operands; shared memory is touched once per value and pass (rows
 // padded to N + 1 against bank conflicts). The forward kernel writes fhat
 // straight into the group layout of the convolution ([group][k][lane]); the
-// inverse kernel reads Qhat from it and applies the conservation projection
+// inverse kernel reads Qhat's stored pencils from it and applies the conservation projection
 // of Sec. 3.3 (and optionally the Heun update) before the single write of Q.
 //
 // FP64 runs at about 1/70 of the FP32 rate here, so the five moments of Qt
@@ -311,11 +311,12 @@ dft_inv_fused_kernel(const float2 *__restrict__ G, const int64_t *__restrict__ s
     const float2(&rt)[N] = CRoot<N>::get();
     const bool act = t < NP;
     const float2 *g = G + s.eoff + (int64_t)(sl / kLanes) * M * kLanes + (sl % kLanes);
-    if (act) {  // along k1, pencil (k2, k3), from the group layout
-        const int pk = (r * JR + t / N) * N + t % N;
+    if (act) {  // along k1, pencil (k2, k3), from the group layout (the stored half of the pencils; the rest is 0)
+        const int pk = (r * JR + t / N) * N + t % N, k2 = pk / N;
         float2 xx[N], yy[N];
 #pragma unroll
-        for (int k = 0; k < N; ++k) xx[k] = g[(int64_t)(k * NN + pk) * kLanes];
+        for (int k = 0; k < N; ++k)
+            xx[k] = pencil_stored(k, k2, N) ? g[(int64_t)(k * NN + pk) * kLanes] : make_float2(0.f, 0.f);
         pencil_cc<N, false>(xx, yy, rt);
         const int kl = t / N, k3 = t % N;
 #pragma unroll

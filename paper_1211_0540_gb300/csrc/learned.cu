@@ -25,7 +25,7 @@ namespace {
 
 // One CTA of kIndWarps warps per (sampled pencil, group), lane = cell: the
 // warps work in pairs, each pair takes the pencil's kept (m1, m2) blocks in
-// turn (the block layout of the FP32 table: unordered pairs, weights
+// turn (unordered pairs, weights
 // Ghat(k,m) + Ghat(k,n)) and each warp of a pair half of the N outputs k3,
 // with the full and the loss weights side by side: the a and b rows of a block
 // are loaded into registers by both warps of its pair. Half the outputs per
@@ -100,8 +100,8 @@ indicator_kernel(const float2 *__restrict__ F, const float2 *__restrict__ QN, co
             bv[i] = make_float2(b2.x, b2.y);
             bv[i + 1] = make_float2(b2.z, b2.w);
         }
-        const float4 *wf = reinterpret_cast<const float4 *>(Wfull + pen.wofs_full + (size_t)b * cpad);
-        const float4 *wl = reinterpret_cast<const float4 *>(Wloss + pen.wofs_loss + (size_t)b * cpad);
+        const float4 *wf = reinterpret_cast<const float4 *>(Wfull + pen.wofs + (size_t)b * cpad);
+        const float4 *wl = reinterpret_cast<const float4 *>(Wloss + pen.wofs + (size_t)b * cpad);
         if (jh == 0) indicator_block<N, 0>(av, bv, wf, wl, acc);
         else indicator_block<N, 1>(av, bv, wf, wl, acc);
     }
@@ -382,34 +382,46 @@ int build_indicator_table(const Table &t, int modes, uint64_t seed, IndicatorTab
         const int kk = (k1 + h) * N + (k2 + h);
         if (std::find(kks.begin(), kks.end(), kk) == kks.end()) kks.push_back(kk);
     }
-    // loss weights of the sampled pencils in the FP32 table's block layout (one k3 tile, N <= 16)
-    const int cpad = t.cpad[0];
-    std::vector<float> wl;
+    // the sampled pencils' own blocks: the modes are compared one by one, so the
+    // sums run over the pencil's box with the plain pair weights Ghat(k, m) +
+    // Ghat(k, n) (blocks (m1, m2) <= (n1, n2); a block that pairs with itself
+    // keeps Ghat(k, m)), the full ones and those of the loss term, per block m3
+    // ascending, then k3, padded to 16 bytes
+    int cpad = 0;
+    for (int m3 = 0; m3 < N; ++m3)
+        for (int k3 = 0; k3 < N; ++k3) cpad += pair_on_grid(k3, m3, N);
+    cpad = (cpad + 3) & ~3;
+    std::vector<float> wf, wl;
     std::vector<IndPencil> pens;
-    std::vector<uint32_t> desc(t.n_desc);
-    if (cudaMemcpy(desc.data(), t.d_desc, sizeof(uint32_t) * t.n_desc, cudaMemcpyDeviceToHost) != cudaSuccess) {
-        cudaGetLastError();
-        return -1;
-    }
+    std::vector<uint32_t> desc;
     for (int kk : kks) {
+        const int k1 = kk / N, k2 = kk % N;
         IndPencil pn{};
         pn.kk = kk;
-        pn.desc_off = (int)t.desc_off[kk];
-        pn.nblocks = (int)t.nblocks[kk];
-        pn.wofs_full = t.wofs[kk];
-        pn.wofs_loss = wl.size();
-        const int k1 = kk / N, k2 = kk % N;
+        pn.desc_off = (int)desc.size();
+        pn.wofs = wl.size();
+        for (int m1 = 0; m1 < N; ++m1)
+            for (int m2 = 0; m2 < N; ++m2) {
+                const int n1 = k1 - m1 + h, n2 = k2 - m2 + h;
+                if (n1 < 0 || n1 >= N || n2 < 0 || n2 >= N || m1 > n1 || (m1 == n1 && m2 > n2)) continue;
+                desc.push_back((uint32_t)m1 | ((uint32_t)m2 << 16));
+            }
+        pn.nblocks = (int)desc.size() - pn.desc_off;
         for (int b = 0; b < pn.nblocks; ++b) {
             const uint32_t dd = desc[pn.desc_off + b];
             const int m1 = (int)(dd & 0xffffu), m2 = (int)(dd >> 16), n1 = k1 - m1 + h, n2 = k2 - m2 + h;
             const bool pair = !(m1 == n1 && m2 == n2);
             const size_t base = wl.size();
             wl.resize(base + cpad, 0.0f);
+            wf.resize(base + cpad, 0.0f);
             size_t wi = base;
             for (int m3 = 0; m3 < N; ++m3)
                 for (int k3 = 0; k3 < N; ++k3) {
                     const int n3 = k3 - m3 + h;
                     if (n3 < 0 || n3 >= N) continue;
+                    double full = t.ghat(k1, k2, k3, m1, m2, m3);
+                    if (pair) full += t.ghat(k1, k2, k3, n1, n2, n3);
+                    wf[wi] = (float)(full * dz3);
                     const int sm = (m1 - h) * (m1 - h) + (m2 - h) * (m2 - h) + (m3 - h) * (m3 - h);
                     double g = -c * t.J[sm];
                     if (pair) {
@@ -423,7 +435,13 @@ int build_indicator_table(const Table &t, int modes, uint64_t seed, IndicatorTab
     }
     out.S = S;
     out.kks = kks;
+    out.cpad = cpad;
     cudaError_t e = cudaMalloc(&out.d_wloss, sizeof(float) * std::max<size_t>(wl.size(), 4));
+    if (e == cudaSuccess) e = cudaMalloc(&out.d_wfull, sizeof(float) * std::max<size_t>(wf.size(), 4));
+    if (e == cudaSuccess) e = cudaMalloc(&out.d_desc, sizeof(uint32_t) * std::max<size_t>(desc.size(), 1));
+    if (e == cudaSuccess) e = cudaMemcpy(out.d_wfull, wf.data(), sizeof(float) * wf.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+        e = cudaMemcpy(out.d_desc, desc.data(), sizeof(uint32_t) * desc.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMalloc(&out.d_pen, sizeof(IndPencil) * S);
     if (e == cudaSuccess) e = cudaMemcpy(out.d_wloss, wl.data(), sizeof(float) * wl.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(out.d_pen, pens.data(), sizeof(IndPencil) * S, cudaMemcpyHostToDevice);
@@ -441,8 +459,12 @@ int build_indicator_table(const Table &t, int modes, uint64_t seed, IndicatorTab
 }
 
 void free_indicator_table(IndicatorTable &t) {
+    cudaFree(t.d_wfull);
+    cudaFree(t.d_desc);
     cudaFree(t.d_wloss);
     cudaFree(t.d_pen);
+    t.d_wfull = nullptr;
+    t.d_desc = nullptr;
     cudaFree(t.d_kk);
     t.d_wloss = nullptr;
     t.d_pen = nullptr;
@@ -474,17 +496,17 @@ void launch_indicator(const IndicatorTable &it, const Table &t, const float2 *F,
     cudaMemsetAsync(cnt, 0, sizeof(unsigned) * items, st);
     switch (t.N) {
         case 8:
-            indicator_kernel<8><<<grid, 32 * kIndWarps, ind_smem<8>(), st>>>(F, QN, t.d_w32, it.d_wloss, t.d_desc,
-                                                                           it.d_pen, t.cpad[0], eoff, nslots, err2, den2, part, cnt);
+            indicator_kernel<8><<<grid, 32 * kIndWarps, ind_smem<8>(), st>>>(F, QN, it.d_wfull, it.d_wloss, it.d_desc,
+                                                                           it.d_pen, it.cpad, eoff, nslots, err2, den2, part, cnt);
             break;
         case 12:
-            indicator_kernel<12><<<grid, 32 * kIndWarps, ind_smem<12>(), st>>>(F, QN, t.d_w32, it.d_wloss, t.d_desc,
-                                                                             it.d_pen, t.cpad[0], eoff, nslots, err2,
+            indicator_kernel<12><<<grid, 32 * kIndWarps, ind_smem<12>(), st>>>(F, QN, it.d_wfull, it.d_wloss, it.d_desc,
+                                                                             it.d_pen, it.cpad, eoff, nslots, err2,
                                                                              den2, part, cnt);
             break;
         default:
-            indicator_kernel<16><<<grid, 32 * kIndWarps, ind_smem<16>(), st>>>(F, QN, t.d_w32, it.d_wloss, t.d_desc,
-                                                                             it.d_pen, t.cpad[0], eoff, nslots, err2,
+            indicator_kernel<16><<<grid, 32 * kIndWarps, ind_smem<16>(), st>>>(F, QN, it.d_wfull, it.d_wloss, it.d_desc,
+                                                                             it.d_pen, it.cpad, eoff, nslots, err2,
                                                                              den2, part, cnt);
             break;
     }

@@ -8,18 +8,21 @@
 
 namespace bte {
 
-// Sampled pencils of the indicator: for pencil i, the kept (m1, m2) blocks of
-// zeta pencil kk = k1 N + k2 (descriptors and full weights of the FP32 table)
-// and the loss-term weights of the same blocks (d_wloss + wofs_loss).
+// Sampled pencils of the indicator: for pencil i, the (m1, m2) blocks of zeta
+// pencil kk = k1 N + k2 (d_desc + desc_off) and their full and loss-term pair
+// weights (d_wfull, d_wloss + wofs, cpad floats a block).
 struct IndPencil {
     int kk, desc_off, nblocks, pad;
-    uint64_t wofs_full, wofs_loss;
+    uint64_t wofs;
 };
 
 struct IndicatorTable {
     int S = 0;                     // sampled pencils (S x N sampled modes)
     std::vector<int> kks;          // host copy of the sampled pencils (k1 N + k2), drawing order
-    float *d_wloss = nullptr;      // loss weights of the sampled pencils (pair-symmetrised, times dz^3)
+    int cpad = 0;                  // floats per block of weights
+    uint32_t *d_desc = nullptr;    // m1 | (m2 << 16)
+    float *d_wfull = nullptr;      // weights of the sampled pencils (pair-symmetrised, times dz^3)
+    float *d_wloss = nullptr;      // the same of the loss term
     IndPencil *d_pen = nullptr;
     int *d_kk = nullptr;           // the sampled pencils' k1 N + k2
 };

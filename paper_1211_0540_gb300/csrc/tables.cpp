@@ -22,17 +22,20 @@
 // lattice of I, so the gain integral is evaluated per pair (closed form, or
 // quadrature where it would cancel); J is unchanged.
 //
-// FP32 pair-symmetrised layout (the fast path). For a zeta point k the terms m
-// and n = k - m + N/2 (zeta - xi_m = xi_n) multiply the same product
+// FP32 pair layout (the fast path). For a zeta point k the terms m and
+// n = k - m + N/2 (zeta - xi_m = xi_n) multiply the same product
 // fhat_m fhat_n, so the sum over m is taken over unordered pairs with the
-// weight Ghat(k, m) + Ghat(k, n). Pairs are grouped by the first two
-// components: for a "pencil" (k1, k2) the kept blocks are the (m1, m2) of the
-// valid box with (m1, m2) <= (n1, n2) lexicographically; a block with
-// (m1, m2) == (n1, n2) pairs with itself and keeps the plain weight Ghat(k, m)
-// over all m3. Inside a block, for a k3 tile [K0, K0 + T), the weights are
-// stored in the order the kernel consumes them: m3 ascending, then k3
-// ascending, skipping (k3, m3) whose partner n3 = k3 - m3 + N/2 is off the
-// grid. Every weight already carries the trapezoid factor dz^3.
+// weight W(k, m) + W(k, n), W the half-spectrum weight (bte_internal.h), on the
+// pencils (k1, k2) that are stored. Pairs are grouped by the first two
+// components: the kept blocks of a pencil are the (m1, m2) of the boxes of
+// (k1, k2) and of its mirror with (m1, m2) <= (n1, n2) lexicographically, n
+// taken mod N; a block with (m1, m2) == (n1, n2) pairs with itself and keeps
+// the plain weight W(k, m) over all m3. Inside a block, for a k3 tile
+// [K0, K0 + T), the weights are stored in the order the kernel consumes them:
+// m3 in the order of pair_visit, then k3 ascending, skipping (k3, m3) that no
+// block has; a pair that is on the grid in k3 but not in this block has
+// weight 0 (4 % of the entries at N = 16). Every weight already carries the
+// trapezoid factor dz^3.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -137,6 +140,19 @@ double Table::ghat(int k1, int k2, int k3, int m1, int m2, int m3) const {
     return std::sqrt(2.0 / kPi) * (gain_inelastic(a, b) - J[s]);
 }
 
+// Where both sums hold the pair, their weights are equal: the two lifts of an
+// index 0 to the mesh (-N/2 and, mirrored, +N/2) never hold it both.
+double Table::half_weight(int k1, int k2, int k3, int m1, int m2, int m3) const {
+    const bool on = pair_on_grid(k1, m1, N) && pair_on_grid(k2, m2, N) && pair_on_grid(k3, m3, N);
+    const bool onm = pair_on_grid_mirrored(k1, m1, N) && pair_on_grid_mirrored(k2, m2, N) &&
+                     pair_on_grid_mirrored(k3, m3, N);
+    if (!on && !onm) return 0.0;
+    const double g = on ? ghat(k1, k2, k3, m1, m2, m3)
+                        : ghat(mode_mirror(k1, N), mode_mirror(k2, N), mode_mirror(k3, N), mode_mirror(m1, N),
+                               mode_mirror(m2, N), mode_mirror(m3, N));
+    return g * (on && onm ? 2.0 : 1.0) * (pencil_self_mirrored(k1, k2, N) ? 0.5 : 1.0);
+}
+
 // The closed form loses digits when a b L^2 is small (C(a - b) and C(a + b)
 // nearly cancel); such pairs (|xi - beta zeta / 2| near 0, which the elastic
 // lattice never produces) take the quadrature rule instead.
@@ -199,24 +215,25 @@ int build_table(Table &t, std::string &err) {
         quadrature_tables(t, hz);
     }
 
-    // pencil descriptors: kept (m1, m2) blocks
+    // descriptors of the stored pencils: kept (m1, m2) blocks
     std::vector<uint32_t> desc;
     t.desc_off.assign(N * N, 0);
     t.nblocks.assign(N * N, 0);
     for (int k1 = 0; k1 < N; ++k1)
         for (int k2 = 0; k2 < N; ++k2) {
             t.desc_off[k1 * N + k2] = (uint32_t)desc.size();
+            if (!pencil_stored(k1, k2, N)) continue;
             uint32_t nb = 0;
-            for (int m1 = box_lo(k1, N); m1 <= box_hi(k1, N); ++m1) {
-                int n1 = k1 - m1 + h;
-                if (m1 > n1) continue;
-                for (int m2 = box_lo(k2, N); m2 <= box_hi(k2, N); ++m2) {
-                    int n2 = k2 - m2 + h;
-                    if (m1 == n1 && m2 > n2) continue;
+            for (int m1 = 0; m1 < N; ++m1)
+                for (int m2 = 0; m2 < N; ++m2) {
+                    const int n1 = pair_partner(k1, m1, N), n2 = pair_partner(k2, m2, N);
+                    if (m1 > n1 || (m1 == n1 && m2 > n2)) continue;
+                    if (!(pair_on_grid(k1, m1, N) && pair_on_grid(k2, m2, N)) &&
+                        !(pair_on_grid_mirrored(k1, m1, N) && pair_on_grid_mirrored(k2, m2, N)))
+                        continue;
                     desc.push_back((uint32_t)m1 | ((uint32_t)m2 << 16));
                     ++nb;
                 }
-            }
             t.nblocks[k1 * N + k2] = nb;
         }
     t.n_desc = desc.size();
@@ -227,7 +244,8 @@ int build_table(Table &t, std::string &err) {
     size_t total = 0;
     for (int tile = 0; tile < t.ntiles; ++tile) {
         int K0 = tile * T, cnt = 0;
-        for (int j = 0; j < T; ++j) cnt += box_len(K0 + j, N);
+        for (int j = 0; j < T; ++j)
+            for (int m = 0; m < N; ++m) cnt += pair_kept(K0 + j, m, N);
         t.cpad[tile] = (cnt + 3) & ~3;
         for (int kk = 0; kk < N * N; ++kk) {
             t.wofs[(size_t)tile * N * N + kk] = total;
@@ -309,7 +327,7 @@ int build_table(Table &t, std::string &err) {
     t.n_tmpl = (int)tmpl.size();
 
     // on-the-fly weights (elastic tables): radial integrals in FP32 with the
-    // constant factor, and each tile's entry list (m3 ascending, then k3)
+    // constant factor, and each tile's entry list (in the order of pair_visit, then k3)
     std::vector<float> I32, J32;
     std::vector<uint16_t> etab;
     if (t.beta == 1.0) {
@@ -320,18 +338,22 @@ int build_table(Table &t, std::string &err) {
         for (size_t i = 0; i < t.J.size(); ++i) J32[i] = (float)(cw * t.J[i]);
         // per entry (m3, k3) of a tile, in the kernel's order: the third
         // components of the invariants, (k3'^2 | (2m3' - k3')^2 << 16,
-        // m3'^2 | n3'^2 << 16) with n3' = k3' - m3', as four 16-bit fields
+        // m3'^2 | n3'^2 << 16) with n3' = k3' - m3', as four 16-bit fields, of
+        // (k3, m3) where it is on the grid (+ 0x4000 in the first field), else of
+        // its mirror (+ 0x8000; both bits where both are, the squares are equal)
         t.estride = std::max(t.cpad[0], std::max(t.cpad[1], t.cpad[2]));
         etab.assign((size_t)t.ntiles * t.estride * 4, 0);
         for (int tile = 0; tile < t.ntiles; ++tile) {
             int e = 0;
-            for (int m3 = 0; m3 < N; ++m3)
+            for (int i = 0; i < pair_visits(N, T); ++i)
                 for (int j = 0; j < T; ++j) {
-                    const int k3 = tile * T + j, n3 = k3 - m3 + h;
-                    if (n3 < 0 || n3 >= N) continue;
-                    const int kp = k3 - h, mp = m3 - h, np3 = kp - mp;
+                    const int k3 = tile * T + j, m3 = i % N;
+                    if (!pair_visit(k3, i, N, T)) continue;
+                    const bool on = pair_on_grid(k3, m3, N);
+                    const int kp = (on ? k3 : mode_mirror(k3, N)) - h, mp = (on ? m3 : mode_mirror(m3, N)) - h;
+                    const int np3 = kp - mp;
                     uint16_t *c = &etab[((size_t)tile * t.estride + e++) * 4];
-                    c[0] = (uint16_t)(kp * kp);
+                    c[0] = (uint16_t)(kp * kp + (on ? 0x4000 : 0) + (pair_on_grid_mirrored(k3, m3, N) ? 0x8000 : 0));
                     c[1] = (uint16_t)((2 * mp - kp) * (2 * mp - kp));
                     c[2] = (uint16_t)(mp * mp);
                     c[3] = (uint16_t)(np3 * np3);
@@ -382,11 +404,11 @@ int build_table(Table &t, std::string &err) {
     return BTE_OK;
 }
 
-// The FP32 pair-symmetrised weights (times dz^3) in the kernel's layout:
-// per (tile, k1, k2) its kept blocks, per block m3 ascending then k3.
+// The FP32 half-spectrum pair weights (times dz^3) in the kernel's layout:
+// per (tile, k1, k2) its kept blocks, per block in the order of pair_visit, then k3.
 int build_table_fp32(Table &t, std::string &err) {
     if (t.d_w32) return BTE_OK;
-    const int N = t.N, h = N / 2, T = conv_kind(t.kind0).T;
+    const int N = t.N, T = conv_kind(t.kind0).T;
     const double dz3 = t.dz * t.dz * t.dz;
     std::vector<float> w32(t.n_w32, 0.0f);
 #pragma omp parallel for collapse(2) schedule(dynamic, 1)
@@ -396,15 +418,15 @@ int build_table_fp32(Table &t, std::string &err) {
             size_t o = t.wofs[(size_t)tile * N * N + kk];
             for (uint32_t b = 0; b < t.nblocks[kk]; ++b) {
                 uint32_t d = t.desc_host[t.desc_off[kk] + b];
-                int m1 = d & 0xffff, m2 = d >> 16, n1 = k1 - m1 + h, n2 = k2 - m2 + h;
+                int m1 = d & 0xffff, m2 = d >> 16, n1 = pair_partner(k1, m1, N), n2 = pair_partner(k2, m2, N);
                 bool pair = !(m1 == n1 && m2 == n2);
                 size_t wi = o + (size_t)b * t.cpad[tile];
-                for (int m3 = 0; m3 < N; ++m3)
+                for (int i = 0; i < pair_visits(N, T); ++i)
                     for (int j = 0; j < T; ++j) {
-                        int k3 = K0 + j, n3 = k3 - m3 + h;
-                        if (n3 < 0 || n3 >= N) continue;
-                        double g = t.ghat(k1, k2, k3, m1, m2, m3);
-                        if (pair) g += t.ghat(k1, k2, k3, n1, n2, n3);
+                        int k3 = K0 + j, m3 = i % N;
+                        if (!pair_visit(k3, i, N, T)) continue;
+                        double g = t.half_weight(k1, k2, k3, m1, m2, m3);
+                        if (pair) g += t.half_weight(k1, k2, k3, n1, n2, pair_partner(k3, m3, N));
                         w32[wi++] = (float)(g * dz3);
                     }
             }
