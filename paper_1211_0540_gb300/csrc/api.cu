@@ -529,8 +529,7 @@ bte_status prepare(bte_ctx *c, Batch *B, int mode, bool step, bool transport) {
     if (mode == BTE_FP64_PLAIN) {
         for (const Segment &sg : B->segs) {
             if (c->tables[sg.table]->N > 32)
-                return fail(c, BTE_EINVAL, "the plain FP64 operator is limited to N <= 32 (its table holds 8 V(N) "
-                                           "bytes: 41 GB at N = 48)");
+                return fail(c, BTE_EINVAL, "the plain FP64 operator is limited to N <= 32");
             int r = build_table_fp64(*c->tables[sg.table], c->err);
             if (r != BTE_OK) return (bte_status)r;
         }
@@ -600,11 +599,11 @@ bte_status enqueue_collide(bte_ctx *c, Batch *B, const double *f, double *Q, int
         for (const Segment &sg : B->segs) {
             const Table *t = c->tables[sg.table];
             if (2 * sg.nvalid <= sg.nslots)  // groups less than half full: lanes over the box instead of cells
-                launch_conv64_cells((const double2 *)c->scratch[SC_F], (double2 *)c->scratch[SC_QH], t->d_w64,
-                                    t->d_w64_off, B->d_slot_off, sg.s0, sg.nslots, t->N, sg.eoff, st);
+                launch_conv64_cells((const double2 *)c->scratch[SC_F], (double2 *)c->scratch[SC_QH], *t,
+                                    B->d_slot_off, sg.s0, sg.nslots, sg.eoff, st);
             else
-                launch_conv64((const double2 *)c->scratch[SC_F], (double2 *)c->scratch[SC_QH], t->d_w64,
-                              t->d_w64_off, t->N, sg.eoff, sg.nslots / kLanes, st);
+                launch_conv64((const double2 *)c->scratch[SC_F], (double2 *)c->scratch[SC_QH], *t, sg.eoff,
+                              sg.nslots / kLanes, st);
             count_launches(c, 1);
         }
         prof_end(c, on, pe_conv, st);

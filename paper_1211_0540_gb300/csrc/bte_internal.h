@@ -90,6 +90,16 @@ struct ConvItem {
 };
 static_assert(sizeof(ConvItem) == 32, "ConvItem layout");
 
+// One zeta point of the FP64 convolution: for each of its pencil's blocks
+// (desc_off ..) the m_count values of m3 from m_first on, mod N, with one
+// weight each from woff on.
+struct Zeta64 {
+    uint64_t woff;
+    uint32_t desc_off;
+    uint16_t nblocks, k1, k2, k3, m_first, m_count;
+};
+static_assert(sizeof(Zeta64) == 24, "Zeta64 layout");
+
 // Per-grid weight table and constants.
 struct Table {
     int N = 0;
@@ -106,9 +116,11 @@ struct Table {
     size_t n_w32 = 0, n_desc = 0;
     float *d_w32 = nullptr;
     uint32_t *d_desc = nullptr;          // m1 | (m2 << 16)
-    // FP64 plain table (times dz^3), valid boxes, zeta-major; built lazily.
+    // FP64 pair weights (times dz^3), zeta-major, and the zeta points of the stored
+    // pencils, costliest first; built lazily.
     double *d_w64 = nullptr;
-    uint64_t *d_w64_off = nullptr;       // per k (M + 1 entries)
+    Zeta64 *d_zeta64 = nullptr;
+    int n_zeta64 = 0;
     size_t n_w64 = 0;
     // On-the-fly weights (beta = 1): I and J in FP32 times sqrt(2/pi) dz^3, and
     // per k3 tile and block entry (kernel order) the third components of the

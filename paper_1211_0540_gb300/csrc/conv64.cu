@@ -1,92 +1,124 @@
-// Plain FP64 weighted convolution (Sec. 3.2), the comparator operator:
-//   Qhat(zeta_k) = sum_{m in box(k)} [Ghat(xi_m, zeta_k) dz^3] fhat_m fhat_{k-m+N/2},
-// a direct double sum over the valid box of each zeta point with FP64
-// weights and FP64 arithmetic. One warp per (32-cell group, zeta point), one
-// lane per cell: the weight stream is warp-uniform and the fhat rows of the
-// group layout are read coalesced. No symmetry, tiling or compensation.
+// FP64 weighted convolution (Sec. 3.2), the comparator operator: the direct
+// double sum with FP64 weights and FP64 arithmetic,
+//   Qhat(zeta_k) = sum over unordered pairs {m, n} of [W(k, m) + W(k, n)] fhat_m fhat_n,
+// at the modes of the stored pencils (half spectrum, bte_internal.h). The FP64
+// units bound it (two FMAs per SM and clock against 128 in FP32), six
+// operations a pair, so what counts is the number of pairs: 2.42 M per cell at
+// N = 16 instead of the 7.08 M terms of the plain sum over m (128 cells: 10.09
+// -> 3.2 ms; six warp instructions of 16 clocks a pair on 152 SMs are 2.95 ms).
+// A zeta point's terms are listed block by block ((m1, m2) of its pencil), its
+// m_count values of m3 from m_first on (mod N), with the weights in that order;
+// zeta points are sorted by cost, the largest first, against a long tail.
 #include "kernels.h"
 
 namespace bte {
 
-__global__ void conv64_plain_kernel(const double2 *__restrict__ F, double2 *__restrict__ Qh,
-                                    const double *__restrict__ W,
-                                    const uint64_t *__restrict__ Woff, int N, int64_t eoff) {
+namespace {
+constexpr int kWarps64 = 4;  // warps per CTA
+}
+
+// One warp per (zeta point, 32-cell group), one lane per cell: the weight is
+// warp-uniform and the fhat rows of the group layout are read coalesced. The
+// groups of one zeta point are neighbours, so they share its weights in L1.
+__global__ void __launch_bounds__(32 * kWarps64) conv64_plain_kernel(const double2 *__restrict__ F,
+                                                                     double2 *__restrict__ Qh,
+                                                                     const double *__restrict__ W,
+                                                                     const Zeta64 *__restrict__ Z, int nz,
+                                                                     const uint32_t *__restrict__ D, int N,
+                                                                     int64_t eoff, int ngroups) {
     const int lane = threadIdx.x & 31;
-    const int M = N * N * N, h = N / 2;
-    const int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (k >= M) return;
-    const int g = blockIdx.y;
-    const double2 *Fg = F + eoff + (int64_t)g * M * kLanes;
-    const int k1 = k / (N * N), k2 = (k / N) % N, k3 = k % N;
-    const int lo1 = max(0, k1 - h + 1), hi1 = min(N - 1, k1 + h);
-    const int lo2 = max(0, k2 - h + 1), hi2 = min(N - 1, k2 + h);
-    const int lo3 = max(0, k3 - h + 1), hi3 = min(N - 1, k3 + h);
-    const double *w = W + Woff[k];
+    const int64_t M = (int64_t)N * N * N;
+    const int64_t id = (int64_t)blockIdx.x * kWarps64 + (threadIdx.x >> 5);
+    if (id >= (int64_t)nz * ngroups) return;
+    const int g = (int)(id % ngroups);
+    const Zeta64 z = Z[id / ngroups];
+    const double2 *Fg = F + eoff + (int64_t)g * M * kLanes + lane;
+    const double *w = W + z.woff;
+    const int k1 = z.k1, k2 = z.k2, cnt = z.m_count, n3_first = pair_partner(z.k3, z.m_first, N);
     double re = 0.0, im = 0.0;
-    for (int m1 = lo1; m1 <= hi1; ++m1)
-        for (int m2 = lo2; m2 <= hi2; ++m2)
-            for (int m3 = lo3; m3 <= hi3; ++m3) {
-                const double g_ = *w++;
-                const double2 a = Fg[(int64_t)((m1 * N + m2) * N + m3) * kLanes + lane];
-                const int n = ((k1 - m1 + h) * N + (k2 - m2 + h)) * N + (k3 - m3 + h);
-                const double2 b = Fg[(int64_t)n * kLanes + lane];
-                re += g_ * (a.x * b.x - a.y * b.y);
-                im += g_ * (a.x * b.y + a.y * b.x);
-            }
-    Qh[eoff + (int64_t)g * M * kLanes + (int64_t)k * kLanes + lane] = make_double2(re, im);
+    for (int b = 0; b < z.nblocks; ++b) {
+        const uint32_t d = D[z.desc_off + b];
+        const int m1 = (int)(d & 0xffffu), m2 = (int)(d >> 16);
+        const double2 *A = Fg + (int64_t)((m1 * N + m2) * N) * kLanes;
+        const double2 *B = Fg + (int64_t)((pair_partner(k1, m1, N) * N + pair_partner(k2, m2, N)) * N) * kLanes;
+        int m3 = z.m_first, n3 = n3_first;
+#pragma unroll 4
+        for (int t = 0; t < cnt; ++t) {
+            const double g_ = w[t];
+            const double2 a = A[m3 * kLanes], c = B[n3 * kLanes];
+            re += g_ * (a.x * c.x - a.y * c.y);
+            im += g_ * (a.x * c.y + a.y * c.x);
+            m3 = m3 + 1 == N ? 0 : m3 + 1;
+            n3 = n3 == 0 ? N - 1 : n3 - 1;
+        }
+        w += cnt;
+    }
+    const int64_t k = (int64_t)(k1 * N + k2) * N + z.k3;
+    Qh[eoff + (int64_t)g * M * kLanes + k * kLanes + lane] = make_double2(re, im);
 }
 
 // Few cells (a partly filled group): one warp per (cell, zeta point), the lanes
-// split the box sum (term q = lane, lane + 32, ... in the box's m1, m2, m3
-// order) and the partial sums are added by a fixed shuffle tree. The same
-// plain FP64 sum, with every lane doing useful work when the group is not
-// full (one cell would otherwise cost as much as 32).
-__global__ void conv64_cells_kernel(const double2 *__restrict__ F, double2 *__restrict__ Qh,
-                                    const double *__restrict__ W, const uint64_t *__restrict__ Woff,
-                                    const int64_t *__restrict__ slot_off, int s0, int N, int64_t eoff) {
+// split the list (term q = lane, lane + 32, ...) and the partial sums are added
+// by a fixed shuffle tree. The same FP64 sum, with every lane doing useful work
+// when the group is not full (one cell would otherwise cost as much as 32).
+__global__ void __launch_bounds__(32 * kWarps64) conv64_cells_kernel(const double2 *__restrict__ F,
+                                                                     double2 *__restrict__ Qh,
+                                                                     const double *__restrict__ W,
+                                                                     const Zeta64 *__restrict__ Z, int nz,
+                                                                     const uint32_t *__restrict__ D,
+                                                                     const int64_t *__restrict__ slot_off, int s0,
+                                                                     int N, int64_t eoff) {
     const int lane = threadIdx.x & 31;
-    const int M = N * N * N, h = N / 2;
-    const int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (k >= M) return;
+    const int64_t M = (int64_t)N * N * N;
+    const int zi = blockIdx.x * kWarps64 + (threadIdx.x >> 5);
     const int slot = blockIdx.y;  // slot within the segment
-    if (slot_off[s0 + slot] < 0) return;
-    const int g = slot / kLanes, cl = slot % kLanes;
-    const double2 *Fg = F + eoff + (int64_t)g * M * kLanes + cl;
-    const int k1 = k / (N * N), k2 = (k / N) % N, k3 = k % N;
-    const int lo1 = max(0, k1 - h + 1), hi1 = min(N - 1, k1 + h);
-    const int lo2 = max(0, k2 - h + 1), hi2 = min(N - 1, k2 + h);
-    const int lo3 = max(0, k3 - h + 1), hi3 = min(N - 1, k3 + h);
-    const int l2 = hi2 - lo2 + 1, l3 = hi3 - lo3 + 1, nt = (hi1 - lo1 + 1) * l2 * l3;
-    const double *w = W + Woff[k];
+    if (zi >= nz || slot_off[s0 + slot] < 0) return;
+    const Zeta64 z = Z[zi];
+    const int64_t cell = eoff + (int64_t)(slot / kLanes) * M * kLanes + slot % kLanes;
+    const double2 *Fg = F + cell;
+    const double *w = W + z.woff;
+    const uint32_t *Dz = D + z.desc_off;
+    const int k1 = z.k1, k2 = z.k2, cnt = z.m_count, n3_first = pair_partner(z.k3, z.m_first, N);
+    const int nt = z.nblocks * cnt, bstep = 32 / cnt, tstep = 32 % cnt;
     double re = 0.0, im = 0.0;
+    int b = lane / cnt, t = lane % cnt;
     for (int q = lane; q < nt; q += 32) {
-        const int m1 = lo1 + q / (l2 * l3), m2 = lo2 + (q / l3) % l2, m3 = lo3 + q % l3;
+        const uint32_t d = Dz[b];
+        const int m1 = (int)(d & 0xffffu), m2 = (int)(d >> 16);
+        int m3 = z.m_first + t, n3 = n3_first - t;
+        m3 -= m3 >= N ? N : 0;
+        n3 += n3 < 0 ? N : 0;
         const double g_ = w[q];
         const double2 a = Fg[(int64_t)((m1 * N + m2) * N + m3) * kLanes];
-        const int n = ((k1 - m1 + h) * N + (k2 - m2 + h)) * N + (k3 - m3 + h);
-        const double2 b = Fg[(int64_t)n * kLanes];
-        re += g_ * (a.x * b.x - a.y * b.y);
-        im += g_ * (a.x * b.y + a.y * b.x);
+        const double2 c =
+            Fg[(int64_t)((pair_partner(k1, m1, N) * N + pair_partner(k2, m2, N)) * N + n3) * kLanes];
+        re += g_ * (a.x * c.x - a.y * c.y);
+        im += g_ * (a.x * c.y + a.y * c.x);
+        b += bstep;
+        t += tstep;
+        if (t >= cnt) {
+            t -= cnt;
+            ++b;
+        }
     }
     for (int o = 16; o > 0; o >>= 1) {
         re += __shfl_xor_sync(0xffffffffu, re, o);
         im += __shfl_xor_sync(0xffffffffu, im, o);
     }
-    if (lane == 0) Qh[eoff + (int64_t)g * M * kLanes + (int64_t)k * kLanes + cl] = make_double2(re, im);
+    if (lane == 0) Qh[cell + ((int64_t)(k1 * N + k2) * N + z.k3) * kLanes] = make_double2(re, im);
 }
 
-void launch_conv64_cells(const double2 *F, double2 *Qh, const double *W, const uint64_t *Woff,
-                         const int64_t *slot_off, int s0, int nslots, int N, int64_t eoff, cudaStream_t st) {
-    const int M = N * N * N, warps = 4;
-    dim3 grid((M + warps - 1) / warps, nslots);
-    conv64_cells_kernel<<<grid, warps * 32, 0, st>>>(F, Qh, W, Woff, slot_off, s0, N, eoff);
+void launch_conv64_cells(const double2 *F, double2 *Qh, const Table &t, const int64_t *slot_off, int s0, int nslots,
+                         int64_t eoff, cudaStream_t st) {
+    dim3 grid((t.n_zeta64 + kWarps64 - 1) / kWarps64, nslots);
+    conv64_cells_kernel<<<grid, 32 * kWarps64, 0, st>>>(F, Qh, t.d_w64, t.d_zeta64, t.n_zeta64, t.d_desc, slot_off,
+                                                        s0, t.N, eoff);
 }
 
-void launch_conv64(const double2 *F, double2 *Qh, const double *W, const uint64_t *Woff, int N,
-                   int64_t eoff, int ngroups, cudaStream_t st) {
-    const int M = N * N * N, warps = 4;
-    dim3 grid((M + warps - 1) / warps, ngroups);
-    conv64_plain_kernel<<<grid, warps * 32, 0, st>>>(F, Qh, W, Woff, N, eoff);
+void launch_conv64(const double2 *F, double2 *Qh, const Table &t, int64_t eoff, int ngroups, cudaStream_t st) {
+    const int64_t warps = (int64_t)t.n_zeta64 * ngroups;
+    conv64_plain_kernel<<<(unsigned)((warps + kWarps64 - 1) / kWarps64), 32 * kWarps64, 0, st>>>(
+        F, Qh, t.d_w64, t.d_zeta64, t.n_zeta64, t.d_desc, t.N, eoff, ngroups);
 }
 
 }  // namespace bte

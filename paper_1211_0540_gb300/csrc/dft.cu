@@ -101,9 +101,9 @@ __global__ void dft_fwd_axis1_group(const C *__restrict__ in, DftSeg s, const C 
 }
 
 // Inverse pass along k1 out of the group layout: out[slot][j1][k2][k3].
-// Threads run lane-fastest so the group rows are read coalesced. HALF: only
-// the stored pencils hold Qhat (half-spectrum convolution), the others are 0.
-template <typename C, bool HALF>
+// Threads run lane-fastest so the group rows are read coalesced. Only the
+// stored pencils hold Qhat (half-spectrum convolution), the others are 0.
+template <typename C>
 __global__ void dft_inv_axis1_group(const C *__restrict__ G, DftSeg s, const C *__restrict__ root,
                                     C *__restrict__ out) {
     using R = typename CT<C>::R;
@@ -119,7 +119,7 @@ __global__ void dft_inv_axis1_group(const C *__restrict__ G, DftSeg s, const C *
         R re = 0, im = 0;
         const int k2 = rest / N;
         for (int k1 = 0; k1 < N; ++k1) {
-            if (HALF && !pencil_stored(k1, k2, N)) continue;
+            if (!pencil_stored(k1, k2, N)) continue;
             cmac<C, +1>(re, im, g[((int64_t)k1 * N * N + rest) * kLanes + lane],
                         root[phase_index(k1 - h, j1 - h, N)]);
         }
@@ -173,8 +173,7 @@ void launch_dft_inverse(const C *G, const int64_t *slot_off, const DftSeg &s, co
     const int M = s.N * s.N * s.N, threads = 128;
     const int ngroups = s.nslots / kLanes;
     int bx = (int)(((int64_t)M * kLanes + threads - 1) / threads);
-    constexpr bool half = sizeof(C) == sizeof(float2);  // the FP64 convolution writes every pencil
-    dft_inv_axis1_group<C, half><<<dim3(bx, ngroups), threads, 0, st>>>(G, s, root, T1);
+    dft_inv_axis1_group<C><<<dim3(bx, ngroups), threads, 0, st>>>(G, s, root, T1);
     dim3 grid = grid_for(M, s.nslots, threads);
     dft_axis2<C, +1><<<grid, threads, 0, st>>>(T1, s, root, T2);
     dft_inv_axis3_real<C><<<grid, threads, 0, st>>>(T2, slot_off, s, root, (typename CT<C>::R)scale, q);

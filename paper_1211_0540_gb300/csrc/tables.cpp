@@ -99,10 +99,6 @@ void quadrature_tables(Table &t, double hz) {
     for (int s = 0; s < t.ns; ++s) t.J[s] = value(0, 4 * s);
 }
 
-inline int box_lo(int k, int N) { return std::max(0, k - N / 2 + 1); }
-inline int box_hi(int k, int N) { return std::min(N - 1, k + N / 2); }
-inline int box_len(int k, int N) { return box_hi(k, N) - box_lo(k, N) + 1; }
-
 }  // namespace
 
 int first_kind_for_N(int N) {
@@ -446,42 +442,69 @@ int build_table_fp32(Table &t, std::string &err) {
     return BTE_OK;
 }
 
-// FP64 table of the plain operator: for each zeta point k (k1-major, k3
-// fastest) the weights Ghat(k, m) dz^3 over its valid box of m (m1-major, m3
-// fastest); off[k] is the prefix sum of the box sizes.
+// FP64 table of the plain operator: for each zeta point of a stored pencil the
+// pair weights W(k, m) + W(k, n) (W(k, m) alone in a block that pairs with
+// itself) times dz^3, per block of the pencil, m3 from m_first on (mod N).
 int build_table_fp64(Table &t, std::string &err) {
     if (t.d_w64) return BTE_OK;
-    const int N = t.N, M = N * N * N;
+    const int N = t.N;
     const double dz3 = t.dz * t.dz * t.dz;
-    std::vector<uint64_t> off(M + 1, 0);
-    for (int k = 0; k < M; ++k) {
-        int k1 = k / (N * N), k2 = (k / N) % N, k3 = k % N;
-        off[k + 1] = off[k] + (uint64_t)box_len(k1, N) * box_len(k2, N) * box_len(k3, N);
+    std::vector<Zeta64> z;
+    uint64_t total = 0;
+    for (int kk = 0; kk < N * N; ++kk) {
+        if (t.nblocks[kk] == 0) continue;
+        for (int k3 = 0; k3 < N; ++k3) {
+            Zeta64 e{};
+            e.woff = total;
+            e.desc_off = t.desc_off[kk];
+            e.nblocks = (uint16_t)t.nblocks[kk];
+            e.k1 = (uint16_t)(kk / N);
+            e.k2 = (uint16_t)(kk % N);
+            e.k3 = (uint16_t)k3;
+            for (int m = 0; m < N; ++m) {  // the kept m3 are one run mod N
+                if (!pair_kept(k3, m, N)) continue;
+                ++e.m_count;
+                if (!pair_kept(k3, (m + N - 1) % N, N)) e.m_first = (uint16_t)m;
+            }
+            total += (uint64_t)e.nblocks * e.m_count;
+            z.push_back(e);
+        }
     }
-    t.n_w64 = off[M];
-    std::vector<double> w((size_t)t.n_w64);
+    t.n_w64 = total;
+    t.n_zeta64 = (int)z.size();
+    std::vector<double> w((size_t)total);
 #pragma omp parallel for schedule(dynamic, 16)
-    for (int k = 0; k < M; ++k) {
-        int k1 = k / (N * N), k2 = (k / N) % N, k3 = k % N;
-        size_t o = off[k];
-        for (int m1 = box_lo(k1, N); m1 <= box_hi(k1, N); ++m1)
-            for (int m2 = box_lo(k2, N); m2 <= box_hi(k2, N); ++m2)
-                for (int m3 = box_lo(k3, N); m3 <= box_hi(k3, N); ++m3)
-                    w[o++] = t.ghat(k1, k2, k3, m1, m2, m3) * dz3;
+    for (int i = 0; i < t.n_zeta64; ++i) {
+        const Zeta64 &e = z[i];
+        size_t o = e.woff;
+        for (int b = 0; b < e.nblocks; ++b) {
+            const uint32_t d = t.desc_host[e.desc_off + b];
+            const int m1 = d & 0xffff, m2 = d >> 16, n1 = pair_partner(e.k1, m1, N), n2 = pair_partner(e.k2, m2, N);
+            const bool pair = !(m1 == n1 && m2 == n2);
+            for (int q = 0; q < e.m_count; ++q) {
+                const int m3 = (e.m_first + q) % N;
+                double g = t.half_weight(e.k1, e.k2, e.k3, m1, m2, m3);
+                if (pair) g += t.half_weight(e.k1, e.k2, e.k3, n1, n2, pair_partner(e.k3, m3, N));
+                w[o++] = g * dz3;
+            }
+        }
     }
+    std::stable_sort(z.begin(), z.end(), [](const Zeta64 &a, const Zeta64 &b) {
+        return (uint64_t)a.nblocks * a.m_count > (uint64_t)b.nblocks * b.m_count;
+    });
     cudaError_t e = cudaMalloc(&t.d_w64, sizeof(double) * std::max<uint64_t>(t.n_w64, 1));
-    if (e == cudaSuccess) e = cudaMalloc(&t.d_w64_off, sizeof(uint64_t) * (M + 1));
+    if (e == cudaSuccess) e = cudaMalloc(&t.d_zeta64, sizeof(Zeta64) * z.size());
     if (e != cudaSuccess) {
+        cudaGetLastError();
         err = std::string("cudaMalloc (FP64 weight table): ") + cudaGetErrorString(e);
         cudaFree(t.d_w64);
-        cudaFree(t.d_w64_off);
+        cudaFree(t.d_zeta64);
         t.d_w64 = nullptr;
-        t.d_w64_off = nullptr;
+        t.d_zeta64 = nullptr;
         return BTE_ENOMEM;
     }
     e = cudaMemcpy(t.d_w64, w.data(), sizeof(double) * t.n_w64, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess)
-        e = cudaMemcpy(t.d_w64_off, off.data(), sizeof(uint64_t) * (M + 1), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(t.d_zeta64, z.data(), sizeof(Zeta64) * z.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         err = std::string("cudaMemcpy (FP64 weight table): ") + cudaGetErrorString(e);
         return BTE_ECUDA;
@@ -500,13 +523,13 @@ void free_table(Table &t) {
     t.d_etab = nullptr;
     cudaFree(t.d_desc);
     cudaFree(t.d_w64);
-    cudaFree(t.d_w64_off);
+    cudaFree(t.d_zeta64);
     cudaFree(t.d_root32);
     cudaFree(t.d_root64);
     t.d_w32 = nullptr;
     t.d_desc = nullptr;
     t.d_w64 = nullptr;
-    t.d_w64_off = nullptr;
+    t.d_zeta64 = nullptr;
     t.d_root32 = nullptr;
     t.d_root64 = nullptr;
 }
