@@ -525,7 +525,10 @@ bte_status prepare(bte_ctx *c, Batch *B, int mode, bool step, bool transport) {
             if ((s = ensure_scratch(c, id, sizeof(double) * (size_t)B->extent)) != BTE_OK) return s;
     }
     for (const Segment &sg : B->segs)
-        if (fused_dft_supported(c->tables[sg.table]->N)) fused_dft_prepare(c->tables[sg.table]->N);
+        if (mode != BTE_FP64_PLAIN && fused_dft_supported(c->tables[sg.table]->N))
+            fused_dft_prepare(c->tables[sg.table]->N);
+        else
+            dft_prepare(c->tables[sg.table]->N);
     if (mode == BTE_FP64_PLAIN) {
         for (const Segment &sg : B->segs) {
             if (c->tables[sg.table]->N > 32)
@@ -551,6 +554,10 @@ bte_status prepare(bte_ctx *c, Batch *B, int mode, bool step, bool transport) {
     return BTE_OK;
 }
 
+// The FP64 convolution takes the cells of a segment whose groups are at most
+// half full one by one (lanes over the sum instead of cells).
+bool by_cells64(const Segment &sg) { return 2 * sg.nvalid <= sg.nslots; }
+
 // What happens after the inverse transform of a collide.
 enum Post { POST_RAW = 0, POST_PROJECT = 1, POST_STAGE1 = 2, POST_STAGE2 = 3 };
 
@@ -573,20 +580,15 @@ bte_status enqueue_collide(bte_ctx *c, Batch *B, const double *f, double *Q, int
         const int on_fwd = prof_begin(c, PK_FORWARD, st, &pe_fwd);
         for (const Segment &sg : B->segs) {
             const Table *t = c->tables[sg.table];
-            DftSeg ds{t->N, sg.s0, sg.nslots, sg.eoff};
+            DftSeg ds{t->N, sg.s0, sg.nslots, sg.eoff, sg.nvalid};
             const double sf = std::pow(2.0 * kPi, -1.5) * t->dv * t->dv * t->dv;
-            if (fp64) {
-                launch_dft_forward<double2>(f, B->d_slot_off, ds, t->d_root64, sf, (double2 *)c->scratch[SC_T1],
-                                            (double2 *)c->scratch[SC_T2], (double2 *)c->scratch[SC_F], c->d_status, st);
-                count_launches(c, 3);
-            } else if (fused_dft_supported(t->N)) {
+            if (fp64 || !fused_dft_supported(t->N))
+                count_launches(c, launch_dft_forward(f, B->d_slot_off, ds, sf, c->scratch[SC_T1], c->scratch[SC_F],
+                                                     fp64 && by_cells64(sg), c->d_status, st));
+            else {
                 launch_dft_forward_fused(f, B->d_slot_off, ds, t->d_root32, sf, (float2 *)c->scratch[SC_F], c->d_status,
                                          st, cfg.split);
                 count_launches(c, 1);
-            } else {
-                launch_dft_forward<float2>(f, B->d_slot_off, ds, t->d_root32, sf, (float2 *)c->scratch[SC_T1],
-                                           (float2 *)c->scratch[SC_T2], (float2 *)c->scratch[SC_F], c->d_status, st);
-                count_launches(c, 3);
             }
             cudaError_t e0 = cudaGetLastError();
             if (e0 != cudaSuccess) return cuda_fail(c, e0, "forward transform launch");
@@ -598,9 +600,9 @@ bte_status enqueue_collide(bte_ctx *c, Batch *B, const double *f, double *Q, int
         const int on = prof_begin(c, PK_CONV64, st, &pe_conv);
         for (const Segment &sg : B->segs) {
             const Table *t = c->tables[sg.table];
-            if (2 * sg.nvalid <= sg.nslots)  // groups less than half full: lanes over the box instead of cells
-                launch_conv64_cells((const double2 *)c->scratch[SC_F], (double2 *)c->scratch[SC_QH], *t,
-                                    B->d_slot_off, sg.s0, sg.nslots, sg.eoff, st);
+            if (by_cells64(sg))
+                launch_conv64_cells((const double2 *)c->scratch[SC_F], (double2 *)c->scratch[SC_QH], *t, sg.nvalid,
+                                    sg.eoff, st);
             else
                 launch_conv64((const double2 *)c->scratch[SC_F], (double2 *)c->scratch[SC_QH], *t, sg.eoff,
                               sg.nslots / kLanes, st);
@@ -655,7 +657,7 @@ bte_status enqueue_collide(bte_ctx *c, Batch *B, const double *f, double *Q, int
     const int on_inv = prof_begin(c, PK_INVERSE, st, &pe_inv);
     for (const Segment &sg : B->segs) {
         const Table *t = c->tables[sg.table];
-        DftSeg ds{t->N, sg.s0, sg.nslots, sg.eoff};
+        DftSeg ds{t->N, sg.s0, sg.nslots, sg.eoff, sg.nvalid};
         const double si = std::pow(2.0 * kPi, -1.5) * t->dz * t->dz * t->dz;
         if (fuse & FUSE_NEXT_FWD) {  // post == POST_STAGE1 (checked by the caller)
             const double sf = std::pow(2.0 * kPi, -1.5) * t->dv * t->dv * t->dv;
@@ -671,17 +673,11 @@ bte_status enqueue_collide(bte_ctx *c, Batch *B, const double *f, double *Q, int
             count_launches(c, 1);
             continue;
         }
-        if (fp64)
-            launch_dft_inverse<double2>((const double2 *)c->scratch[SC_QH], B->d_slot_off, ds, t->d_root64, si,
-                                        (double2 *)c->scratch[SC_T1], (double2 *)c->scratch[SC_T2], Q, st);
-        else
-            launch_dft_inverse<float2>((const float2 *)c->scratch[SC_QH], B->d_slot_off, ds, t->d_root32, si,
-                                       (float2 *)c->scratch[SC_T1], (float2 *)c->scratch[SC_T2], Q, st);
-        count_launches(c, 3);
-        if (post != POST_RAW) {
-            launch_project(Q, B->d_slot_off, sg.s0, sg.nslots, proj_args(t), post - 1, x, y, qp, a, st);
-            count_launches(c, 1);
-        }
+        // post - 1: the projection's mode (ProjArgs), -1 for the raw Qt
+        double *mom = fp64 ? (double *)((double2 *)c->scratch[SC_T2] + sg.eoff)
+                           : (double *)((float2 *)c->scratch[SC_T2] + sg.eoff);
+        count_launches(c, launch_dft_inverse(c->scratch[SC_QH], B->d_slot_off, ds, si, c->scratch[SC_T1], mom, Q,
+                                             fp64 && by_cells64(sg), proj_args(t), post - 1, x, y, qp, a, st));
     }
     prof_end(c, on_inv, pe_inv, st);
     prof_end(c, on_all, pe_all, st);
@@ -849,7 +845,7 @@ bte_status enqueue_indicator(bte_ctx *c, Batch *B, const double *f, const double
     if ((s = ensure_scratch(c, SC_MISC, sizeof(float) * indicator_scratch_floats(*c->ind, t->N, B->nslots))) !=
         BTE_OK)
         return s;
-    DftSeg ds{t->N, sg.s0, sg.nslots, sg.eoff};
+    DftSeg ds{t->N, sg.s0, sg.nslots, sg.eoff, sg.nvalid};
     const double sf = std::pow(2.0 * kPi, -1.5) * t->dv * t->dv * t->dv;
     // sector order; one CTA per cell once the cells fill the SMs (the fastest for
     // this transform alone), else the batch's tuned split

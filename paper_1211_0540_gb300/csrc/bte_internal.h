@@ -135,7 +135,6 @@ struct Table {
     int n_tmpl = 0;
     // DFT roots exp(2 pi i t / N), t in [0, N)
     float2 *d_root32 = nullptr;
-    double2 *d_root64 = nullptr;
     // Projection: (C C^T)^{-1}, row-major 5x5 (C without the dv^3 factor folded in)
     double ainv[25];
     // Host FP64 radial tables on integer invariants (kept for the lazy FP64 table)

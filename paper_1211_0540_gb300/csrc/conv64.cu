@@ -65,16 +65,14 @@ __global__ void __launch_bounds__(32 * kWarps64) conv64_cells_kernel(const doubl
                                                                      double2 *__restrict__ Qh,
                                                                      const double *__restrict__ W,
                                                                      const Zeta64 *__restrict__ Z, int nz,
-                                                                     const uint32_t *__restrict__ D,
-                                                                     const int64_t *__restrict__ slot_off, int s0,
-                                                                     int N, int64_t eoff) {
+                                                                     const uint32_t *__restrict__ D, int N,
+                                                                     int64_t eoff) {
     const int lane = threadIdx.x & 31;
     const int64_t M = (int64_t)N * N * N;
     const int zi = blockIdx.x * kWarps64 + (threadIdx.x >> 5);
-    const int slot = blockIdx.y;  // slot within the segment
-    if (zi >= nz || slot_off[s0 + slot] < 0) return;
+    if (zi >= nz) return;
     const Zeta64 z = Z[zi];
-    const int64_t cell = eoff + (int64_t)(slot / kLanes) * M * kLanes + slot % kLanes;
+    const int64_t cell = eoff + (int64_t)blockIdx.y * M;  // fhat and Qhat cell-major
     const double2 *Fg = F + cell;
     const double *w = W + z.woff;
     const uint32_t *Dz = D + z.desc_off;
@@ -82,6 +80,7 @@ __global__ void __launch_bounds__(32 * kWarps64) conv64_cells_kernel(const doubl
     const int nt = z.nblocks * cnt, bstep = 32 / cnt, tstep = 32 % cnt;
     double re = 0.0, im = 0.0;
     int b = lane / cnt, t = lane % cnt;
+#pragma unroll 4
     for (int q = lane; q < nt; q += 32) {
         const uint32_t d = Dz[b];
         const int m1 = (int)(d & 0xffffu), m2 = (int)(d >> 16);
@@ -89,9 +88,8 @@ __global__ void __launch_bounds__(32 * kWarps64) conv64_cells_kernel(const doubl
         m3 -= m3 >= N ? N : 0;
         n3 += n3 < 0 ? N : 0;
         const double g_ = w[q];
-        const double2 a = Fg[(int64_t)((m1 * N + m2) * N + m3) * kLanes];
-        const double2 c =
-            Fg[(int64_t)((pair_partner(k1, m1, N) * N + pair_partner(k2, m2, N)) * N + n3) * kLanes];
+        const double2 a = Fg[(m1 * N + m2) * N + m3];
+        const double2 c = Fg[(pair_partner(k1, m1, N) * N + pair_partner(k2, m2, N)) * N + n3];
         re += g_ * (a.x * c.x - a.y * c.y);
         im += g_ * (a.x * c.y + a.y * c.x);
         b += bstep;
@@ -105,14 +103,12 @@ __global__ void __launch_bounds__(32 * kWarps64) conv64_cells_kernel(const doubl
         re += __shfl_xor_sync(0xffffffffu, re, o);
         im += __shfl_xor_sync(0xffffffffu, im, o);
     }
-    if (lane == 0) Qh[cell + ((int64_t)(k1 * N + k2) * N + z.k3) * kLanes] = make_double2(re, im);
+    if (lane == 0) Qh[cell + (k1 * N + k2) * N + z.k3] = make_double2(re, im);
 }
 
-void launch_conv64_cells(const double2 *F, double2 *Qh, const Table &t, const int64_t *slot_off, int s0, int nslots,
-                         int64_t eoff, cudaStream_t st) {
-    dim3 grid((t.n_zeta64 + kWarps64 - 1) / kWarps64, nslots);
-    conv64_cells_kernel<<<grid, 32 * kWarps64, 0, st>>>(F, Qh, t.d_w64, t.d_zeta64, t.n_zeta64, t.d_desc, slot_off,
-                                                        s0, t.N, eoff);
+void launch_conv64_cells(const double2 *F, double2 *Qh, const Table &t, int nvalid, int64_t eoff, cudaStream_t st) {
+    dim3 grid((t.n_zeta64 + kWarps64 - 1) / kWarps64, nvalid);
+    conv64_cells_kernel<<<grid, 32 * kWarps64, 0, st>>>(F, Qh, t.d_w64, t.d_zeta64, t.n_zeta64, t.d_desc, t.N, eoff);
 }
 
 void launch_conv64(const double2 *F, double2 *Qh, const Table &t, int64_t eoff, int ngroups, cudaStream_t st) {

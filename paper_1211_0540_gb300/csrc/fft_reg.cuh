@@ -15,8 +15,8 @@
 // root[t] = exp(2 pi i t / NT): w_n^t = root[(t NT / n) mod NT]. Indices 0,
 // NT/4, NT/2 and 3NT/4 are +-1 and +-i and cost no multiplication; with the
 // loops unrolled every index is a compile-time constant, so on the device the
-// table (in constant memory) supplies FMA operands directly. Host and device:
-// the same code is checked against the dense sum on the CPU.
+// table (in constant memory) supplies FMA operands directly. FP32 and FP64,
+// host and device: the same code is checked against the dense sum on the CPU.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -24,48 +24,58 @@
 namespace bte {
 namespace fftr {
 
-__host__ __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__host__ __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
-__host__ __device__ __forceinline__ float2 cneg(float2 a) { return make_float2(-a.x, -a.y); }
+// The vector types: float2 or double2, by overloads.
+__host__ __device__ __forceinline__ float2 mk(float a, float b) { return make_float2(a, b); }
+__host__ __device__ __forceinline__ double2 mk(double a, double b) { return make_double2(a, b); }
+__host__ __device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
+__host__ __device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
+
+template <class V>
+__host__ __device__ __forceinline__ V cadd(V a, V b) { return mk(a.x + b.x, a.y + b.y); }
+template <class V>
+__host__ __device__ __forceinline__ V csub(V a, V b) { return mk(a.x - b.x, a.y - b.y); }
+template <class V>
+__host__ __device__ __forceinline__ V cneg(V a) { return mk(-a.x, -a.y); }
 // i s a for s = +1 or -1
-template <int S>
-__host__ __device__ __forceinline__ float2 cmul_i(float2 a) {
-    return S > 0 ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x);
+template <int S, class V>
+__host__ __device__ __forceinline__ V cmul_i(V a) {
+    return S > 0 ? mk(-a.y, a.x) : mk(a.y, -a.x);
 }
 
 // v w_NT^(S t), t >= 0 (compile-time after unrolling)
-template <int NT, int S>
-__host__ __device__ __forceinline__ float2 twiddle(float2 v, int t, const float2 (&rt)[NT]) {
+template <int NT, int S, class V>
+__host__ __device__ __forceinline__ V twiddle(V v, int t, const V (&rt)[NT]) {
     const int u = ((S * t) % NT + NT) % NT;
     if (u == 0) return v;
     if (2 * u == NT) return cneg(v);
     if (4 * u == NT) return cmul_i<1>(v);
     if (4 * u == 3 * NT) return cmul_i<-1>(v);
-    const float2 w = rt[u];
-    return make_float2(fmaf(v.x, w.x, -(v.y * w.y)), fmaf(v.x, w.y, v.y * w.x));
+    const V w = rt[u];
+    return mk(fma_(v.x, w.x, -(v.y * w.y)), fma_(v.x, w.y, v.y * w.x));
 }
 
 // In place: x <- DFT_S(x) of size N inside a top-level transform of size NT.
-template <int N, int S, int NT>
-__host__ __device__ __forceinline__ void fft(float2 (&x)[N], const float2 (&rt)[NT]) {
+template <int N, int S, int NT, class V>
+__host__ __device__ __forceinline__ void fft(V (&x)[N], const V (&rt)[NT]) {
     static_assert(NT % N == 0, "sub-transform size");
     if constexpr (N == 1) {
     } else if constexpr (N == 2) {
-        const float2 a = x[0], b = x[1];
+        const V a = x[0], b = x[1];
         x[0] = cadd(a, b);
         x[1] = csub(a, b);
     } else if constexpr (N == 3) {
         // w_3^S = -1/2 + i S sin(2 pi / 3); sin(2 pi / 3) = Im root[NT / 3]
-        const float s3 = rt[NT / 3].y;
-        const float2 a = x[0], t = cadd(x[1], x[2]), u = csub(x[1], x[2]);
-        const float2 m = make_float2(fmaf(-0.5f, t.x, a.x), fmaf(-0.5f, t.y, a.y));
-        const float2 r = cmul_i<S>(make_float2(s3 * u.x, s3 * u.y));
+        const auto s3 = rt[NT / 3].y;
+        const V a = x[0], t = cadd(x[1], x[2]), u = csub(x[1], x[2]);
+        const decltype(a.x) half = -0.5f;
+        const V m = mk(fma_(half, t.x, a.x), fma_(half, t.y, a.y));
+        const V r = cmul_i<S>(mk(s3 * u.x, s3 * u.y));
         x[0] = cadd(a, t);
         x[1] = cadd(m, r);
         x[2] = csub(m, r);
     } else if constexpr (N == 4) {
-        const float2 a = cadd(x[0], x[2]), b = csub(x[0], x[2]);
-        const float2 c = cadd(x[1], x[3]), d = cmul_i<S>(csub(x[1], x[3]));
+        const V a = cadd(x[0], x[2]), b = csub(x[0], x[2]);
+        const V c = cadd(x[1], x[3]), d = cmul_i<S>(csub(x[1], x[3]));
         x[0] = cadd(a, c);
         x[1] = cadd(b, d);
         x[2] = csub(a, c);
@@ -73,10 +83,10 @@ __host__ __device__ __forceinline__ void fft(float2 (&x)[N], const float2 (&rt)[
     } else {
         constexpr int R = N % 4 == 0 ? 4 : (N % 3 == 0 ? 3 : 2);
         constexpr int N2 = N / R;
-        float2 A[R][N2];
+        V A[R][N2];
 #pragma unroll
         for (int j2 = 0; j2 < N2; ++j2) {
-            float2 v[R];
+            V v[R];
 #pragma unroll
             for (int j1 = 0; j1 < R; ++j1) v[j1] = x[N2 * j1 + j2];
             fft<R, S, NT>(v, rt);
@@ -85,7 +95,7 @@ __host__ __device__ __forceinline__ void fft(float2 (&x)[N], const float2 (&rt)[
         }
 #pragma unroll
         for (int k1 = 0; k1 < R; ++k1) {
-            float2 u[N2];
+            V u[N2];
 #pragma unroll
             for (int j2 = 0; j2 < N2; ++j2) u[j2] = A[k1][j2];
             fft<N2, S, NT>(u, rt);
@@ -98,8 +108,8 @@ __host__ __device__ __forceinline__ void fft(float2 (&x)[N], const float2 (&rt)[
 // Centred transform of one pencil (N/2 even):
 //   y_k = sum_j x_j w^(S (k - N/2)(j - N/2)) = (-1)^k sum_j (-1)^j x_j w^(S j k),
 // since w^(-N/2 k) = (-1)^k and w^((N/2)^2) = (-1)^(N/2) = 1.
-template <int N, int S>
-__host__ __device__ __forceinline__ void centred(float2 (&y)[N], const float2 (&rt)[N]) {
+template <int N, int S, class V>
+__host__ __device__ __forceinline__ void centred(V (&y)[N], const V (&rt)[N]) {
     static_assert(N % 4 == 0, "N/2 must be even");
 #pragma unroll
     for (int j = 1; j < N; j += 2) y[j] = cneg(y[j]);

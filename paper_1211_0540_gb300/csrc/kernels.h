@@ -12,6 +12,7 @@ struct DftSeg {
     int s0;        // first slot of the segment (global slot index)
     int nslots;    // slots in the segment (multiple of 32)
     int64_t eoff;  // complex-element offset of slot s0 in scratch / group buffers
+    int nvalid = 0;  // slots that hold a cell, the first ones (read by the transforms of dft.cu only)
 };
 
 // Projection (Sec. 3.3), optionally fused with the RK2 update:
@@ -22,12 +23,16 @@ struct ProjArgs {
     double ainv[25];
 };
 
-template <typename C>
-void launch_dft_forward(const double *f, const int64_t *slot_off, const DftSeg &s, const C *root,
-                        double scale, C *T1, C *T2, C *G, int *status, cudaStream_t st);
-template <typename C>
-void launch_dft_inverse(const C *G, const int64_t *slot_off, const DftSeg &s, const C *root,
-                        double scale, C *T1, C *T2, double *q, cudaStream_t st);
+// Transforms of the FP64 operator (N <= 32; T and G hold double2) and of FP32 at
+// N = 48 (float2), dft.cu. cell: fhat / Qhat cell-major instead of the group
+// layout. mom: 5 N doubles per slot of scratch. mode of the inverse: -1 raw Qt,
+// else the projection's (ProjArgs). Both return the kernels launched.
+void dft_prepare(int N);  // outside stream capture
+int launch_dft_forward(const double *f, const int64_t *slot_off, const DftSeg &s, double scale, void *T, void *G,
+                       bool cell, int *status, cudaStream_t st);
+int launch_dft_inverse(const void *G, const int64_t *slot_off, const DftSeg &s, double scale, void *T, double *mom,
+                       double *q, bool cell, const ProjArgs &pa, int mode, const double *x, double *y,
+                       const double *qp, double a, cudaStream_t st);
 
 // FP32 convolution (persistent, work queue of ConvItems).
 constexpr int kMaxTables = 16;
@@ -81,9 +86,8 @@ cudaError_t conv32_launch(const ConvLaunch &L, const ConvParams &p, cudaStream_t
 
 // FP64 convolution of one segment (the modes of the stored pencils).
 void launch_conv64(const double2 *F, double2 *Qh, const Table &t, int64_t eoff, int ngroups, cudaStream_t st);
-// the same for a segment with few valid cells: one warp per (valid slot, zeta)
-void launch_conv64_cells(const double2 *F, double2 *Qh, const Table &t, const int64_t *slot_off, int s0, int nslots,
-                         int64_t eoff, cudaStream_t st);
+// the same for a segment with few valid cells: one warp per (valid slot, zeta), fhat and Qhat cell-major
+void launch_conv64_cells(const double2 *F, double2 *Qh, const Table &t, int nvalid, int64_t eoff, cudaStream_t st);
 
 void launch_project(double *Q, const int64_t *slot_off, int s0, int nslots, const ProjArgs &pa,
                     int mode, const double *X, double *Y, const double *Qp, double a,

@@ -39,9 +39,10 @@ constexpr int kIndPairs = kIndWarps / 2;
 // acc = full (re, im) per output, then loss (re, im). The weight of the pair
 // (m3, k3) sits at its rank among the block's valid pairs (m3 major, k3 minor),
 // a compile-time index after unrolling.
+// The full and the loss weights alternate in fours.
 template <int N, int JH>
-__device__ __forceinline__ void indicator_block(const float2 (&av)[N], const float2 (&bv)[N], const float4 *wf,
-                                                const float4 *wl, float (&acc)[2 * N]) {
+__device__ __forceinline__ void indicator_block(const float2 (&av)[N], const float2 (&bv)[N], const float4 *w,
+                                                float (&acc)[2 * N]) {
     constexpr int H = N / 2, J0 = JH * H;
     int wi = 0;
 #pragma unroll
@@ -51,7 +52,7 @@ __device__ __forceinline__ void indicator_block(const float2 (&av)[N], const flo
             const int n3 = j - m3 + H;
             if (n3 < 0 || n3 >= N) continue;
             if (j >= J0 && j < J0 + H) {
-                const float4 f4 = wf[wi >> 2], l4 = wl[wi >> 2];
+                const float4 f4 = w[2 * (wi >> 2)], l4 = w[2 * (wi >> 2) + 1];
                 const int q = wi & 3;
                 const float wF = q == 0 ? f4.x : q == 1 ? f4.y : q == 2 ? f4.z : f4.w;
                 const float wL = q == 0 ? l4.x : q == 1 ? l4.y : q == 2 ? l4.z : l4.w;
@@ -73,9 +74,8 @@ __device__ __forceinline__ void indicator_block(const float2 (&av)[N], const flo
 // waiting) adds half 0 and half 1 in that order and forms the errors.
 template <int N>
 __global__ void __launch_bounds__(32 * kIndWarps, 2)
-indicator_kernel(const float2 *__restrict__ F, const float2 *__restrict__ QN, const float *__restrict__ Wfull,
-                 const float *__restrict__ Wloss, const uint32_t *__restrict__ desc, const IndPencil *__restrict__ pens,
-                 int cpad, int64_t eoff, int nslots, float *err2, float *den2, float *part, unsigned *cnt) {
+indicator_kernel(const float2 *__restrict__ F, const float2 *__restrict__ QN, const float *__restrict__ W,
+                 const uint32_t *__restrict__ desc, const IndPencil *__restrict__ pens, int cpad, int64_t eoff, int nslots, float *err2, float *den2, float *part, unsigned *cnt) {
     constexpr int M = N * N * N, H = N / 2;
     extern __shared__ __align__(16) float red[];  // [kIndPairs][4 N][32]
     const int p = blockIdx.x, g = blockIdx.y, half = blockIdx.z, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -100,10 +100,9 @@ indicator_kernel(const float2 *__restrict__ F, const float2 *__restrict__ QN, co
             bv[i] = make_float2(b2.x, b2.y);
             bv[i + 1] = make_float2(b2.z, b2.w);
         }
-        const float4 *wf = reinterpret_cast<const float4 *>(Wfull + pen.wofs + (size_t)b * cpad);
-        const float4 *wl = reinterpret_cast<const float4 *>(Wloss + pen.wofs + (size_t)b * cpad);
-        if (jh == 0) indicator_block<N, 0>(av, bv, wf, wl, acc);
-        else indicator_block<N, 1>(av, bv, wf, wl, acc);
+        const float4 *w = reinterpret_cast<const float4 *>(W + pen.wofs + (size_t)b * 2 * cpad);
+        if (jh == 0) indicator_block<N, 0>(av, bv, w, acc);
+        else indicator_block<N, 1>(av, bv, w, acc);
     }
     // the pair's 4 N sums: full (re, im) of output k3 at 2 k3, loss at 2 N + 2 k3
 #pragma unroll
@@ -391,7 +390,7 @@ int build_indicator_table(const Table &t, int modes, uint64_t seed, IndicatorTab
     for (int m3 = 0; m3 < N; ++m3)
         for (int k3 = 0; k3 < N; ++k3) cpad += pair_on_grid(k3, m3, N);
     cpad = (cpad + 3) & ~3;
-    std::vector<float> wf, wl;
+    std::vector<float> w;
     std::vector<IndPencil> pens;
     std::vector<uint32_t> desc;
     for (int kk : kks) {
@@ -399,7 +398,7 @@ int build_indicator_table(const Table &t, int modes, uint64_t seed, IndicatorTab
         IndPencil pn{};
         pn.kk = kk;
         pn.desc_off = (int)desc.size();
-        pn.wofs = wl.size();
+        pn.wofs = w.size();
         for (int m1 = 0; m1 < N; ++m1)
             for (int m2 = 0; m2 < N; ++m2) {
                 const int n1 = k1 - m1 + h, n2 = k2 - m2 + h;
@@ -411,24 +410,25 @@ int build_indicator_table(const Table &t, int modes, uint64_t seed, IndicatorTab
             const uint32_t dd = desc[pn.desc_off + b];
             const int m1 = (int)(dd & 0xffffu), m2 = (int)(dd >> 16), n1 = k1 - m1 + h, n2 = k2 - m2 + h;
             const bool pair = !(m1 == n1 && m2 == n2);
-            const size_t base = wl.size();
-            wl.resize(base + cpad, 0.0f);
-            wf.resize(base + cpad, 0.0f);
-            size_t wi = base;
+            const size_t base = w.size();
+            w.resize(base + 2 * (size_t)cpad, 0.0f);
+            size_t wi = 0;
             for (int m3 = 0; m3 < N; ++m3)
                 for (int k3 = 0; k3 < N; ++k3) {
                     const int n3 = k3 - m3 + h;
                     if (n3 < 0 || n3 >= N) continue;
                     double full = t.ghat(k1, k2, k3, m1, m2, m3);
                     if (pair) full += t.ghat(k1, k2, k3, n1, n2, n3);
-                    wf[wi] = (float)(full * dz3);
+                    float *const e = &w[base + 8 * (wi / 4) + wi % 4];  // four full weights, then their loss parts
+                    ++wi;
+                    e[0] = (float)(full * dz3);
                     const int sm = (m1 - h) * (m1 - h) + (m2 - h) * (m2 - h) + (m3 - h) * (m3 - h);
                     double g = -c * t.J[sm];
                     if (pair) {
                         const int sn = (n1 - h) * (n1 - h) + (n2 - h) * (n2 - h) + (n3 - h) * (n3 - h);
                         g += -c * t.J[sn];
                     }
-                    wl[wi++] = (float)(g * dz3);
+                    e[4] = (float)(g * dz3);
                 }
         }
         pens.push_back(pn);
@@ -436,14 +436,12 @@ int build_indicator_table(const Table &t, int modes, uint64_t seed, IndicatorTab
     out.S = S;
     out.kks = kks;
     out.cpad = cpad;
-    cudaError_t e = cudaMalloc(&out.d_wloss, sizeof(float) * std::max<size_t>(wl.size(), 4));
-    if (e == cudaSuccess) e = cudaMalloc(&out.d_wfull, sizeof(float) * std::max<size_t>(wf.size(), 4));
+    cudaError_t e = cudaMalloc(&out.d_w, sizeof(float) * std::max<size_t>(w.size(), 4));
     if (e == cudaSuccess) e = cudaMalloc(&out.d_desc, sizeof(uint32_t) * std::max<size_t>(desc.size(), 1));
-    if (e == cudaSuccess) e = cudaMemcpy(out.d_wfull, wf.data(), sizeof(float) * wf.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = cudaMemcpy(out.d_desc, desc.data(), sizeof(uint32_t) * desc.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMalloc(&out.d_pen, sizeof(IndPencil) * S);
-    if (e == cudaSuccess) e = cudaMemcpy(out.d_wloss, wl.data(), sizeof(float) * wl.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(out.d_w, w.data(), sizeof(float) * w.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(out.d_pen, pens.data(), sizeof(IndPencil) * S, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMalloc(&out.d_kk, sizeof(int) * S);
     if (e == cudaSuccess) e = cudaMemcpy(out.d_kk, kks.data(), sizeof(int) * S, cudaMemcpyHostToDevice);
@@ -459,14 +457,12 @@ int build_indicator_table(const Table &t, int modes, uint64_t seed, IndicatorTab
 }
 
 void free_indicator_table(IndicatorTable &t) {
-    cudaFree(t.d_wfull);
+    cudaFree(t.d_w);
     cudaFree(t.d_desc);
-    cudaFree(t.d_wloss);
     cudaFree(t.d_pen);
-    t.d_wfull = nullptr;
+    t.d_w = nullptr;
     t.d_desc = nullptr;
     cudaFree(t.d_kk);
-    t.d_wloss = nullptr;
     t.d_pen = nullptr;
     t.d_kk = nullptr;
 }
@@ -496,16 +492,16 @@ void launch_indicator(const IndicatorTable &it, const Table &t, const float2 *F,
     cudaMemsetAsync(cnt, 0, sizeof(unsigned) * items, st);
     switch (t.N) {
         case 8:
-            indicator_kernel<8><<<grid, 32 * kIndWarps, ind_smem<8>(), st>>>(F, QN, it.d_wfull, it.d_wloss, it.d_desc,
+            indicator_kernel<8><<<grid, 32 * kIndWarps, ind_smem<8>(), st>>>(F, QN, it.d_w, it.d_desc,
                                                                            it.d_pen, it.cpad, eoff, nslots, err2, den2, part, cnt);
             break;
         case 12:
-            indicator_kernel<12><<<grid, 32 * kIndWarps, ind_smem<12>(), st>>>(F, QN, it.d_wfull, it.d_wloss, it.d_desc,
+            indicator_kernel<12><<<grid, 32 * kIndWarps, ind_smem<12>(), st>>>(F, QN, it.d_w, it.d_desc,
                                                                              it.d_pen, it.cpad, eoff, nslots, err2,
                                                                              den2, part, cnt);
             break;
         default:
-            indicator_kernel<16><<<grid, 32 * kIndWarps, ind_smem<16>(), st>>>(F, QN, it.d_wfull, it.d_wloss, it.d_desc,
+            indicator_kernel<16><<<grid, 32 * kIndWarps, ind_smem<16>(), st>>>(F, QN, it.d_w, it.d_desc,
                                                                              it.d_pen, it.cpad, eoff, nslots, err2,
                                                                              den2, part, cnt);
             break;

@@ -10,7 +10,7 @@ namespace bte {
 
 // Sampled pencils of the indicator: for pencil i, the (m1, m2) blocks of zeta
 // pencil kk = k1 N + k2 (d_desc + desc_off) and their full and loss-term pair
-// weights (d_wfull, d_wloss + wofs, cpad floats a block).
+// weights (d_w + wofs, 2 cpad floats a block, alternating in fours).
 struct IndPencil {
     int kk, desc_off, nblocks, pad;
     uint64_t wofs;
@@ -21,8 +21,7 @@ struct IndicatorTable {
     std::vector<int> kks;          // host copy of the sampled pencils (k1 N + k2), drawing order
     int cpad = 0;                  // floats per block of weights
     uint32_t *d_desc = nullptr;    // m1 | (m2 << 16)
-    float *d_wfull = nullptr;      // weights of the sampled pencils (pair-symmetrised, times dz^3)
-    float *d_wloss = nullptr;      // the same of the loss term
+    float *d_w = nullptr;          // weights of the sampled pencils (pair-symmetrised, times dz^3), full and loss
     IndPencil *d_pen = nullptr;
     int *d_kk = nullptr;           // the sampled pencils' k1 N + k2
 };

@@ -287,11 +287,9 @@ int build_table(Table &t, std::string &err) {
 
     // DFT roots exp(2 pi i t / N)
     std::vector<float2> r32(N);
-    std::vector<double2> r64(N);
     for (int s = 0; s < N; ++s) {
         double c = std::cos(2.0 * kPi * s / N), sn = std::sin(2.0 * kPi * s / N);
         r32[s] = make_float2((float)c, (float)sn);
-        r64[s] = make_double2(c, sn);
     }
 
     // one group's work items, costliest first (stable, so ties keep (tile, k1, k2) order)
@@ -365,7 +363,6 @@ int build_table(Table &t, std::string &err) {
     if (e == cudaSuccess && !etab.empty()) e = cudaMalloc(&t.d_etab, sizeof(uint16_t) * etab.size());
     if (e == cudaSuccess) e = cudaMalloc(&t.d_desc, sizeof(uint32_t) * std::max<size_t>(t.n_desc, 1));
     if (e == cudaSuccess) e = cudaMalloc(&t.d_root32, sizeof(float2) * N);
-    if (e == cudaSuccess) e = cudaMalloc(&t.d_root64, sizeof(double2) * N);
     if (e != cudaSuccess) {
         err = std::string("cudaMalloc (weight table): ") + cudaGetErrorString(e);
         free_table(t);
@@ -382,7 +379,6 @@ int build_table(Table &t, std::string &err) {
     if (e == cudaSuccess)
         e = cudaMemcpy(t.d_desc, desc.data(), sizeof(uint32_t) * t.n_desc, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(t.d_root32, r32.data(), sizeof(float2) * N, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(t.d_root64, r64.data(), sizeof(double2) * N, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         err = std::string("cudaMemcpy (weight table): ") + cudaGetErrorString(e);
         free_table(t);
@@ -525,13 +521,11 @@ void free_table(Table &t) {
     cudaFree(t.d_w64);
     cudaFree(t.d_zeta64);
     cudaFree(t.d_root32);
-    cudaFree(t.d_root64);
     t.d_w32 = nullptr;
     t.d_desc = nullptr;
     t.d_w64 = nullptr;
     t.d_zeta64 = nullptr;
     t.d_root32 = nullptr;
-    t.d_root64 = nullptr;
 }
 
 }  // namespace bte
