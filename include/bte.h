@@ -300,7 +300,9 @@ bte_status bte_graph_count(const bte_ctx *ctx, int64_t *count);
  *                      ranges (chosen when the batch is built, by simulating
  *                      the work queue on 3 CTAs per SM); the half that
  *                      finishes second adds both halves' sums in a fixed
- *                      order (deterministic); 0 runs every pencil whole;
+ *                      order (deterministic), and batches of few cells run a
+ *                      convolution with pairs instead of cells in the lanes;
+ *                      0 runs every pencil whole;
  *       "learned_tol_ppm" fallback threshold of the learned mode in 1e-6 units;
  *       "dft_fuse_stages" 1 (default): in an FP32 Heun step the first stage's
  *                      inverse transform also forms the second stage's forward

@@ -558,6 +558,21 @@ bte_status prepare(bte_ctx *c, Batch *B, int mode, bool step, bool transport) {
 // half full one by one (lanes over the sum instead of cells).
 bool by_cells64(const Segment &sg) { return 2 * sg.nvalid <= sg.nslots; }
 
+// The batch has so few cells that the FP32 convolution runs with pairs in lanes
+// (conv32_cells.cu), part of the split plan (conv_split 1) of variant 4. Its cost
+// is proportional to the cells, one segment after the other, and equals that of
+// the kernels with cells in lanes at the limit: the shares of the limit add up.
+bool by_cells32(const bte_ctx *c, const Batch *B, const ConvCfg &g) {
+    if (g.impl != 4 || !g.csplit || c->debug_conv_stall) return false;
+    double share = 0.0;
+    for (const Segment &sg : B->segs) {
+        const int limit = conv32_cells_limit(c->tables[sg.table]->N);
+        if (sg.nvalid > limit) return false;
+        share += (double)sg.nvalid / limit;
+    }
+    return share <= 1.0;
+}
+
 // What happens after the inverse transform of a collide.
 enum Post { POST_RAW = 0, POST_PROJECT = 1, POST_STAGE1 = 2, POST_STAGE2 = 3 };
 
@@ -573,6 +588,7 @@ bte_status enqueue_collide(bte_ctx *c, Batch *B, const double *f, double *Q, int
     NvtxRange range_collide("bte_collide");
     const bool fp64 = mode == BTE_FP64_PLAIN;
     const ConvCfg cfg = cfg_of(c, B);
+    const bool cells32 = !fp64 && by_cells32(c, B, cfg);
     ProfEntry pe_all{}, pe_conv{}, pe_fwd{}, pe_inv{};
     const int on_all = prof_begin(c, PK_COLLIDE, st, &pe_all);
     if (!(fuse & FUSE_SKIP_FWD)) {
@@ -580,7 +596,7 @@ bte_status enqueue_collide(bte_ctx *c, Batch *B, const double *f, double *Q, int
         const int on_fwd = prof_begin(c, PK_FORWARD, st, &pe_fwd);
         for (const Segment &sg : B->segs) {
             const Table *t = c->tables[sg.table];
-            DftSeg ds{t->N, sg.s0, sg.nslots, sg.eoff, sg.nvalid};
+            DftSeg ds{t->N, sg.s0, sg.nslots, sg.eoff, sg.nvalid, cells32};
             const double sf = std::pow(2.0 * kPi, -1.5) * t->dv * t->dv * t->dv;
             if (fp64 || !fused_dft_supported(t->N))
                 count_launches(c, launch_dft_forward(f, B->d_slot_off, ds, sf, c->scratch[SC_T1], c->scratch[SC_F],
@@ -609,6 +625,13 @@ bte_status enqueue_collide(bte_ctx *c, Batch *B, const double *f, double *Q, int
             count_launches(c, 1);
         }
         prof_end(c, on, pe_conv, st);
+    } else if (cells32) {
+        const int on = prof_begin(c, PK_CONV32, st, &pe_conv);
+        for (const Segment &sg : B->segs)
+            launch_conv32_cells((const float2 *)c->scratch[SC_F], (float2 *)c->scratch[SC_QH], *c->tables[sg.table],
+                                sg.nvalid, sg.eoff, st);
+        prof_end(c, on, pe_conv, st);
+        count_launches(c, (int)B->segs.size());
     } else {
         ConvLaunch L;
         cudaError_t e = conv32_configure(B->kinds_mask, c->num_sms, cfg.warps, cfg.stages, cfg.impl, &L);
@@ -657,7 +680,7 @@ bte_status enqueue_collide(bte_ctx *c, Batch *B, const double *f, double *Q, int
     const int on_inv = prof_begin(c, PK_INVERSE, st, &pe_inv);
     for (const Segment &sg : B->segs) {
         const Table *t = c->tables[sg.table];
-        DftSeg ds{t->N, sg.s0, sg.nslots, sg.eoff, sg.nvalid};
+        DftSeg ds{t->N, sg.s0, sg.nslots, sg.eoff, sg.nvalid, cells32};
         const double si = std::pow(2.0 * kPi, -1.5) * t->dz * t->dz * t->dz;
         if (fuse & FUSE_NEXT_FWD) {  // post == POST_STAGE1 (checked by the caller)
             const double sf = std::pow(2.0 * kPi, -1.5) * t->dv * t->dv * t->dv;
@@ -1495,6 +1518,8 @@ bte_status bte_autotune(bte_ctx *c, const double *f, const bte_instance *inst, i
     double *Qtmp = (double *)c->scratch[SC_Q2];
     bool small_n = true;
     for (const Segment &sg : B->segs) small_n = small_n && c->tables[sg.table]->N <= 16;
+    ConvCfg split_cfg;
+    const bool cells = by_cells32(c, B, split_cfg);  // conv_split 1 of variant 4: pairs in lanes
     const std::string key = tune_key(B);
     const bool had = c->tuned.count(key) != 0;
     const ConvCfg before = had ? c->tuned[key] : ConvCfg{};
@@ -1514,7 +1539,7 @@ bte_status bte_autotune(bte_ctx *c, const double *f, const bte_instance *inst, i
                     for (int split : {4, 2, 1})
                         for (int csplit : {1, 0}) {
                         if (!small_n && split != 4) continue;
-                        if (csplit && (impl != 4 || B->nsplit == 0)) continue;
+                        if (csplit && (impl != 4 || (B->nsplit == 0 && !cells))) continue;
                         // kinds of N = 48: variant 4, and 3 when they are the only kinds
                         if ((B->kinds_mask >> 7) && impl != 4 && !(impl == 3 && B->kinds_mask == (128u | 256u | 512u)))
                             continue;

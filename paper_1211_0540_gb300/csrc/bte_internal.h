@@ -133,6 +133,11 @@ struct Table {
     // which bte_collide_noalloc expands its work list on the device.
     ConvItem *d_tmpl = nullptr;
     int n_tmpl = 0;
+    // The convolution with pairs in lanes (N <= 32): per tile the entries of a block
+    // (m3 | n3 << 8, conv32_cells_entries(N) a tile), and the entry of each (visit,
+    // output j), [tile][pair_visits][T], -1 if none
+    uint16_t *d_ent = nullptr;
+    int16_t *d_rk = nullptr;
     // DFT roots exp(2 pi i t / N), t in [0, N)
     float2 *d_root32 = nullptr;
     // Projection: (C C^T)^{-1}, row-major 5x5 (C without the dv^3 factor folded in)
@@ -249,6 +254,9 @@ struct bte_ctx {
 };
 
 namespace bte {
+
+// conv32_cells.cu: entries per k3 tile, padded to whole warps (0: N unsupported)
+int conv32_cells_entries(int N);
 
 // tables.cpp
 int build_table(Table &t, std::string &err);

@@ -95,6 +95,13 @@ __device__ __forceinline__ void pencil_cr(const float2 (&x)[N], float (&y)[N], c
     for (int k = 0; k < N; ++k) y[k] = z[k].x;
 }
 
+// Mode 0 of a slot's fhat or Qhat and the distance between modes: the group
+// layout of the convolution, or cell-major (DftSeg.cells).
+__device__ __forceinline__ int64_t cell_base(const DftSeg &s, int sl, int64_t M) {
+    return s.eoff + (s.cells ? sl * M : (int64_t)(sl / kLanes) * M * kLanes + sl % kLanes);
+}
+__device__ __forceinline__ int cell_stride(const DftSeg &s) { return s.cells ? 1 : kLanes; }
+
 // Cluster barrier without memory ordering: only keeps every CTA of the
 // cluster resident until all of them got here (their remote reads of this
 // CTA's shared memory have completed, since the values were consumed).
@@ -159,10 +166,11 @@ dft_fwd_fused_kernel(const double *__restrict__ f, const int64_t *__restrict__ s
     const int r = (int)cl.block_rank(), sl = blockIdx.x / C, t = threadIdx.x;
     const int64_t off = slot_off[s.s0 + sl];
     if (off == -2) return;  // a slot of a group that holds no cell this call (nothing reads it)
-    float2 *g = G + s.eoff + (int64_t)(sl / kLanes) * M * kLanes;
-    const int ln = sl % kLanes;
-    auto gi = [ln](int e) -> int64_t { return SECTOR ? sector_index(e, ln) : (int64_t)e * kLanes + ln; };
+    float2 *g = SECTOR ? G + s.eoff + (int64_t)(sl / kLanes) * M * kLanes : G + cell_base(s, sl, M);
+    const int ln = sl % kLanes, stride = cell_stride(s);
+    auto gi = [ln, stride](int e) -> int64_t { return SECTOR ? sector_index(e, ln) : (int64_t)e * stride; };
     if (off < 0) {  // padding lane of a group (the whole cluster leaves here): zero fhat
+        if (!SECTOR && s.cells) return;
         for (int e = r * (M / C) + t; e < (r + 1) * (M / C); e += S::NT) g[gi(e)] = make_float2(0.f, 0.f);
         return;
     }
@@ -190,7 +198,7 @@ dft_fwd_fused_kernel(const double *__restrict__ f, const int64_t *__restrict__ s
         for (int k = 0; k < N; ++k) B[(jl * N + k) * N + k3] = y[k];
     }
     cell_sync<C>(cl);
-    if (act) {  // along j1, pencil (k2, k3), rows from every CTA of the cluster, into the group layout
+    if (act) {  // along j1, pencil (k2, k3), rows from every CTA of the cluster, into fhat's layout
         const int k2 = r * JR + t / N, k3 = t % N;
         const float2 *src[C];
 #pragma unroll
@@ -310,13 +318,14 @@ dft_inv_fused_kernel(const float2 *__restrict__ G, const int64_t *__restrict__ s
     }
     const float2(&rt)[N] = CRoot<N>::get();
     const bool act = t < NP;
-    const float2 *g = G + s.eoff + (int64_t)(sl / kLanes) * M * kLanes + (sl % kLanes);
-    if (act) {  // along k1, pencil (k2, k3), from the group layout (the stored half of the pencils; the rest is 0)
+    const float2 *g = G + cell_base(s, sl, M);
+    const int stride = cell_stride(s);
+    if (act) {  // along k1, pencil (k2, k3), from Qhat's layout (the stored half of the pencils; the rest is 0)
         const int pk = (r * JR + t / N) * N + t % N, k2 = pk / N;
         float2 xx[N], yy[N];
 #pragma unroll
         for (int k = 0; k < N; ++k)
-            xx[k] = pencil_stored(k, k2, N) ? g[(int64_t)(k * NN + pk) * kLanes] : make_float2(0.f, 0.f);
+            xx[k] = pencil_stored(k, k2, N) ? g[(int64_t)(k * NN + pk) * stride] : make_float2(0.f, 0.f);
         pencil_cc<N, false>(xx, yy, rt);
         const int kl = t / N, k3 = t % N;
 #pragma unroll
@@ -498,7 +507,7 @@ dft_inv_fused_kernel(const float2 *__restrict__ G, const int64_t *__restrict__ s
             for (int k = 0; k < N; ++k) Bf[(jl * N + k) * N + k3] = yy[k];
         }
         cell_sync<C>(cl);
-        if (act) {  // along j1, pencil (k2, k3), rows from every CTA of the cluster, into the group layout
+        if (act) {  // along j1, pencil (k2, k3), rows from every CTA of the cluster, into fhat's layout
             const int k2 = r * JR + t / N, k3 = t % N;
             const float2 *src[C];
 #pragma unroll
@@ -507,17 +516,19 @@ dft_inv_fused_kernel(const float2 *__restrict__ G, const int64_t *__restrict__ s
 #pragma unroll
             for (int j = 0; j < N; ++j) xx[j] = src[j / JR][((j % JR) * N + k2) * N + k3];
             pencil_cc<N, true>(xx, yy, rt);
-            float2 *go = Gout + s.eoff + (int64_t)(sl / kLanes) * M * kLanes + (sl % kLanes);
+            float2 *go = Gout + cell_base(s, sl, M);
             const int pk = k2 * N + k3;
 #pragma unroll
             for (int k = 0; k < N; ++k)
-                go[(int64_t)(k * NN + pk) * kLanes] = make_float2(fscale * yy[k].x, fscale * yy[k].y);
+                go[(int64_t)(k * NN + pk) * stride] = make_float2(fscale * yy[k].x, fscale * yy[k].y);
         }
         if constexpr (C > 1) cluster_barrier_relaxed();  // no CTA leaves while its slab may still be read
     }
 }
 
 namespace {
+// cell-major: the padding slots have nothing to write
+int grid_slots(const DftSeg &s) { return s.cells ? s.nvalid : s.nslots; }
 template <int N, int C>
 void fwd_launch(const double *f, const int64_t *slot_off, const DftSeg &s, const float2 *root, double scale,
                 float2 *G, int *status, cudaStream_t st, bool sector) {
@@ -529,7 +540,7 @@ void fwd_launch(const double *f, const int64_t *slot_off, const DftSeg &s, const
             return;
         }
     }
-    dft_fwd_fused_kernel<N, C><<<s.nslots * C, S::NT, S::smem_fwd, st>>>(f, slot_off, s, root, (float)scale, G,
+    dft_fwd_fused_kernel<N, C><<<grid_slots(s) * C, S::NT, S::smem_fwd, st>>>(f, slot_off, s, root, (float)scale, G,
                                                                         status);
 }
 template <int N, int C>
@@ -537,7 +548,7 @@ void inv_launch(const float2 *G, const int64_t *slot_off, const DftSeg &s, const
                 double *q, const ProjArgs &pa, int mode, const double *x, double *y, const double *qp, double a,
                 cudaStream_t st) {
     using S = FusedShape<N, C>;
-    dft_inv_fused_kernel<N, C><<<s.nslots * C, S::NT, S::smem_inv, st>>>(G, slot_off, s, root, (float)scale, q, pa,
+    dft_inv_fused_kernel<N, C><<<grid_slots(s) * C, S::NT, S::smem_inv, st>>>(G, slot_off, s, root, (float)scale, q, pa,
                                                                         mode, x, y, qp, a);
 }
 template <int N, int C>
@@ -545,7 +556,7 @@ void inv_fwd_launch(const float2 *G, const int64_t *slot_off, const DftSeg &s, c
                     double *q, const ProjArgs &pa, const double *x, double a, double fscale, float2 *Gout,
                     int *status, cudaStream_t st) {
     using S = FusedShape<N, C>;
-    dft_inv_fused_kernel<N, C, true><<<s.nslots * C, S::NT, S::smem_inv, st>>>(
+    dft_inv_fused_kernel<N, C, true><<<grid_slots(s) * C, S::NT, S::smem_inv, st>>>(
         G, slot_off, s, root, (float)scale, q, pa, 2, x, nullptr, nullptr, a, Gout, (float)fscale, status);
 }
 template <int N, int C>

@@ -13,6 +13,9 @@ struct DftSeg {
     int nslots;    // slots in the segment (multiple of 32)
     int64_t eoff;  // complex-element offset of slot s0 in scratch / group buffers
     int nvalid = 0;  // slots that hold a cell, the first ones (read by the transforms of dft.cu only)
+    // FP32 fhat and Qhat cell-major ([slot][m], the convolution with pairs in
+    // lanes) instead of the group layout
+    bool cells = false;
 };
 
 // Projection (Sec. 3.3), optionally fused with the RK2 update:
@@ -83,6 +86,12 @@ struct ConvLaunch {
 cudaError_t conv32_configure(unsigned kinds_mask, int num_sms, int warps_per_cta, int stages, int impl,
                              ConvLaunch *out);
 cudaError_t conv32_launch(const ConvLaunch &L, const ConvParams &p, cudaStream_t st);
+
+// FP32 convolution of one segment with pairs in lanes, for few cells; fhat and
+// Qhat cell-major. Faster than the kernels with cells in lanes up to
+// conv32_cells_limit(N) cells.
+int conv32_cells_limit(int N);
+void launch_conv32_cells(const float2 *F, float2 *Qh, const Table &t, int nvalid, int64_t eoff, cudaStream_t st);
 
 // FP64 convolution of one segment (the modes of the stored pencils).
 void launch_conv64(const double2 *F, double2 *Qh, const Table &t, int64_t eoff, int ngroups, cudaStream_t st);

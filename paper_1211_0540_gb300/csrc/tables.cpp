@@ -355,12 +355,29 @@ int build_table(Table &t, std::string &err) {
         }
     }
 
+    // the entries of a block for the convolution with pairs in lanes
+    const int ne = conv32_cells_entries(N), nv = pair_visits(N, T);
+    std::vector<uint16_t> ent((size_t)t.ntiles * ne, 0);
+    std::vector<int16_t> rk(ne ? (size_t)t.ntiles * nv * T : 0, -1);
+    for (int tile = 0; ne && tile < t.ntiles; ++tile) {
+        int e = 0;
+        for (int i = 0; i < nv; ++i)
+            for (int j = 0; j < T; ++j) {
+                const int k3 = tile * T + j, m3 = i % N;
+                if (!pair_visit(k3, i, N, T)) continue;
+                ent[(size_t)tile * ne + e] = (uint16_t)(m3 | pair_partner(k3, m3, N) << 8);
+                rk[((size_t)tile * nv + i) * T + j] = (int16_t)e++;
+            }
+    }
+
     // upload
     cudaError_t e = cudaSuccess;
     e = cudaMalloc(&t.d_tmpl, sizeof(ConvItem) * std::max<size_t>(tmpl.size(), 1));
     if (e == cudaSuccess && !I32.empty()) e = cudaMalloc(&t.d_I32, sizeof(float) * I32.size());
     if (e == cudaSuccess && !J32.empty()) e = cudaMalloc(&t.d_J32, sizeof(float) * J32.size());
     if (e == cudaSuccess && !etab.empty()) e = cudaMalloc(&t.d_etab, sizeof(uint16_t) * etab.size());
+    if (e == cudaSuccess && ne) e = cudaMalloc(&t.d_ent, sizeof(uint16_t) * ent.size());
+    if (e == cudaSuccess && ne) e = cudaMalloc(&t.d_rk, sizeof(int16_t) * rk.size());
     if (e == cudaSuccess) e = cudaMalloc(&t.d_desc, sizeof(uint32_t) * std::max<size_t>(t.n_desc, 1));
     if (e == cudaSuccess) e = cudaMalloc(&t.d_root32, sizeof(float2) * N);
     if (e != cudaSuccess) {
@@ -374,6 +391,10 @@ int build_table(Table &t, std::string &err) {
         e = cudaMemcpy(t.d_I32, I32.data(), sizeof(float) * I32.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess && !J32.empty())
         e = cudaMemcpy(t.d_J32, J32.data(), sizeof(float) * J32.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && ne)
+        e = cudaMemcpy(t.d_ent, ent.data(), sizeof(uint16_t) * ent.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && ne)
+        e = cudaMemcpy(t.d_rk, rk.data(), sizeof(int16_t) * rk.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess && !etab.empty())
         e = cudaMemcpy(t.d_etab, etab.data(), sizeof(uint16_t) * etab.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
@@ -514,6 +535,10 @@ void free_table(Table &t) {
     cudaFree(t.d_I32);
     cudaFree(t.d_J32);
     cudaFree(t.d_etab);
+    cudaFree(t.d_ent);
+    cudaFree(t.d_rk);
+    t.d_ent = nullptr;
+    t.d_rk = nullptr;
     t.d_tmpl = nullptr;
     t.d_I32 = t.d_J32 = nullptr;
     t.d_etab = nullptr;
