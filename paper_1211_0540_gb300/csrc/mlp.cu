@@ -38,15 +38,15 @@ __device__ __forceinline__ float gelu_grad(float x) {
     return 0.5f * (1.0f + t) + 0.5f * x * (1.0f - t * t) * k0 * (1.0f + 3.0f * k1 * x * x);
 }
 
-// One CTA per batch row: rho, x (bf16, optionally transposed) and the target.
+// One CTA per batch row: rho, x (bf16) and, in training, the target.
 // Each value is converted to FP32 once (kept in shared memory, M <= 4096) and
 // rho is summed in double-float FP32: its ~1e-7 relative precision only
 // scales the surrogate's input and output, whose conservation the projection
 // restores exactly.
 __global__ void __launch_bounds__(kT) prep_kernel(const double *__restrict__ f, const int64_t *__restrict__ off,
                                                    int B, int M, double dv3, float s_in, __nv_bfloat16 *X,
-                                                   __nv_bfloat16 *Xt, int ldt, double *rho_out,
-                                                   const double *__restrict__ Q, float s_out, float *T) {
+                                                   double *rho_out, const double *__restrict__ Q, float s_out,
+                                                   float *T) {
     const int r = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const double *fr = f + off[r];
     __shared__ float xs[4096];
@@ -54,12 +54,13 @@ __global__ void __launch_bounds__(kT) prep_kernel(const double *__restrict__ f, 
     __shared__ double rho_s;
     Df s{0.f, 0.f};
     int j = threadIdx.x;
-    for (; j + 3 * kT < M; j += 4 * kT) {  // four loads in flight per thread, summed in the same order
-        double d[4];
+    constexpr int kAhead = 8;
+    for (; j + (kAhead - 1) * kT < M; j += kAhead * kT) {  // loads in flight per thread, summed in the same order
+        double d[kAhead];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) d[u] = fr[j + u * kT];
+        for (int u = 0; u < kAhead; ++u) d[u] = fr[j + u * kT];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < kAhead; ++u) {
             const float v = fpc::narrow(d[u]);  // integer pipes, not the FP64 unit
             xs[j + u * kT] = v;
             df_add(s, v);
@@ -87,16 +88,53 @@ __global__ void __launch_bounds__(kT) prep_kernel(const double *__restrict__ f, 
     __syncthreads();
     const double rho = rho_s;
     const float a = rho != 0.0 ? (float)((double)s_in / rho) : 0.f;  // a vacuum cell (rho = 0) gets x = 0
-    for (int j = threadIdx.x; j < M; j += blockDim.x) {
-        const __nv_bfloat16 x = __float2bfloat16_rn(xs[j] * a);
-        X[(size_t)r * M + j] = x;
-        if (Xt) Xt[(size_t)j * ldt + r] = x;
-    }
+    // M is a multiple of 64: two values a thread
+    __nv_bfloat162 *X2 = reinterpret_cast<__nv_bfloat162 *>(X + (size_t)r * M);
+    for (int j = threadIdx.x; j < M / 2; j += kT) X2[j] = __floats2bfloat162_rn(xs[2 * j] * a, xs[2 * j + 1] * a);
     if (T) {
         const double c = (double)s_out / (rho * rho);
         const double *qr = Q + off[r];
-        for (int j = threadIdx.x; j < M; j += blockDim.x) T[(size_t)r * M + j] = (float)(qr[j] * c);
+        for (int j = threadIdx.x; j < M; j += kT) T[(size_t)r * M + j] = fpc::narrow(qr[j] * c);
     }
+}
+
+// The transposed copies that the weight gradients read as their K operand go
+// through shared memory in tiles of 64 x 64, 16-byte rows on both sides: stored
+// from the row kernels, each 2-byte value took a sector of its own (batch 1024,
+// M = 4096: the input's kernel 59 -> 44 us with its transpose, the loss 43 -> 23,
+// the GELU's backward pass 13 -> 8).
+constexpr int kTile = 64, kTileLd = kTile + 2;
+
+// the tile (rows r0.., columns c0..) of s to out[c][ldt], rows up to the tile's end
+// (rows past the batch are 0: the padding columns of the transposed array)
+__device__ __forceinline__ void store_tile_t(const __nv_bfloat16 (&s)[kTile][kTileLd], __nv_bfloat16 *out, int ldt,
+                                             int r0, int c0) {
+    for (int i = threadIdx.x; i < kTile * kTile / 8; i += kT) {
+        const int c = i / (kTile / 8), q = 8 * (i % (kTile / 8));
+        __align__(16) __nv_bfloat16 v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = s[q + k][c];
+        *reinterpret_cast<uint4 *>(out + (size_t)(c0 + c) * ldt + r0 + q) = *reinterpret_cast<const uint4 *>(v);
+    }
+}
+
+// out[c][ldt] = x[r][n] transposed; n a multiple of 64, ldt of 128.
+__global__ void __launch_bounds__(kT) transpose_kernel(const __nv_bfloat16 *__restrict__ x, int B, int n,
+                                                       __nv_bfloat16 *__restrict__ out, int ldt) {
+    __shared__ __nv_bfloat16 s[kTile][kTileLd];
+    const int c0 = blockIdx.x * kTile, r0 = blockIdx.y * kTile;
+    for (int i = threadIdx.x; i < kTile * kTile / 8; i += kT) {
+        const int r = i / (kTile / 8), q = 8 * (i % (kTile / 8));
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (r0 + r < B) v = *reinterpret_cast<const uint4 *>(x + (size_t)(r0 + r) * n + c0 + q);
+        uint32_t *o = reinterpret_cast<uint32_t *>(&s[r][q]);
+        o[0] = v.x;
+        o[1] = v.y;
+        o[2] = v.z;
+        o[3] = v.w;
+    }
+    __syncthreads();
+    store_tile_t(s, out, ldt, r0, c0);
 }
 
 // Per cell of a uniform array: rho = sum f dv^3 and sum_j Q_j^2 / rho^4 (the
@@ -127,22 +165,20 @@ __global__ void __launch_bounds__(kT) target_norm_kernel(const double *__restric
     }
 }
 
-// d = Y - T; loss partial per row; dY = 2 d / (B M) in bf16 (row-major and transposed) and FP32.
+// d = Y - T; loss partial per row; dY = 2 d / (B M) in bf16 and FP32.
 __global__ void __launch_bounds__(kT) loss_kernel(const float *__restrict__ Y, const float *__restrict__ T, int B,
-                                                   int M, __nv_bfloat16 *dY, __nv_bfloat16 *dYt, int ldt, float *dYf,
-                                                   double *loss_rows) {
+                                                   int M, __nv_bfloat16 *dY, float *dYf, double *loss_rows) {
     const int r = blockIdx.x;
     __shared__ double red[kT / 32];
     const float g = 2.0f / ((float)B * (float)M);
     double s = 0.0;
-    for (int j = threadIdx.x; j < M; j += blockDim.x) {
+    for (int j = threadIdx.x; j < M; j += kT) {
         const float d = Y[(size_t)r * M + j] - T[(size_t)r * M + j];
-        s += (double)d * d;
+        const double w = fpc::widen(d);
+        s = fma(w, w, s);
         const float gd = g * d;
         dYf[(size_t)r * M + j] = gd;
-        const __nv_bfloat16 b = __float2bfloat16_rn(gd);
-        dY[(size_t)r * M + j] = b;
-        dYt[(size_t)j * ldt + r] = b;
+        dY[(size_t)r * M + j] = __float2bfloat16_rn(gd);
     }
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
@@ -154,30 +190,60 @@ __global__ void __launch_bounds__(kT) loss_kernel(const float *__restrict__ Y, c
     }
 }
 
-// dZ = (dH + dH2) * gelu'(Z): bf16 row-major (optional), bf16 transposed, FP32.
-__global__ void gelu_bwd_kernel(const float *__restrict__ dH, const float *__restrict__ dH2,
-                                const float *__restrict__ Z, int B, int n, __nv_bfloat16 *dZ, __nv_bfloat16 *dZt,
-                                int ldt, float *dZf) {
-    const int64_t total = (int64_t)B * n;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int r = (int)(i / n), c = (int)(i % n);
-        float d = dH[i];
-        if (dH2) d += dH2[i];
-        const float v = d * gelu_grad(Z[i]);
-        dZf[i] = v;
-        const __nv_bfloat16 b = __float2bfloat16_rn(v);
-        if (dZ) dZ[i] = b;
-        dZt[(size_t)c * ldt + r] = b;
+// dZ = (dH + dH2) * gelu'(Z) in tiles of 64 x 64: bf16 row-major (optional), bf16
+// transposed, FP32. n is a multiple of 64.
+__global__ void __launch_bounds__(kT) gelu_bwd_kernel(const float *__restrict__ dH, const float *__restrict__ dH2,
+                                                      const float *__restrict__ Z, int B, int n, __nv_bfloat16 *dZ,
+                                                      __nv_bfloat16 *dZt, int ldt, float *dZf) {
+    __shared__ __nv_bfloat16 s[kTile][kTileLd];
+    const int c0 = blockIdx.x * kTile, r0 = blockIdx.y * kTile;
+    for (int i = threadIdx.x; i < kTile * kTile / 2; i += kT) {
+        const int r = i / (kTile / 2), c = 2 * (i % (kTile / 2));
+        const size_t o = (size_t)(r0 + r) * n + c0 + c;
+        __nv_bfloat162 b = __floats2bfloat162_rn(0.f, 0.f);
+        if (r0 + r < B) {
+            const float2 h = *reinterpret_cast<const float2 *>(dH + o), z = *reinterpret_cast<const float2 *>(Z + o);
+            const float2 h2 = dH2 ? *reinterpret_cast<const float2 *>(dH2 + o) : make_float2(0.f, 0.f);
+            const float v0 = (dH2 ? h.x + h2.x : h.x) * gelu_grad(z.x);
+            const float v1 = (dH2 ? h.y + h2.y : h.y) * gelu_grad(z.y);
+            *reinterpret_cast<float2 *>(dZf + o) = make_float2(v0, v1);
+            b = __floats2bfloat162_rn(v0, v1);
+            if (dZ) *reinterpret_cast<__nv_bfloat162 *>(dZ + o) = b;
+        }
+        *reinterpret_cast<__nv_bfloat162 *>(&s[r][c]) = b;
     }
+    __syncthreads();
+    store_tile_t(s, dZt, ldt, r0, c0);
 }
 
-// out[c] = sum over rows of x[r][c] (fixed order).
-__global__ void colsum_kernel(const float *__restrict__ x, int B, int n, float *out) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= n) return;
-    float s = 0.f;
-    for (int r = 0; r < B; ++r) s += x[(size_t)r * n + c];
-    out[c] = s;
+// out[c] = sum over rows of x[r][c]: 32 columns per CTA, its 32 rows of threads
+// take every 32nd row (four loads in flight) and are added by a fixed tree. One
+// thread per column took 70 us for 1024 rows, whatever the columns (a chain of
+// 1024 loads); 6 us now.
+constexpr int kColRows = 32;
+__global__ void __launch_bounds__(32 * kColRows) colsum_kernel(const float *__restrict__ x, int B, int n, float *out) {
+    __shared__ float s[kColRows][33];
+    const int cx = threadIdx.x & 31, ry = threadIdx.x >> 5, c = blockIdx.x * 32 + cx;
+    float a = 0.f;
+    if (c < n) {
+        int r = ry;
+        for (; r + 3 * kColRows < B; r += 4 * kColRows) {
+            float v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = x[(size_t)(r + u * kColRows) * n + c];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) a += v[u];
+        }
+        for (; r < B; r += kColRows) a += x[(size_t)r * n + c];
+    }
+    s[ry][cx] = a;
+    __syncthreads();
+#pragma unroll
+    for (int o = kColRows / 2; o > 0; o >>= 1) {
+        if (ry < o) s[ry][cx] += s[ry + o][cx];
+        __syncthreads();
+    }
+    if (ry == 0 && c < n) out[c] = s[0][cx];
 }
 
 __global__ void adamw_kernel(float *p, const float *__restrict__ g, float *m, float *v, int64_t n, float lr, float b1,
@@ -305,8 +371,9 @@ int Mlp::run(const double *f, const double *Qt, int B, bool training, int *statu
                         std::make_pair((void *)dZ1t, bh)})
             if (cudaMemsetAsync(pr.first, 0, pr.second, st) != cudaSuccess) return -1;
     }
-    prep_kernel<<<B, kT, 0, st>>>(f, rows, B, M, dv3, s_in, X, training ? Xt : nullptr, Bp, rho, Qt, s_out,
-                                  training ? T : nullptr);
+    prep_kernel<<<B, kT, 0, st>>>(f, rows, B, M, dv3, s_in, X, rho, Qt, s_out, training ? T : nullptr);
+    const int tr = (B + kTile - 1) / kTile;  // tiles of rows
+    if (training) transpose_kernel<<<dim3(M / kTile, tr), kT, 0, st>>>(X, B, M, Xt, Bp);
     GemmEpi g1;
     g1.bias = params + off_b1();
     g1.out_f32 = training ? Z1 : nullptr;
@@ -336,8 +403,9 @@ int Mlp::run(const double *f, const double *Qt, int B, bool training, int *statu
     if (gemm_bf16(H2, w3, B, M, H, g3, status, st)) return -1;
     if (!training) return 0;
     // backward
-    loss_kernel<<<B, kT, 0, st>>>(Y, T, B, M, dY, dYt, Bp, dYf, loss_rows);
-    colsum_kernel<<<(M + kT - 1) / kT, kT, 0, st>>>(dYf, B, M, grads + off_b3());
+    loss_kernel<<<B, kT, 0, st>>>(Y, T, B, M, dY, dYf, loss_rows);
+    transpose_kernel<<<dim3(M / kTile, tr), kT, 0, st>>>(dY, B, M, dYt, Bp);
+    colsum_kernel<<<(M + 31) / 32, 32 * kColRows, 0, st>>>(dYf, B, M, grads + off_b3());
     GemmEpi gw3;  // dW3 = dY^T H2   [M x H]
     gw3.out_f32 = grads + off_W3();
     gw3.ld_f32 = H;
@@ -346,8 +414,8 @@ int Mlp::run(const double *f, const double *Qt, int B, bool training, int *statu
     gh2.out_f32 = dH2;
     gh2.ld_f32 = H;
     if (gemm_bf16(dY, w3t, B, H, M, gh2, status, st)) return -1;
-    gelu_bwd_kernel<<<blocks_for((int64_t)B * H, kT), kT, 0, st>>>(dH2, nullptr, Z2, B, H, dZ2, dZ2t, Bp, dZf);
-    colsum_kernel<<<(H + kT - 1) / kT, kT, 0, st>>>(dZf, B, H, grads + off_b2());
+    gelu_bwd_kernel<<<dim3(H / kTile, tr), kT, 0, st>>>(dH2, nullptr, Z2, B, H, dZ2, dZ2t, Bp, dZf);
+    colsum_kernel<<<(H + 31) / 32, 32 * kColRows, 0, st>>>(dZf, B, H, grads + off_b2());
     GemmEpi gw2;  // dW2 = dZ2^T H1  [H x H]
     gw2.out_f32 = grads + off_W2();
     gw2.ld_f32 = H;
@@ -356,8 +424,8 @@ int Mlp::run(const double *f, const double *Qt, int B, bool training, int *statu
     gh1.out_f32 = dH1;
     gh1.ld_f32 = H;
     if (gemm_bf16(dZ2, w2t, B, H, H, gh1, status, st)) return -1;
-    gelu_bwd_kernel<<<blocks_for((int64_t)B * H, kT), kT, 0, st>>>(dH1, dH2, Z1, B, H, nullptr, dZ1t, Bp, dZf);
-    colsum_kernel<<<(H + kT - 1) / kT, kT, 0, st>>>(dZf, B, H, grads + off_b1());
+    gelu_bwd_kernel<<<dim3(H / kTile, tr), kT, 0, st>>>(dH1, dH2, Z1, B, H, nullptr, dZ1t, Bp, dZf);
+    colsum_kernel<<<(H + 31) / 32, 32 * kColRows, 0, st>>>(dZf, B, H, grads + off_b1());
     GemmEpi gw1;  // dW1 = dZ1^T X   [H x M]
     gw1.out_f32 = grads + off_W1();
     gw1.ld_f32 = M;
