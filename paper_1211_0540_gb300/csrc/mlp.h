@@ -27,9 +27,14 @@ struct Mlp {
     float *Z1 = nullptr, *Z2 = nullptr, *Y = nullptr, *T = nullptr, *dYf = nullptr, *dH2 = nullptr, *dH1 = nullptr,
           *dZf = nullptr;
     double *rho = nullptr, *loss_rows = nullptr;
-    int64_t *rowoff = nullptr;  // row offsets of the current call (uploaded)
     int64_t *rowuni = nullptr;  // i * M for i < bcap: rows of a contiguous block of cells
     std::vector<void *> allocs, act_allocs;
+    // pinned slots of the gradient's copy to the host (allocated by the first large one)
+    static constexpr size_t kSlotBytes = (size_t)1 << 20;
+    static constexpr int kSlots = 24;
+    char *slots = nullptr;
+    cudaEvent_t slot_ready[kSlots] = {};
+    bool ensure_slots();
 
     ~Mlp();
     bool alloc(void **p, size_t bytes);
@@ -44,7 +49,7 @@ struct Mlp {
     size_t nparams() const;
     void refresh_bf16(cudaStream_t st);
     int run(const double *f, const double *Qt, int B, bool training, int *status, cudaStream_t st,
-            const int64_t *rows = nullptr);
+            const int64_t *rows);
     void adam_step(float lr, float wd, cudaStream_t st);
 };
 
