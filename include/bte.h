@@ -296,12 +296,12 @@ bte_status bte_graph_count(const bte_ctx *ctx, int64_t *count);
  *       "graph_cache" captured step graphs kept (1..2^20, default 32; see
  *                      bte_graph_count);
  *       "conv_split"  variant 4: 1 (default) runs the batch's plan in which
- *                      the costliest pencil items are cut into two block
- *                      ranges (chosen when the batch is built, by simulating
- *                      the work queue on 3 CTAs per SM); the half that
- *                      finishes second adds both halves' sums in a fixed
- *                      order (deterministic), and batches of few cells run a
- *                      convolution with pairs instead of cells in the lanes;
+ *                      pencil items are cut into block ranges (chosen when the
+ *                      batch is built, by simulating the work queue on the
+ *                      resident CTAs); the part that finishes last adds all
+ *                      parts' sums in a fixed order (deterministic), and
+ *                      batches of few cells run a convolution with pairs
+ *                      instead of cells in the lanes;
  *                      0 runs every pencil whole;
  *       "learned_tol_ppm" fallback threshold of the learned mode in 1e-6 units;
  *       "dft_fuse_stages" 1 (default): in an FP32 Heun step the first stage's

@@ -38,10 +38,11 @@ struct Batch {
     int64_t *d_slot_out = nullptr;
     ConvItem *d_items = nullptr;
     int nitems = 0;
-    // the same work with the costliest items split into two block ranges
-    // (convolution variant 4): items, split codes, partial sums, counters
-    // ([0] the queue, [1 + sid] the halves of split sid that finished)
+    // the same work with items split into block ranges (convolution variants 4, 5):
+    // items, split codes, the parts' sums (nsplit slots), counters ([0] the queue,
+    // [1 + first slot] the finished parts of a split item)
     ConvItem *d_items_split = nullptr;
+    int *d_halves = nullptr;   // the split codes as halves, when no item has more parts
     int nitems_split = 0, nsplit = 0;
     int *d_split = nullptr;
     float *d_part = nullptr;
@@ -226,106 +227,140 @@ void free_batch(Batch *B) {
     cudaFree(B->d_items);
     cudaFree(B->d_items_split);
     cudaFree(B->d_split);
+    cudaFree(B->d_halves);
     cudaFree(B->d_part);
     cudaFree(B->d_counters);
     delete B;
 }
 
-// Makespan of the atomic queue as list scheduling: items in queue order, each
-// taken by the first of W equal workers to become free (LPT when the costs
-// are sorted in decreasing order).
-double lpt_makespan(const std::vector<double> &cost, int W) {
-    std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
-    for (int w = 0; w < W; ++w) free_at.push(0.0);
+// Makespan of the work queue: S SMs with up to K CTAs each take the pieces in
+// order, one whenever a CTA is free; a CTA runs at rate[k] when k are active on
+// its SM (the CTAs share the FMA pipes, a lone one cannot fill them).
+double queue_makespan(const std::vector<double> &cost, int S, int K, const double *rate) {
+    struct Sm {
+        double t = 0.0;
+        int n = 0;
+        double left[3];
+    };
+    std::vector<Sm> sm(S);
+    size_t q = 0;
+    for (int k = 0; k < K; ++k)
+        for (int s = 0; s < S && q < cost.size(); ++s) sm[s].left[sm[s].n++] = cost[q++];
+    using Event = std::pair<double, int>;  // the SM's next completion
+    std::priority_queue<Event, std::vector<Event>, std::greater<Event>> heap;
+    auto push = [&](int s) {
+        const Sm &m = sm[s];
+        if (m.n) heap.push({m.t + *std::min_element(m.left, m.left + m.n) / rate[m.n], s});
+    };
+    for (int s = 0; s < S; ++s) push(s);
     double end = 0.0;
-    for (double x : cost) {
-        const double t = free_at.top() + x;
-        free_at.pop();
-        free_at.push(t);
-        end = std::max(end, t);
+    while (!heap.empty()) {
+        const Event e = heap.top();
+        heap.pop();
+        Sm &m = sm[e.second];
+        const double done = (e.first - m.t) * rate[m.n];
+        m.t = end = e.first;
+        double *least = std::min_element(m.left, m.left + m.n);
+        *least = m.left[m.n - 1];
+        --m.n;
+        for (int i = 0; i < m.n; ++i) m.left[i] -= done;
+        if (q < cost.size()) m.left[m.n++] = cost[q++];
+        push(e.second);
     }
     return end;
 }
 
-// Split plan of the convolution's queue for variant 4 (3 CTAs of 4 warps per
-// SM): the costliest items are cut into two block ranges. Item cost in block
-// times of one CTA: ceil(blocks / 4) plus one for the item's first copies and
-// its reduction. Splits go level by level (all unsplit pieces of the current
-// largest cost at once, at least 8 blocks a half) down to the smallest
-// splittable cost; the level with the shortest simulated makespan is kept
-// (single levels often leave it unchanged, so there is no early stop).
-// out: the items in queue order; code[i] = -1 or 2 sid + half.
+// Split plan of the convolution's queue for variants 4 and 5 (CTAs of 4 warps, 3
+// per SM, 2 where the wide kinds' shared memory allows no more): every item is cut
+// into equal block ranges of at most u blocks a warp, with the u (or no cut) that
+// gives the shortest simulated queue. In units of a pair (12 ns with 12 warps on
+// the SM) a block costs its entries + 40, an item 300 (first copies, reduction), a
+// part 450 (its sums go through L2), and a CTA runs 1.2 and 1.5 times as fast with
+// one and no neighbour: fitted to measured launches of 12 values of u on 20 batch
+// shapes, where this choice loses 1 % to the best u on average. N = 16: 32 cells
+// 50.9 -> 35.4 us (u = 8), 56 cells 70.8 -> 52.7 (10), 96 cells 96.2 -> 68.0 (12), 128
+// cells 99.4 -> 86.4 (20), from 256 cells on every cut is slower; N = 12, 37 cells
+// 25.1 -> 22.3 (6). Small predicted gains are not taken (the wide kinds' first, where
+// 5 % predicted measured as 4 % lost).
+// out: the items in queue order; code[i]: ConvParams::split; *slots: parts' slots.
 void plan_splits(const bte_ctx *c, const std::vector<ConvItem> &items, std::vector<ConvItem> &out,
-                 std::vector<int> &code) {
-    struct Piece {
-        ConvItem it;
-        int code;
+                 std::vector<int> &code, int *slots) {
+    out.clear();
+    code.clear();
+    *slots = 0;
+    unsigned kinds = 0;
+    for (const ConvItem &it : items) kinds |= 1u << it.kind;
+    const bool wide = (kinds & ~7u) != 0;
+    const int K = wide ? 2 : 3, W = K * c->num_sms;
+    static const double rate3[4] = {0.0, 1.5, 1.2, 1.0}, rate2[3] = {0.0, 1.25, 1.0};
+    if (items.empty() || items.size() > (size_t)16 * W) return;  // long queues have no tail to cut
+    // N < 16: halves at most (37 cells N = 12, one collide: 45.9 us in halves, 47.0
+    // in three parts, for which the model predicts less)
+    auto parts_of = [&](const ConvItem &it, int u) {
+        const int per_warp = ((int)it.nblocks + 3) / 4, most = c->tables[it.table]->N < 16 ? 2 : (int)kMaxParts;
+        return std::min((per_warp + u - 1) / u, most);
     };
-    const int W = 3 * c->num_sms;
-    auto cost_of = [](const ConvItem &it) { return (double)((it.nblocks + 3) / 4) + 1.0; };
-    auto order = [&](std::vector<Piece> &v) {
-        std::stable_sort(v.begin(), v.end(),
-                         [&](const Piece &a, const Piece &b) { return cost_of(a.it) > cost_of(b.it); });
+    auto first_block = [](const ConvItem &it, int parts, int p) { return (uint32_t)((uint64_t)it.nblocks * p / parts); };
+    struct Piece {
+        double cost;
+        int item, part, parts;
+    };
+    auto pieces = [&](int u) {
+        std::vector<Piece> v;
+        for (int i = 0; i < (int)items.size(); ++i) {
+            const ConvItem &it = items[i];
+            const Table *t = c->tables[it.table];
+            const double block = t->cpad[it.kind - t->kind0] + 40.0;
+            const int P = parts_of(it, u);
+            for (int p = 0; p < P; ++p) {
+                const uint32_t nb = first_block(it, P, p + 1) - first_block(it, P, p);
+                v.push_back({(double)((nb + 3) / 4) * block + (P > 1 ? 450.0 : 300.0), i, p, P});
+            }
+        }
+        std::stable_sort(v.begin(), v.end(), [](const Piece &a, const Piece &b) { return a.cost > b.cost; });
+        return v;
     };
     auto makespan = [&](const std::vector<Piece> &v) {
         std::vector<double> cs(v.size());
-        for (size_t i = 0; i < v.size(); ++i) cs[i] = cost_of(v[i].it);
-        return lpt_makespan(cs, W);
+        for (size_t i = 0; i < v.size(); ++i) cs[i] = v[i].cost;
+        return queue_makespan(cs, c->num_sms, K, wide ? rate2 : rate3);
     };
-    std::vector<Piece> cur(items.size());
-    for (size_t i = 0; i < items.size(); ++i) cur[i] = Piece{items[i], -1};
-    out.clear();
-    code.clear();
-    if (items.empty() || items.size() > 65536) {  // large batches have no tail to cut
-        return;
+    const int whole = 1 << 20;
+    int best_u = whole;
+    double best = makespan(pieces(whole)) * (wide ? 0.9 : 0.98);
+    for (int u : {32, 24, 20, 16, 12, 10, 8, 6, 5, 4}) {
+        const std::vector<Piece> v = pieces(u);
+        if (v.size() > (size_t)16 * W) break;
+        const double m = makespan(v);
+        if (m < best) {
+            best = m;
+            best_u = u;
+        }
     }
-    double best = makespan(cur);
-    std::vector<Piece> best_state;  // empty: no split
-    int nsplit = 0, best_nsplit = 0;
-    for (int level = 0; level < 64; ++level) {
-        // the largest cost among unsplit pieces that can be cut
-        double top = -1.0;
-        for (const Piece &p : cur)
-            if (p.code < 0 && p.it.nblocks >= 16) top = std::max(top, cost_of(p.it));
-        if (top < 0.0) break;
-        std::vector<Piece> trial;
-        trial.reserve(cur.size() * 2);
-        int ns = nsplit;
-        for (const Piece &p : cur) {
-            if (p.code < 0 && p.it.nblocks >= 16 && cost_of(p.it) == top) {
-                const Table *t = c->tables[p.it.table];
-                const int tile = p.it.kind - t->kind0;
-                const uint32_t b0 = p.it.nblocks / 2;
-                Piece a = p, b = p;
-                a.it.nblocks = b0;
-                a.code = 2 * ns;
-                b.it.desc_off = p.it.desc_off + b0;
-                b.it.wofs = p.it.wofs + (uint64_t)b0 * t->cpad[tile];
-                b.it.nblocks = p.it.nblocks - b0;
-                b.code = 2 * ns + 1;
-                ++ns;
-                trial.push_back(a);
-                trial.push_back(b);
-            } else {
-                trial.push_back(p);
+    if (best_u == whole) return;
+    const std::vector<Piece> v = pieces(best_u);
+    std::vector<int> first(items.size(), -1);
+    for (const Piece &p : v) {
+        const ConvItem &it = items[p.item];
+        ConvItem o = it;
+        if (p.parts > 1) {
+            const Table *t = c->tables[it.table];
+            const uint32_t b0 = first_block(it, p.parts, p.part);
+            o.nblocks = first_block(it, p.parts, p.part + 1) - b0;
+            o.desc_off = it.desc_off + b0;
+            o.wofs = it.wofs + (uint64_t)b0 * t->cpad[it.kind - t->kind0];
+            if (first[p.item] < 0) {
+                first[p.item] = *slots;
+                *slots += p.parts;
             }
         }
-        order(trial);
-        const double m = makespan(trial);
-        cur.swap(trial);
-        nsplit = ns;
-        if (m < best * 0.999) {
-            best = m;
-            best_state = cur;
-            best_nsplit = nsplit;
-        }
+        out.push_back(o);
+        code.push_back(p.parts > 1 ? first[p.item] | p.part << 20 | p.parts << 25 : -1);
     }
-    if (best_nsplit == 0) return;
-    out.resize(best_state.size());
-    code.resize(best_state.size());
-    for (size_t i = 0; i < best_state.size(); ++i) {
-        out[i] = best_state[i].it;
-        code[i] = best_state[i].code;
+    if (*slots > kMaxSplitSlots || *slots == 0) {  // cannot be coded, or nothing to cut
+        out.clear();
+        code.clear();
+        *slots = 0;
     }
 }
 
@@ -448,17 +483,24 @@ bte_status get_batch(bte_ctx *c, const bte_instance *inst, int64_t ninst, Batch 
     B->nitems = (int)sorted.size();
     std::vector<ConvItem> split_items;
     std::vector<int> split_code;
-    plan_splits(c, sorted, split_items, split_code);
+    plan_splits(c, sorted, split_items, split_code, &B->nsplit);
     B->nitems_split = (int)split_items.size();
-    B->nsplit = 0;
-    for (int v : split_code) B->nsplit = std::max(B->nsplit, v / 2 + 1);
+    std::vector<int> halves;
+    for (int code : split_code) {
+        if (code >= 0 && (code >> 25) > 2) {
+            halves.clear();
+            break;
+        }
+        halves.push_back(code < 0 ? -1 : (code & (kMaxSplitSlots - 1)) + ((code >> 20) & 31));
+    }
     cudaError_t e = cudaMalloc(&B->d_slot_off, sizeof(int64_t) * slot_off.size());
     if (e == cudaSuccess) e = cudaMalloc(&B->d_slot_out, sizeof(int64_t) * slot_out.size());
     if (e == cudaSuccess) e = cudaMalloc(&B->d_items, sizeof(ConvItem) * std::max<size_t>(sorted.size(), 1));
     if (e == cudaSuccess && B->nsplit > 0) {
         e = cudaMalloc(&B->d_items_split, sizeof(ConvItem) * split_items.size());
         if (e == cudaSuccess) e = cudaMalloc(&B->d_split, sizeof(int) * split_code.size());
-        if (e == cudaSuccess) e = cudaMalloc(&B->d_part, sizeof(float) * kSplitFloats * 2 * (size_t)B->nsplit);
+        if (e == cudaSuccess && !halves.empty()) e = cudaMalloc(&B->d_halves, sizeof(int) * halves.size());
+        if (e == cudaSuccess) e = cudaMalloc(&B->d_part, sizeof(float) * kSplitFloats * (size_t)B->nsplit);
     }
     if (e == cudaSuccess) e = cudaMalloc(&B->d_counters, sizeof(unsigned) * (1 + (size_t)B->nsplit));
     if (e != cudaSuccess) {
@@ -475,6 +517,8 @@ bte_status get_batch(bte_ctx *c, const bte_instance *inst, int64_t ninst, Batch 
                        cudaMemcpyHostToDevice);
         if (e == cudaSuccess)
             e = cudaMemcpy(B->d_split, split_code.data(), sizeof(int) * split_code.size(), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess && !halves.empty())
+            e = cudaMemcpy(B->d_halves, halves.data(), sizeof(int) * halves.size(), cudaMemcpyHostToDevice);
     }
     if (e != cudaSuccess) {
         free_batch(B);
@@ -513,6 +557,11 @@ ProjArgs proj_args(const Table *t) {
     return pa;
 }
 
+// Whether the batch's plan needs the convolution kernel for more than two parts.
+bool parts_kernel(const Batch *B, const ConvCfg &g) {
+    return g.impl == 4 && g.csplit && B->nsplit > 0 && !B->d_halves;
+}
+
 // Allocate everything a collide/step on this batch needs (never inside capture).
 bte_status prepare(bte_ctx *c, Batch *B, int mode, bool step, bool transport) {
     bte_status s;
@@ -548,7 +597,7 @@ bte_status prepare(bte_ctx *c, Batch *B, int mode, bool step, bool transport) {
                 if (r != BTE_OK) return (bte_status)r;
             }
         }
-        cudaError_t e = conv32_configure(B->kinds_mask, c->num_sms, g.warps, g.stages, g.impl, &L);
+        cudaError_t e = conv32_configure(B->kinds_mask, c->num_sms, g.warps, g.stages, g.impl, &L, parts_kernel(B, g));
         if (e != cudaSuccess) return cuda_fail(c, e, "convolution kernel configuration");
     }
     return BTE_OK;
@@ -634,15 +683,17 @@ bte_status enqueue_collide(bte_ctx *c, Batch *B, const double *f, double *Q, int
         count_launches(c, (int)B->segs.size());
     } else {
         ConvLaunch L;
-        cudaError_t e = conv32_configure(B->kinds_mask, c->num_sms, cfg.warps, cfg.stages, cfg.impl, &L);
+        const bool split = cfg.impl >= 4 && cfg.csplit && B->nsplit > 0;
+        cudaError_t e = conv32_configure(B->kinds_mask, c->num_sms, cfg.warps, cfg.stages, cfg.impl, &L,
+                                         parts_kernel(B, cfg));
         if (e != cudaSuccess) return cuda_fail(c, e, "convolution kernel configuration");
         ConvParams p{};
-        const bool split = cfg.impl >= 4 && cfg.csplit && B->nsplit > 0;
         p.items = split ? B->d_items_split : B->d_items;
         p.nitems = split ? B->nitems_split : B->nitems;
         p.counter = B->d_counters;
         if (split) {
             p.split = B->d_split;
+            p.halves = B->d_halves;
             p.part = B->d_part;
             p.split_cnt = B->d_counters + 1;
         }

@@ -33,13 +33,13 @@ std::recursive_mutex g_conv_cfg_mu;  // guards the caches below (contexts on sev
 }  // namespace
 
 cudaError_t conv32_configure(unsigned kinds_mask, int num_sms, int warps_per_cta, int stages, int impl,
-                             ConvLaunch *out) {
+                             ConvLaunch *out, bool parts) {
     std::lock_guard<std::recursive_mutex> lock(g_conv_cfg_mu);
     // keyed by device too: the shared-memory attribute is set per device
-    static std::map<std::tuple<int, unsigned, int, int, int, int>, ConvLaunch> cache;
+    static std::map<std::tuple<int, unsigned, int, int, int, int, bool>, ConvLaunch> cache;
     int dev = 0;
     cudaGetDevice(&dev);
-    auto key = std::make_tuple(dev, kinds_mask, num_sms, warps_per_cta, stages, impl);
+    auto key = std::make_tuple(dev, kinds_mask, num_sms, warps_per_cta, stages, impl, parts);
     auto itc = cache.find(key);
     if (itc != cache.end()) {
         *out = itc->second;
@@ -51,9 +51,9 @@ cudaError_t conv32_configure(unsigned kinds_mask, int num_sms, int warps_per_cta
         // stage of 8 KB rows would cost a resident CTA, which the block-level
         // latency hiding does not buy back.
         ConvLaunch a{}, b{};
-        cudaError_t e1 = conv32_configure(kinds_mask, num_sms, warps_per_cta, 1, impl, &a);
+        cudaError_t e1 = conv32_configure(kinds_mask, num_sms, warps_per_cta, 1, impl, &a, parts);
         if (e1 != cudaSuccess) return e1;
-        e1 = conv32_configure(kinds_mask, num_sms, warps_per_cta, 2, impl, &b);
+        e1 = conv32_configure(kinds_mask, num_sms, warps_per_cta, 2, impl, &b, parts);
         if (e1 != cudaSuccess) return e1;
         *out = b.grid >= a.grid ? b : a;
         cache[key] = *out;
@@ -83,8 +83,9 @@ cudaError_t conv32_configure(unsigned kinds_mask, int num_sms, int warps_per_cta
     } else {
         const bool packed = impl >= 2;
 #define BTE_PICK(M)                                                                             \
-    L.fn = impl == 5   ? conv32_sums_kernel<M, true>                                           \
-           : impl == 4 ? conv32_sums_kernel<M>                                                 \
+    L.fn = impl == 5   ? conv32_sums_kernel<M, true, true>                                     \
+           : impl == 4 ? (parts ? conv32_sums_kernel<M, false, true>                           \
+                                : conv32_sums_kernel<M, false, (M & ~7u) != 0>)                \
            : impl == 3 ? conv32_coop_kernel<M, true, 2>                                        \
                        : (packed ? conv32_coop_kernel<M, true> : conv32_coop_kernel<M, false>)
 #define BTE_PICK4(M) L.fn = conv32_sums_wide(M, impl == 5)

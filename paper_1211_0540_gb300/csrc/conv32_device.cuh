@@ -674,7 +674,7 @@ __device__ bool coop_item_sm(WarpRing &r, const ConvItem &it, const ConvParams &
     return ok;
 }
 
-// Half `sp & 1` of split item sp >> 1: the warps' sums reduced in the fixed
+// Half `sp & 1` of split item sp >> 1 (ConvParams::halves): the warps' sums reduced in the fixed
 // warp order into part[], then the CTA that finishes second (an atomic count,
 // no waiting) adds half 0 and half 1 in that order and stores Q.
 template <class K>
@@ -714,6 +714,58 @@ __device__ __forceinline__ void coop_reduce_split(const ConvItem &it, const Conv
         lr += __ldcg(b + kLanes);
         two_sum(si, li, __ldcg(b + 2 * kLanes));
         li += __ldcg(b + 3 * kLanes);
+        Q[t * kLanes] = make_float2(sr + lr, si + li);
+    }
+}
+
+// The item's sums reduced over the warps in a fixed order: to Qhat, or, for a part
+// of a split item (code sp, ConvParams::split), to part[]; the CTA whose part
+// finishes last (an atomic count, no waiting) then adds the parts in order.
+template <class K>
+__device__ __forceinline__ void coop_reduce_parts(const ConvItem &it, const ConvParams &p, int lane, int warp,
+                                                  int nwarps, const char *ring0, int warp_smem, int sums_off,
+                                                  int sp, int *s_last) {
+    constexpr int T = K::T;
+    float2 *Q = p.Qh + it.fofs + ((size_t)(it.k1 * K::N + it.k2) * K::N + K::K0) * kLanes + lane;
+    const int first = sp & (kMaxSplitSlots - 1);
+    float *o0 = p.part + (size_t)(first + ((sp >> 20) & 31)) * kSplitFloats + lane;
+    for (int t = warp; t < T; t += nwarps) {
+        float sr = 0.f, lr = 0.f, si = 0.f, li = 0.f;
+        for (int w = 0; w < nwarps; ++w) {
+            const float *red = reinterpret_cast<const float *>(ring0 + (size_t)w * warp_smem + sums_off);
+            two_sum(sr, lr, red[(2 * t) * kLanes + lane]);
+            lr += red[(2 * T + 2 * t) * kLanes + lane];
+            two_sum(si, li, red[(2 * t + 1) * kLanes + lane]);
+            li += red[(2 * T + 2 * t + 1) * kLanes + lane];
+        }
+        if (sp < 0) {
+            Q[t * kLanes] = make_float2(sr + lr, si + li);
+        } else {
+            float *o = o0 + (size_t)t * 4 * kLanes;
+            o[0] = sr;
+            o[kLanes] = lr;
+            o[2 * kLanes] = si;
+            o[3 * kLanes] = li;
+        }
+    }
+    if (sp < 0) return;
+    const int parts = sp >> 25;
+    __threadfence();  // this part's sums before the count
+    __syncthreads();
+    if (threadIdx.x == 0) *s_last = atomicAdd(p.split_cnt + first, 1u) == (unsigned)(parts - 1);
+    __syncthreads();
+    if (!*s_last) return;
+    __threadfence();  // the other parts' sums after the count
+    for (int t = warp; t < T; t += nwarps) {
+        const float *a = p.part + (size_t)first * kSplitFloats + (size_t)t * 4 * kLanes + lane;
+        float sr = 0.f, lr = 0.f, si = 0.f, li = 0.f;
+#pragma unroll 1
+        for (int q = 0; q < parts; ++q, a += kSplitFloats) {
+            two_sum(sr, lr, __ldcg(a));
+            lr += __ldcg(a + kLanes);
+            two_sum(si, li, __ldcg(a + 2 * kLanes));
+            li += __ldcg(a + 3 * kLanes);
+        }
         Q[t * kLanes] = make_float2(sr + lr, si + li);
     }
 }
@@ -763,7 +815,7 @@ __device__ __forceinline__ void gen_first_any(const WarpRing &r, const ConvItem 
 // item is taken from the queue (into *s_next) and each warp issues the copies
 // of its first block into its now idle ring before the CTA reduces this item's
 // sums, which live outside the rings.
-template <class K, unsigned MASK, bool OTF>
+template <class K, unsigned MASK, bool OTF, bool PARTS>
 __device__ __forceinline__ bool coop_run_sm(WarpRing &r, const ConvItem &it, const ConvParams &p, int lane,
                                             int warp, int nwarps, char *ring0, int *abort_flag, float *sums,
                                             int sums_off, int sp, int *s_last, bool pre, int *s_next, int nitems) {
@@ -786,7 +838,8 @@ __device__ __forceinline__ bool coop_run_sm(WarpRing &r, const ConvItem &it, con
         __syncwarp();
     }
     if (!*abort_flag) {
-        if (sp < 0) coop_reduce<K>(it, p, lane, warp, nwarps, ring0, p.warp_smem, sums_off);
+        if (PARTS) coop_reduce_parts<K>(it, p, lane, warp, nwarps, ring0, p.warp_smem, sums_off, sp, s_last);
+        else if (sp < 0) coop_reduce<K>(it, p, lane, warp, nwarps, ring0, p.warp_smem, sums_off);
         else coop_reduce_split<K>(it, p, lane, warp, nwarps, ring0, p.warp_smem, sums_off, sp, s_last);
     }
     __syncthreads();
@@ -799,7 +852,9 @@ __device__ __forceinline__ bool coop_run_sm(WarpRing &r, const ConvItem &it, con
 // 24, 64 cells: 437 against 398 us for the 255-register variant 3).
 constexpr int sums_min_ctas(unsigned mask) { return mask & ~7u ? 2 : 3; }
 
-template <unsigned MASK, bool OTF = false>
+// PARTS: items may be split into more than two parts (ConvParams::split); false:
+// into halves at most (ConvParams::halves).
+template <unsigned MASK, bool OTF, bool PARTS>
 __global__ void __launch_bounds__(128, sums_min_ctas(MASK)) conv32_sums_kernel(ConvParams p) {
     extern __shared__ __align__(128) char smem[];
     __shared__ int s_item, s_abort, s_last, s_nitems;
@@ -829,19 +884,20 @@ __global__ void __launch_bounds__(128, sums_min_ctas(MASK)) conv32_sums_kernel(C
         const int idx = s_item;
         if (idx >= nitems || s_abort) break;
         const ConvItem it = p.items[idx];
-        const int sp = p.split ? p.split[idx] : -1;
+        const int *split = PARTS ? p.split : p.halves;
+        const int sp = split ? split[idx] : -1;
         bool ok = true, ran = true;
         switch (it.kind) {
-            case 0: if (MASK & 1u) ok = coop_run_sm<K8, MASK, OTF>(r, it, p, lane, warp, nwarps, smem, &s_abort, sums, ring, sp, &s_last, pre, &s_item, nitems); else ran = false; break;
-            case 1: if (MASK & 2u) ok = coop_run_sm<K12, MASK, OTF>(r, it, p, lane, warp, nwarps, smem, &s_abort, sums, ring, sp, &s_last, pre, &s_item, nitems); else ran = false; break;
-            case 2: if (MASK & 4u) ok = coop_run_sm<K16, MASK, OTF>(r, it, p, lane, warp, nwarps, smem, &s_abort, sums, ring, sp, &s_last, pre, &s_item, nitems); else ran = false; break;
-            case 3: if (MASK & 8u) ok = coop_run_sm<K24a, MASK, OTF>(r, it, p, lane, warp, nwarps, smem, &s_abort, sums, ring, sp, &s_last, pre, &s_item, nitems); else ran = false; break;
-            case 4: if (MASK & 16u) ok = coop_run_sm<K24b, MASK, OTF>(r, it, p, lane, warp, nwarps, smem, &s_abort, sums, ring, sp, &s_last, pre, &s_item, nitems); else ran = false; break;
-            case 5: if (MASK & 32u) ok = coop_run_sm<K32a, MASK, OTF>(r, it, p, lane, warp, nwarps, smem, &s_abort, sums, ring, sp, &s_last, pre, &s_item, nitems); else ran = false; break;
-            case 6: if (MASK & 64u) ok = coop_run_sm<K32b, MASK, OTF>(r, it, p, lane, warp, nwarps, smem, &s_abort, sums, ring, sp, &s_last, pre, &s_item, nitems); else ran = false; break;
-            case 7: if (MASK & 128u) ok = coop_run_sm<K48a, MASK, OTF>(r, it, p, lane, warp, nwarps, smem, &s_abort, sums, ring, sp, &s_last, pre, &s_item, nitems); else ran = false; break;
-            case 8: if (MASK & 256u) ok = coop_run_sm<K48b, MASK, OTF>(r, it, p, lane, warp, nwarps, smem, &s_abort, sums, ring, sp, &s_last, pre, &s_item, nitems); else ran = false; break;
-            case 9: if (MASK & 512u) ok = coop_run_sm<K48c, MASK, OTF>(r, it, p, lane, warp, nwarps, smem, &s_abort, sums, ring, sp, &s_last, pre, &s_item, nitems); else ran = false; break;
+            case 0: if (MASK & 1u) ok = coop_run_sm<K8, MASK, OTF, PARTS>(r, it, p, lane, warp, nwarps, smem, &s_abort, sums, ring, sp, &s_last, pre, &s_item, nitems); else ran = false; break;
+            case 1: if (MASK & 2u) ok = coop_run_sm<K12, MASK, OTF, PARTS>(r, it, p, lane, warp, nwarps, smem, &s_abort, sums, ring, sp, &s_last, pre, &s_item, nitems); else ran = false; break;
+            case 2: if (MASK & 4u) ok = coop_run_sm<K16, MASK, OTF, PARTS>(r, it, p, lane, warp, nwarps, smem, &s_abort, sums, ring, sp, &s_last, pre, &s_item, nitems); else ran = false; break;
+            case 3: if (MASK & 8u) ok = coop_run_sm<K24a, MASK, OTF, PARTS>(r, it, p, lane, warp, nwarps, smem, &s_abort, sums, ring, sp, &s_last, pre, &s_item, nitems); else ran = false; break;
+            case 4: if (MASK & 16u) ok = coop_run_sm<K24b, MASK, OTF, PARTS>(r, it, p, lane, warp, nwarps, smem, &s_abort, sums, ring, sp, &s_last, pre, &s_item, nitems); else ran = false; break;
+            case 5: if (MASK & 32u) ok = coop_run_sm<K32a, MASK, OTF, PARTS>(r, it, p, lane, warp, nwarps, smem, &s_abort, sums, ring, sp, &s_last, pre, &s_item, nitems); else ran = false; break;
+            case 6: if (MASK & 64u) ok = coop_run_sm<K32b, MASK, OTF, PARTS>(r, it, p, lane, warp, nwarps, smem, &s_abort, sums, ring, sp, &s_last, pre, &s_item, nitems); else ran = false; break;
+            case 7: if (MASK & 128u) ok = coop_run_sm<K48a, MASK, OTF, PARTS>(r, it, p, lane, warp, nwarps, smem, &s_abort, sums, ring, sp, &s_last, pre, &s_item, nitems); else ran = false; break;
+            case 8: if (MASK & 256u) ok = coop_run_sm<K48b, MASK, OTF, PARTS>(r, it, p, lane, warp, nwarps, smem, &s_abort, sums, ring, sp, &s_last, pre, &s_item, nitems); else ran = false; break;
+            case 9: if (MASK & 512u) ok = coop_run_sm<K48c, MASK, OTF, PARTS>(r, it, p, lane, warp, nwarps, smem, &s_abort, sums, ring, sp, &s_last, pre, &s_item, nitems); else ran = false; break;
             default: ran = false; break;
         }
         if (!ok) break;

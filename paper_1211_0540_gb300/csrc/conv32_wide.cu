@@ -9,8 +9,8 @@
 namespace bte {
 
 void (*conv32_sums_wide(unsigned mask, bool otf))(ConvParams) {
-    if (mask == (128u | 256u | 512u)) return otf ? conv32_sums_kernel<896u, true> : conv32_sums_kernel<896u, false>;
-    return otf ? conv32_sums_kernel<1023u, true> : conv32_sums_kernel<1023u, false>;
+    if (mask == (128u | 256u | 512u)) return otf ? conv32_sums_kernel<896u, true, true> : conv32_sums_kernel<896u, false, true>;
+    return otf ? conv32_sums_kernel<1023u, true, true> : conv32_sums_kernel<1023u, false, true>;
 }
 
 }  // namespace bte

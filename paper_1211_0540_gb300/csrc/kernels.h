@@ -53,12 +53,15 @@ struct ConvParams {
     int merge;      // blocks per TwoSum merge
     int warp_smem;  // bytes of ring per warp
     int stall;      // testing the timeout path: each warp never issues its first block
-    // Items split into two block ranges (conv_impl 4 only; null: no splits).
-    // split[i] = -1, or 2 sid + half: the two halves write their reduced sums to
-    // part[(2 sid + half) * kSplitFloats ...]; the CTA that finishes second
-    // (split_cnt[sid], zeroed before the launch) adds half 0 and half 1 in that
-    // order and writes Q.
+    // Items split into up to kMaxParts block ranges (conv_impl 4, 5; null: no
+    // splits). split[i] = -1, or the parts' first slot | part << 20 | parts << 25:
+    // each part writes its reduced sums to part[(first + part) * kSplitFloats ...];
+    // the CTA that finishes last (split_cnt[first], zeroed before the launch) adds
+    // the parts in order and writes Q.
     const int *split;
+    // the same where no item has more than two parts, for the kernels that take
+    // halves only: -1, or 2 sid + half (slots 2 sid, 2 sid + 1; split_cnt[sid])
+    const int *halves;
     float *part;
     unsigned *split_cnt;
     // Weights built on the fly (conv_impl 5): per table the FP32 radial tables
@@ -71,7 +74,8 @@ struct ConvParams {
     int nq[kMaxTables];
     int estride[kMaxTables];
 };
-constexpr int kSplitFloats = 16 * 4 * 32;  // per half: T <= 16 outputs x (hi, lo) x (re, im) x 32 lanes
+constexpr int kSplitFloats = 16 * 4 * 32;  // per part: T <= 16 outputs x (hi, lo) x (re, im) x 32 lanes
+constexpr int kMaxParts = 16, kMaxSplitSlots = 1 << 20;
 int conv_stage_bytes(int kind);
 struct ConvLaunch {
     void (*fn)(ConvParams);
@@ -83,8 +87,11 @@ struct ConvLaunch {
 // impl: 0 = one warp per item, 1 = CTA-cooperative items, 2 = cooperative + packed f32x2,
 // 3 = as 2 at 2 CTAs per SM, 4 = as 2 with the compensated sums in shared memory,
 // 5 = as 4 with every block's weights built on the fly from the radial tables.
+// parts: variant 4 on a list whose items are split into more than two parts (the
+// kinds of N <= 16 have a kernel for halves too; the register-capped pair loop of
+// N = 16 runs 1.7 % faster beside the smaller reduction).
 cudaError_t conv32_configure(unsigned kinds_mask, int num_sms, int warps_per_cta, int stages, int impl,
-                             ConvLaunch *out);
+                             ConvLaunch *out, bool parts = false);
 cudaError_t conv32_launch(const ConvLaunch &L, const ConvParams &p, cudaStream_t st);
 
 // FP32 convolution of one segment with pairs in lanes, for few cells; fhat and
