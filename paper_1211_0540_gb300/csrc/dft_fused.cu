@@ -47,9 +47,13 @@ struct FusedShape {
     static constexpr int P = N + 1;      // padded pencil stride
     // forward: A (own pencils, padded) + B (own slab, read by the cluster)
     static constexpr size_t smem_fwd = sizeof(float2) * (NP * P + JR * NN);
-    // inverse: A (own slab, read by the cluster) + B (own pencils, padded) + R (FP32 Qt, padded) + base
-    static constexpr size_t smem_inv = sizeof(float2) * (JR * NN + NP * P) + sizeof(float) * NP * P +
-                                       sizeof(double) * NP;
+    // inverse: A (own slab, read by the cluster) + B (own pencils, padded) + base + R (FP32 Qt, padded).
+    // Without the time update R takes A's place: at N = 16 with one CTA per cell 69 KB, three CTAs per SM
+    // instead of two (1024 cells 56.8 -> 53.8 us). With it the registers allow two anyway, and the update
+    // with the next forward transform is faster with R apart (128 cells 38.2 against 40.5 us).
+    static constexpr size_t smem_inv_proj = sizeof(float2) * (JR * NN + NP * P) + sizeof(double) * NP;
+    static constexpr size_t smem_inv = smem_inv_proj + sizeof(float) * NP * P;
+    static_assert(sizeof(float) * NP * P <= sizeof(float2) * JR * NN, "R fits in A");
     static_assert(N % C == 0, "slabs must split evenly");
 };
 
@@ -271,8 +275,9 @@ dft_fwd_pencils_kernel(const double *__restrict__ f, const int64_t *__restrict__
 // its own slab, narrowed to FP32, is the input of the next stage's forward
 // transform, which the cluster then runs as dft_fwd_fused_kernel would
 // (the same passes on the same values: fhat of f* into Gout, scaled by
-// fscale), in the inverse's shared memory.
-template <int N, int C_, bool FWD = false>
+// fscale), in the inverse's shared memory. UPD: compiled for modes 2 and 3 (the
+// update's operands in registers); without it for modes 0 and 1.
+template <int N, int C_, bool FWD = false, bool UPD = true>
 __global__ void __cluster_dims__(C_, 1, 1) __launch_bounds__(FusedShape<N, C_>::NT)
 dft_inv_fused_kernel(const float2 *__restrict__ G, const int64_t *__restrict__ slot_off, DftSeg s,
                      const float2 *__restrict__ root, float scale, double *__restrict__ q, ProjArgs pa,
@@ -285,8 +290,9 @@ dft_inv_fused_kernel(const float2 *__restrict__ G, const int64_t *__restrict__ s
     extern __shared__ __align__(16) char smem_raw[];
     float2 *A = reinterpret_cast<float2 *>(smem_raw);  // [kl][j1][k3], read by the cluster
     float2 *B = A + JR * NN;                            // [jl][j2] rows of P, index k3
-    float *R = reinterpret_cast<float *>(B + NP * P);   // Qt, [jl][j2] rows of P, index j3
-    double *base = reinterpret_cast<double *>(R + NP * P);
+    double *base = reinterpret_cast<double *>(B + NP * P);
+    // Qt, [jl][j2] rows of P, index j3 (in A: its last readers are a barrier away)
+    float *R = UPD ? reinterpret_cast<float *>(base + NP) : reinterpret_cast<float *>(A);
     __shared__ float red[32][10];
     __shared__ float part[10];
     __shared__ double sg[N], lam[5];
@@ -297,11 +303,12 @@ dft_inv_fused_kernel(const float2 *__restrict__ G, const int64_t *__restrict__ s
     // memory latency overlaps the three passes
     constexpr int MS = M / C, IT = (MS + S::NT - 1) / S::NT;
     constexpr bool PF = IT <= 16;  // prefetch while the operands fit in registers
+    constexpr bool LD = PF && UPD;
     const double *xo = x ? x + off + (int64_t)r * MS : nullptr;
     double *yo = y ? y + off + (int64_t)r * MS : nullptr;
     const double *qpo = qp ? qp + off + (int64_t)r * MS : nullptr;
-    double u[PF ? IT : 1], w[PF ? IT : 1];
-    if (!PF) {
+    double u[LD ? IT : 1], w[LD ? IT : 1];
+    if constexpr (!LD) {
     } else if (mode == 2) {
 #pragma unroll
         for (int i = 0; i < IT; ++i) {
@@ -455,10 +462,9 @@ dft_inv_fused_kernel(const float2 *__restrict__ G, const int64_t *__restrict__ s
                     const double fs = fma(a, v, u[i]);
                     bad |= !fpc::finite64(fs);
                     R[p * P + j3] = fpc::narrow(fs);  // each value is read and rewritten by this thread only
-                } else if (mode == 2) {
-                    yo[e] = fma(a, v, u[i]);
-                } else if (mode == 3) {
-                    yo[e] = fma(a, w[i] + v, u[i]);
+                } else if constexpr (UPD) {
+                    if (mode == 2) yo[e] = fma(a, v, u[i]);
+                    else if (mode == 3) yo[e] = fma(a, w[i] + v, u[i]);
                 }
             }
         }
@@ -472,10 +478,9 @@ dft_inv_fused_kernel(const float2 *__restrict__ G, const int64_t *__restrict__ s
                 const double fs = fma(a, v, xo[e]);
                 bad |= !fpc::finite64(fs);
                 R[p * P + j3] = fpc::narrow(fs);
-            } else if (mode == 2) {
-                yo[e] = fma(a, v, xo[e]);
-            } else if (mode == 3) {
-                yo[e] = fma(a, qpo[e] + v, yo[e]);
+            } else if constexpr (UPD) {
+                if (mode == 2) yo[e] = fma(a, v, xo[e]);
+                else if (mode == 3) yo[e] = fma(a, qpo[e] + v, yo[e]);
             }
         }
     }
@@ -548,8 +553,12 @@ void inv_launch(const float2 *G, const int64_t *slot_off, const DftSeg &s, const
                 double *q, const ProjArgs &pa, int mode, const double *x, double *y, const double *qp, double a,
                 cudaStream_t st) {
     using S = FusedShape<N, C>;
-    dft_inv_fused_kernel<N, C><<<grid_slots(s) * C, S::NT, S::smem_inv, st>>>(G, slot_off, s, root, (float)scale, q, pa,
-                                                                        mode, x, y, qp, a);
+    if (mode >= 2)
+        dft_inv_fused_kernel<N, C><<<grid_slots(s) * C, S::NT, S::smem_inv, st>>>(G, slot_off, s, root, (float)scale, q,
+                                                                                 pa, mode, x, y, qp, a);
+    else
+        dft_inv_fused_kernel<N, C, false, false><<<grid_slots(s) * C, S::NT, S::smem_inv_proj, st>>>(
+            G, slot_off, s, root, (float)scale, q, pa, mode, x, y, qp, a);
 }
 template <int N, int C>
 void inv_fwd_launch(const float2 *G, const int64_t *slot_off, const DftSeg &s, const float2 *root, double scale,
@@ -567,6 +576,8 @@ void prepare_one() {
         cudaFuncSetAttribute(dft_fwd_fused_kernel<N, C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)S::smem_fwd);
     cudaFuncSetAttribute(dft_inv_fused_kernel<N, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem_inv);
+    cudaFuncSetAttribute(dft_inv_fused_kernel<N, C, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)S::smem_inv_proj);
     cudaFuncSetAttribute(dft_inv_fused_kernel<N, C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)S::smem_inv);
 }
@@ -576,7 +587,16 @@ void prepare_n() {
     prepare_one<N, 2>();
     prepare_one<N, 4>();
 }
-int norm_split(int split) { return split == 1 || split == 2 ? split : 4; }
+// CTAs per cell: 1 or 2 as asked; 4 (the default) while the cells are few, one
+// once they alone give about 5 warps per SM, from where it is the faster one
+// (forward + inverse, 4 against 1 CTAs per cell: N = 16, 56 cells 27.4 / 28.6 us, 128
+// 31.5 / 29.2, 1024 129.6 / 110.4; N = 12, 128 cells 25.1 / 23.1, 512 47.7 / 35.3;
+// N = 8, 256 cells 19.8 / 20.1, 1024 46.1 / 26.2).
+constexpr int kOneCtaWarps = 5 * 152;
+int norm_split(int split, const DftSeg &s) {
+    if (split == 1 || split == 2) return split;
+    return (int64_t)grid_slots(s) * ((s.N * s.N + 31) / 32) >= kOneCtaWarps ? 1 : 4;
+}
 template <int N>
 void upload_roots(const float2 (&sym)[N]) {
     float2 h[N];
@@ -611,7 +631,7 @@ void fused_dft_prepare(int N) {
 }
 
 #define BTE_SPLIT_DISPATCH(FN, N, ...)                 \
-    switch (norm_split(split)) {                       \
+    switch (norm_split(split, s)) {                    \
         case 1: FN<N, 1>(__VA_ARGS__); break;          \
         case 2: FN<N, 2>(__VA_ARGS__); break;          \
         default: FN<N, 4>(__VA_ARGS__); break;         \
@@ -667,7 +687,7 @@ void launch_dft_inverse_forward_fused(const float2 *G, const int64_t *slot_off, 
         case 8:
         case 12:
         case 16:
-            switch (norm_split(split)) {
+            switch (norm_split(split, s)) {
                 case 1:
                     if (s.N == 8) inv_fwd_launch<8, 1>(G, slot_off, s, root, scale, q, pa, x, a, fscale, Gout, status, st);
                     else if (s.N == 12) inv_fwd_launch<12, 1>(G, slot_off, s, root, scale, q, pa, x, a, fscale, Gout, status, st);

@@ -126,7 +126,8 @@ void launch_dft_forward_pencils(const double *f, const int64_t *slot_off, const 
 __host__ __device__ __forceinline__ int64_t sector_index(int64_t e, int lane) {
     return ((e >> 2) << 7) + ((int64_t)lane << 2) + (e & 3);
 }
-// split: CTAs (a thread-block cluster) per cell, 1, 2 or 4 (other values: 4);
+// split: CTAs (a thread-block cluster) per cell, 1, 2 or 4 (other values: 4; one
+// instead of 4 where the cells alone fill the SMs);
 // sector: fhat in the sector order (N <= 16) instead of the convolution's
 // group layout
 void launch_dft_forward_fused(const double *f, const int64_t *slot_off, const DftSeg &s, const float2 *root,
