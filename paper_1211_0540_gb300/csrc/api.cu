@@ -932,7 +932,7 @@ bte_status enqueue_indicator(bte_ctx *c, Batch *B, const double *f, const double
     float *d2 = e2 + (size_t)B->nslots * c->ind->S;
     *ind = d2 + (size_t)B->nslots * c->ind->S;
     launch_indicator(*c->ind, *t, (const float2 *)c->scratch[SC_F], (const float2 *)c->scratch[SC_QH], sg.eoff,
-                     sg.nslots, sg.nvalid, e2, d2, *ind, st);
+                     sg.nslots, sg.nvalid, e2, d2, *ind, c->d_status, st);
     count_launches(c, 4);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? BTE_OK : cuda_fail(c, e, "indicator launch");

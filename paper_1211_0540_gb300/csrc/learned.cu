@@ -14,6 +14,7 @@
 #include <cmath>
 #include <vector>
 
+#include "bulk.cuh"
 #include "learned.h"
 #include "fpconv.cuh"
 #include "project.cuh"
@@ -27,19 +28,44 @@ namespace {
 // warps work in pairs, each pair takes the pencil's kept (m1, m2) blocks in
 // turn (unordered pairs, weights
 // Ghat(k,m) + Ghat(k,n)) and each warp of a pair half of the N outputs k3,
-// with the full and the loss weights side by side: the a and b rows of a block
-// are loaded into registers by both warps of its pair. Half the outputs per
-// warp keep the kernel at two CTAs per SM. Partial sums are added across the
-// pairs in a fixed order, then compared with the transform of the projected
-// surrogate output.
+// with the full and the loss weights side by side. A block's a and b rows and
+// its weights come by bulk copies into a two-deep ring of the pair, issued two
+// blocks ahead (read straight from L2 the loads left the FMA pipe 34 % busy:
+// 1024 cells, N = 16, 57 us, with the ring 50). Half the outputs per warp keep the kernel at
+// two CTAs per SM. Partial sums are added across the pairs in a fixed order, then
+// compared with the transform of the projected surrogate output.
 constexpr int kIndWarps = 8;
 constexpr int kIndPairs = kIndWarps / 2;
+constexpr int kIndStages = 2;
+constexpr int kIndBlocks = 16;  // blocks of a part
+
+// Pairs of one block for the outputs of half jh, in groups of four weights.
+template <int N>
+__host__ __device__ constexpr int ind_groups(int jh) {
+    int c = 0;
+    for (int m = 0; m < N; ++m)
+        for (int j = jh * N / 2; j < (jh + 1) * N / 2; ++j) c += pair_on_grid(j, m, N);
+    return (c + 3) / 4;
+}
+// Floats of a block's weights: half 0, then half 1, four full and four loss weights in turn.
+template <int N>
+__host__ __device__ constexpr int ind_weights() {
+    return 8 * (ind_groups<N>(0) + ind_groups<N>(1));
+}
+template <int N>
+constexpr int ind_stage_bytes() {
+    return 2 * N * kLanes * 8 + 4 * ind_weights<N>();
+}
+template <int N>
+constexpr size_t ind_smem() {
+    const size_t ring = (size_t)kIndPairs * kIndStages * ind_stage_bytes<N>(), red = sizeof(float) * kIndPairs * 4 * N * kLanes;
+    return ring > red ? ring : red;
+}
 
 // The pair sums of one block for the outputs k3 in [JH N/2, (JH + 1) N/2):
 // acc = full (re, im) per output, then loss (re, im). The weight of the pair
-// (m3, k3) sits at its rank among the block's valid pairs (m3 major, k3 minor),
-// a compile-time index after unrolling.
-// The full and the loss weights alternate in fours.
+// (m3, k3) sits at its rank among the half's pairs (m3 major, k3 minor), a
+// compile-time index after unrolling.
 template <int N, int JH>
 __device__ __forceinline__ void indicator_block(const float2 (&av)[N], const float2 (&bv)[N], const float4 *w,
                                                 float (&acc)[2 * N]) {
@@ -48,62 +74,102 @@ __device__ __forceinline__ void indicator_block(const float2 (&av)[N], const flo
 #pragma unroll
     for (int m3 = 0; m3 < N; ++m3)
 #pragma unroll
-        for (int j = 0; j < N; ++j) {
+        for (int j = J0; j < J0 + H; ++j) {
             const int n3 = j - m3 + H;
             if (n3 < 0 || n3 >= N) continue;
-            if (j >= J0 && j < J0 + H) {
-                const float4 f4 = w[2 * (wi >> 2)], l4 = w[2 * (wi >> 2) + 1];
-                const int q = wi & 3;
-                const float wF = q == 0 ? f4.x : q == 1 ? f4.y : q == 2 ? f4.z : f4.w;
-                const float wL = q == 0 ? l4.x : q == 1 ? l4.y : q == 2 ? l4.z : l4.w;
-                const float pr = av[m3].x * bv[n3].x - av[m3].y * bv[n3].y;
-                const float pi = av[m3].x * bv[n3].y + av[m3].y * bv[n3].x;
-                const int o = j - J0;
-                acc[2 * o] = fmaf(wF, pr, acc[2 * o]);
-                acc[2 * o + 1] = fmaf(wF, pi, acc[2 * o + 1]);
-                acc[N + 2 * o] = fmaf(wL, pr, acc[N + 2 * o]);
-                acc[N + 2 * o + 1] = fmaf(wL, pi, acc[N + 2 * o + 1]);
-            }
+            const float4 f4 = w[2 * (wi >> 2)], l4 = w[2 * (wi >> 2) + 1];
+            const int q = wi & 3;
+            const float wF = q == 0 ? f4.x : q == 1 ? f4.y : q == 2 ? f4.z : f4.w;
+            const float wL = q == 0 ? l4.x : q == 1 ? l4.y : q == 2 ? l4.z : l4.w;
+            const float pr = av[m3].x * bv[n3].x - av[m3].y * bv[n3].y;
+            const float pi = av[m3].x * bv[n3].y + av[m3].y * bv[n3].x;
+            const int o = j - J0;
+            acc[2 * o] = fmaf(wF, pr, acc[2 * o]);
+            acc[2 * o + 1] = fmaf(wF, pi, acc[2 * o + 1]);
+            acc[N + 2 * o] = fmaf(wL, pr, acc[N + 2 * o]);
+            acc[N + 2 * o + 1] = fmaf(wL, pi, acc[N + 2 * o + 1]);
             ++wi;
         }
 }
 
-// The pencil's blocks are split between two CTAs (blockIdx.z = half) so that
-// the S x groups items fill the GPU; each half reduces its pairs in a fixed
-// order into part[], and the half that finishes second (an atomic count, no
-// waiting) adds half 0 and half 1 in that order and forms the errors.
+// A pencil has between N^2/8 and N^2/2 blocks: it is cut into parts of
+// kIndBlocks blocks, one CTA each (blockIdx.z), so that the S x groups items
+// fill the GPU and no SM is left with a whole long pencil. Each part reduces
+// its pairs in a fixed order into part[], and the part that finishes last (an
+// atomic count, no waiting) adds the parts in their order and forms the errors.
+// 1024 cells, N = 16, 8 / 16 / 24 / 32 blocks a part: 59.7 / 51.0 / 48.2 / 57.6 us;
+// 16 leaves a small batch with more CTAs (the indicator of a few cells 67 -> 47 us).
 template <int N>
 __global__ void __launch_bounds__(32 * kIndWarps, 2)
 indicator_kernel(const float2 *__restrict__ F, const float2 *__restrict__ QN, const float *__restrict__ W,
-                 const uint32_t *__restrict__ desc, const IndPencil *__restrict__ pens, int cpad, int64_t eoff, int nslots, float *err2, float *den2, float *part, unsigned *cnt) {
-    constexpr int M = N * N * N, H = N / 2;
-    extern __shared__ __align__(16) float red[];  // [kIndPairs][4 N][32]
-    const int p = blockIdx.x, g = blockIdx.y, half = blockIdx.z, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+                 const uint32_t *__restrict__ desc, const IndPencil *__restrict__ pens, int parts,
+                 int64_t eoff, int nslots, float *err2, float *den2, float *part, unsigned *cnt, int *status) {
+    constexpr int M = N * N * N, H = N / 2, ROW = N * kLanes * 8, STAGE = ind_stage_bytes<N>();
+    extern __shared__ __align__(128) char ind_raw[];
+    __shared__ __align__(8) uint64_t s_full[kIndPairs][kIndStages];
+    __shared__ bool s_last;
+    float *red = reinterpret_cast<float *>(ind_raw);  // [kIndPairs][4 N][32], after the ring's last use
+    const int p = blockIdx.x, g = blockIdx.y, z = blockIdx.z, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int pair = warp >> 1, jh = warp & 1;
     const IndPencil pen = pens[p];
+    const int nz = (pen.nblocks + kIndBlocks - 1) / kIndBlocks;
+    if (z >= nz) return;
     const int k1 = pen.kk / N, k2 = pen.kk % N;
     const float2 *Fg = F + eoff + (int64_t)g * M * kLanes;  // fhat in the sector order of the group
+    char *ring = ind_raw + (size_t)pair * kIndStages * STAGE;
+    const bool producer = jh == 0 && lane == 0;
+    if (producer) {
+        for (int s = 0; s < kIndStages; ++s) mbar_init(smem_u32(&s_full[pair][s]), 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
     float acc[2 * N];  // this warp's outputs: full (re, im) per k3, then loss (re, im)
 #pragma unroll
     for (int i = 0; i < 2 * N; ++i) acc[i] = 0.f;
-    const int bmid = pen.nblocks / 2, bend = half ? pen.nblocks : bmid;
-    for (int b = (half ? bmid : 0) + pair; b < bend; b += kIndPairs) {
-        const uint32_t d = desc[pen.desc_off + b];
+    const int b0 = z * kIndBlocks + pair, bend = min((z + 1) * kIndBlocks, pen.nblocks);
+    const int n = b0 < bend ? (bend - b0 + kIndPairs - 1) / kIndPairs : 0;
+    auto issue = [&](int i) {  // rows of a group are N * 256 bytes, whole sectors
+        const int b = b0 + i * kIndPairs, s = i % kIndStages;
+        const uint32_t d = desc[pen.desc_off + b], bar = smem_u32(&s_full[pair][s]), dst = smem_u32(ring + s * STAGE);
         const int m1 = (int)(d & 0xffffu), m2 = (int)(d >> 16), n1 = k1 - m1 + H, n2 = k2 - m2 + H;
-        float2 av[N], bv[N];
+        mbar_expect_tx(bar, STAGE);
+        bulk_g2s(dst, Fg + (int64_t)((m1 * N + m2) * N) * kLanes, ROW, bar);
+        bulk_g2s(dst + ROW, Fg + (int64_t)((n1 * N + n2) * N) * kLanes, ROW, bar);
+        bulk_g2s(dst + 2 * ROW, W + pen.wofs + (size_t)b * ind_weights<N>(), 4 * ind_weights<N>(), bar);
+    };
+    if (producer)
+        for (int i = 0; i < kIndStages && i < n; ++i) issue(i);
+    bool live = true;  // until a wait runs out: then the pair only keeps its barriers
+    for (int i = 0; i < n; ++i) {
+        const int s = i % kIndStages;
+        if (live) live = __all_sync(0xffffffffu, mbar_wait_bounded(smem_u32(&s_full[pair][s]), (i / kIndStages) & 1));
+        if (live) {
+            const char *st = ring + s * STAGE;
+            float2 av[N], bv[N];
 #pragma unroll
-        for (int i = 0; i < N; i += 2) {  // two modes of the lane per 16-byte load (rows start on a sector)
-            const float4 a2 = *reinterpret_cast<const float4 *>(Fg + sector_index((m1 * N + m2) * N + i, lane));
-            const float4 b2 = *reinterpret_cast<const float4 *>(Fg + sector_index((n1 * N + n2) * N + i, lane));
-            av[i] = make_float2(a2.x, a2.y);
-            av[i + 1] = make_float2(a2.z, a2.w);
-            bv[i] = make_float2(b2.x, b2.y);
-            bv[i + 1] = make_float2(b2.z, b2.w);
+            for (int e = 0; e < N; e += 2) {  // two modes of the lane per 16-byte load (rows start on a sector)
+                const float4 a2 = *reinterpret_cast<const float4 *>(st + 8 * sector_index(e, lane));
+                const float4 b2 = *reinterpret_cast<const float4 *>(st + ROW + 8 * sector_index(e, lane));
+                av[e] = make_float2(a2.x, a2.y);
+                av[e + 1] = make_float2(a2.z, a2.w);
+                bv[e] = make_float2(b2.x, b2.y);
+                bv[e + 1] = make_float2(b2.z, b2.w);
+            }
+            const float4 *w = reinterpret_cast<const float4 *>(st + 2 * ROW);
+            if (jh == 0) indicator_block<N, 0>(av, bv, w, acc);
+            else indicator_block<N, 1>(av, bv, w + 2 * ind_groups<N>(0), acc);
         }
-        const float4 *w = reinterpret_cast<const float4 *>(W + pen.wofs + (size_t)b * 2 * cpad);
-        if (jh == 0) indicator_block<N, 0>(av, bv, w, acc);
-        else indicator_block<N, 1>(av, bv, w, acc);
+        asm volatile("bar.sync %0, 64;" ::"r"(pair + 1) : "memory");  // both warps have read the stage
+        if (producer && live && i + kIndStages < n) {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            issue(i + kIndStages);
+        }
+        if (!live && lane == 0) atomicOr(status, ST_TIMEOUT);
     }
+    if (producer && !live)  // no copy stays in flight (bounded again)
+        for (int s = 0; s < kIndStages; ++s)
+            for (uint32_t ph = 0; ph < 2; ++ph) mbar_wait_bounded(smem_u32(&s_full[pair][s]), ph);
+    __syncthreads();  // the ring becomes the reduction's buffer
     // the pair's 4 N sums: full (re, im) of output k3 at 2 k3, loss at 2 N + 2 k3
 #pragma unroll
     for (int o = 0; o < H; ++o) {
@@ -114,42 +180,45 @@ indicator_kernel(const float2 *__restrict__ F, const float2 *__restrict__ QN, co
         red[(pair * 4 * N + 2 * N + 2 * k3 + 1) * kLanes + lane] = acc[N + 2 * o + 1];
     }
     __syncthreads();
-    if (warp != 0) return;
     const size_t item = (size_t)p * gridDim.y + g;
-    float *mine = part + (item * 2 + half) * (4 * N * kLanes) + lane;
-    for (int i = 0; i < 4 * N; ++i) {
+    float *mine = part + (item * parts + z) * (4 * N * kLanes);
+    for (int i = threadIdx.x; i < 4 * N * kLanes; i += 32 * kIndWarps) {
         float v = 0.f;
-        for (int w = 0; w < kIndPairs; ++w) v += red[((size_t)w * 4 * N + i) * kLanes + lane];
-        mine[i * kLanes] = v;
+        for (int w = 0; w < kIndPairs; ++w) v += red[(size_t)w * 4 * N * kLanes + i];
+        mine[i] = v;
     }
-    __threadfence();  // this half's sums before the count
-    __syncwarp();
-    unsigned old = 0;
-    if (lane == 0) old = atomicAdd(cnt + item, 1u);
-    old = __shfl_sync(0xffffffffu, old, 0);
-    if (old != 1u) return;
-    __threadfence();  // the other half's sums after the count
-    const float *h0 = part + item * 2 * (4 * N * kLanes) + lane, *h1 = h0 + 4 * N * kLanes;
+    __threadfence();  // this part's sums before the count
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(cnt + item, 1u) == (unsigned)nz - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();  // the other parts' sums after the count
+    const float *h = part + item * parts * (4 * N * kLanes) + lane;
     float e = 0.f, dn = 0.f;
     const float2 *qn = QN + eoff + (int64_t)g * M * kLanes + (int64_t)pen.kk * N * kLanes + lane;
-    for (int j = 0; j < N; ++j) {
-        const float fr = __ldcg(h0 + (2 * j) * kLanes) + __ldcg(h1 + (2 * j) * kLanes);
-        const float fi = __ldcg(h0 + (2 * j + 1) * kLanes) + __ldcg(h1 + (2 * j + 1) * kLanes);
-        const float lr = __ldcg(h0 + (2 * N + 2 * j) * kLanes) + __ldcg(h1 + (2 * N + 2 * j) * kLanes);
-        const float li = __ldcg(h0 + (2 * N + 2 * j + 1) * kLanes) + __ldcg(h1 + (2 * N + 2 * j + 1) * kLanes);
+    for (int j = warp; j < N; j += kIndWarps) {
+        float v[4] = {};
+        for (int i = 0; i < nz; ++i)
+#pragma unroll
+            for (int o = 0; o < 4; ++o)
+                v[o] += __ldcg(h + (i * 4 * N + (o >> 1) * 2 * N + 2 * j + (o & 1)) * kLanes);
         const float2 q = qn[(int64_t)j * kLanes];
-        const float dr = q.x - fr, di = q.y - fi;
+        const float dr = q.x - v[0], di = q.y - v[1];
         e += dr * dr + di * di;
-        dn += lr * lr + li * li;
+        dn += v[2] * v[2] + v[3] * v[3];
+    }
+    red[warp * kLanes + lane] = e;  // the pairs' sums were read before the count
+    red[(kIndWarps + warp) * kLanes + lane] = dn;
+    __syncthreads();
+    if (warp != 0) return;
+    e = dn = 0.f;
+    for (int w = 0; w < kIndWarps; ++w) {
+        e += red[w * kLanes + lane];
+        dn += red[(kIndWarps + w) * kLanes + lane];
     }
     const int slot = g * kLanes + lane;
     err2[(size_t)p * nslots + slot] = e;
     den2[(size_t)p * nslots + slot] = dn;
-}
-
-template <int N>
-constexpr size_t ind_smem() {
-    return sizeof(float) * kIndPairs * 4 * N * kLanes;
 }
 
 __global__ void indicator_reduce_kernel(const float *__restrict__ err2, const float *__restrict__ den2, int S,
@@ -384,15 +453,13 @@ int build_indicator_table(const Table &t, int modes, uint64_t seed, IndicatorTab
     // the sampled pencils' own blocks: the modes are compared one by one, so the
     // sums run over the pencil's box with the plain pair weights Ghat(k, m) +
     // Ghat(k, n) (blocks (m1, m2) <= (n1, n2); a block that pairs with itself
-    // keeps Ghat(k, m)), the full ones and those of the loss term, per block m3
-    // ascending, then k3, padded to 16 bytes
-    int cpad = 0;
-    for (int m3 = 0; m3 < N; ++m3)
-        for (int k3 = 0; k3 < N; ++k3) cpad += pair_on_grid(k3, m3, N);
-    cpad = (cpad + 3) & ~3;
+    // keeps Ghat(k, m)), the full ones and those of the loss term, for the
+    // outputs k3 < N/2 and then the others, each m3 ascending, then k3, in groups
+    // of four full and four loss weights
     std::vector<float> w;
     std::vector<IndPencil> pens;
     std::vector<uint32_t> desc;
+    int parts = 1;
     for (int kk : kks) {
         const int k1 = kk / N, k2 = kk % N;
         IndPencil pn{};
@@ -406,36 +473,39 @@ int build_indicator_table(const Table &t, int modes, uint64_t seed, IndicatorTab
                 desc.push_back((uint32_t)m1 | ((uint32_t)m2 << 16));
             }
         pn.nblocks = (int)desc.size() - pn.desc_off;
+        parts = std::max(parts, (pn.nblocks + kIndBlocks - 1) / kIndBlocks);
         for (int b = 0; b < pn.nblocks; ++b) {
             const uint32_t dd = desc[pn.desc_off + b];
             const int m1 = (int)(dd & 0xffffu), m2 = (int)(dd >> 16), n1 = k1 - m1 + h, n2 = k2 - m2 + h;
             const bool pair = !(m1 == n1 && m2 == n2);
-            const size_t base = w.size();
-            w.resize(base + 2 * (size_t)cpad, 0.0f);
-            size_t wi = 0;
-            for (int m3 = 0; m3 < N; ++m3)
-                for (int k3 = 0; k3 < N; ++k3) {
-                    const int n3 = k3 - m3 + h;
-                    if (n3 < 0 || n3 >= N) continue;
-                    double full = t.ghat(k1, k2, k3, m1, m2, m3);
-                    if (pair) full += t.ghat(k1, k2, k3, n1, n2, n3);
-                    float *const e = &w[base + 8 * (wi / 4) + wi % 4];  // four full weights, then their loss parts
-                    ++wi;
-                    e[0] = (float)(full * dz3);
-                    const int sm = (m1 - h) * (m1 - h) + (m2 - h) * (m2 - h) + (m3 - h) * (m3 - h);
-                    double g = -c * t.J[sm];
-                    if (pair) {
-                        const int sn = (n1 - h) * (n1 - h) + (n2 - h) * (n2 - h) + (n3 - h) * (n3 - h);
-                        g += -c * t.J[sn];
+            for (int jh = 0; jh < 2; ++jh) {
+                size_t wi = 0;
+                const size_t base = w.size();
+                for (int m3 = 0; m3 < N; ++m3)
+                    for (int k3 = jh * h; k3 < (jh + 1) * h; ++k3) {
+                        const int n3 = k3 - m3 + h;
+                        if (n3 < 0 || n3 >= N) continue;
+                        double full = t.ghat(k1, k2, k3, m1, m2, m3);
+                        const int sm = (m1 - h) * (m1 - h) + (m2 - h) * (m2 - h) + (m3 - h) * (m3 - h);
+                        double g = -c * t.J[sm];
+                        if (pair) {
+                            const int sn = (n1 - h) * (n1 - h) + (n2 - h) * (n2 - h) + (n3 - h) * (n3 - h);
+                            full += t.ghat(k1, k2, k3, n1, n2, n3);
+                            g += -c * t.J[sn];
+                        }
+                        if (wi % 4 == 0) w.resize(w.size() + 8, 0.0f);
+                        float *const e = &w[base + 8 * (wi / 4) + wi % 4];
+                        ++wi;
+                        e[0] = (float)(full * dz3);
+                        e[4] = (float)(g * dz3);
                     }
-                    e[4] = (float)(g * dz3);
-                }
+            }
         }
         pens.push_back(pn);
     }
     out.S = S;
+    out.parts = parts;
     out.kks = kks;
-    out.cpad = cpad;
     cudaError_t e = cudaMalloc(&out.d_w, sizeof(float) * std::max<size_t>(w.size(), 4));
     if (e == cudaSuccess) e = cudaMalloc(&out.d_desc, sizeof(uint32_t) * std::max<size_t>(desc.size(), 1));
     if (e == cudaSuccess)
@@ -479,33 +549,27 @@ void launch_post_project(const float *Y, const double *rho, int B, int N, float 
 
 size_t indicator_scratch_floats(const IndicatorTable &it, int N, int nslots) {
     const size_t items = (size_t)it.S * (nslots / kLanes);
-    return 2 * (size_t)it.S * nslots + nslots + items * 2 * 4 * N * kLanes + items;
+    return 2 * (size_t)it.S * nslots + nslots + items * it.parts * 4 * N * kLanes + items;
 }
 
 void launch_indicator(const IndicatorTable &it, const Table &t, const float2 *F, const float2 *QN, int64_t eoff,
-                      int nslots, int nvalid, float *err2, float *den2, float *ind, cudaStream_t st) {
-    dim3 grid(it.S, nslots / kLanes, 2);
-    // after err2, den2 and ind: the halves' partial sums, then the per-item counts
+                      int nslots, int nvalid, float *err2, float *den2, float *ind, int *status,
+                      cudaStream_t st) {
+    dim3 grid(it.S, nslots / kLanes, it.parts);
+    // after err2, den2 and ind: the parts' sums, then the per-item counts
     const size_t items = (size_t)it.S * (nslots / kLanes);
     float *part = ind + nslots;
-    unsigned *cnt = reinterpret_cast<unsigned *>(part + items * 2 * 4 * t.N * kLanes);
+    unsigned *cnt = reinterpret_cast<unsigned *>(part + items * it.parts * 4 * t.N * kLanes);
     cudaMemsetAsync(cnt, 0, sizeof(unsigned) * items, st);
+#define BTE_INDICATOR(n) \
+    indicator_kernel<n><<<grid, 32 * kIndWarps, ind_smem<n>(), st>>>(F, QN, it.d_w, it.d_desc, it.d_pen, it.parts, \
+                                                                     eoff, nslots, err2, den2, part, cnt, status)
     switch (t.N) {
-        case 8:
-            indicator_kernel<8><<<grid, 32 * kIndWarps, ind_smem<8>(), st>>>(F, QN, it.d_w, it.d_desc,
-                                                                           it.d_pen, it.cpad, eoff, nslots, err2, den2, part, cnt);
-            break;
-        case 12:
-            indicator_kernel<12><<<grid, 32 * kIndWarps, ind_smem<12>(), st>>>(F, QN, it.d_w, it.d_desc,
-                                                                             it.d_pen, it.cpad, eoff, nslots, err2,
-                                                                             den2, part, cnt);
-            break;
-        default:
-            indicator_kernel<16><<<grid, 32 * kIndWarps, ind_smem<16>(), st>>>(F, QN, it.d_w, it.d_desc,
-                                                                             it.d_pen, it.cpad, eoff, nslots, err2,
-                                                                             den2, part, cnt);
-            break;
+        case 8: BTE_INDICATOR(8); break;
+        case 12: BTE_INDICATOR(12); break;
+        default: BTE_INDICATOR(16); break;
     }
+#undef BTE_INDICATOR
     indicator_reduce_kernel<<<(nslots + 255) / 256, 256, 0, st>>>(err2, den2, it.S, nslots, nvalid, ind);
 }
 

@@ -10,7 +10,7 @@ namespace bte {
 
 // Sampled pencils of the indicator: for pencil i, the (m1, m2) blocks of zeta
 // pencil kk = k1 N + k2 (d_desc + desc_off) and their full and loss-term pair
-// weights (d_w + wofs, 2 cpad floats a block, alternating in fours).
+// weights (d_w + wofs, ind_weights(N) floats a block; learned.cu).
 struct IndPencil {
     int kk, desc_off, nblocks, pad;
     uint64_t wofs;
@@ -18,8 +18,8 @@ struct IndPencil {
 
 struct IndicatorTable {
     int S = 0;                     // sampled pencils (S x N sampled modes)
+    int parts = 1;                 // CTAs of the longest pencil
     std::vector<int> kks;          // host copy of the sampled pencils (k1 N + k2), drawing order
-    int cpad = 0;                  // floats per block of weights
     uint32_t *d_desc = nullptr;    // m1 | (m2 << 16)
     float *d_w = nullptr;          // weights of the sampled pencils (pair-symmetrised, times dz^3), full and loss
     IndPencil *d_pen = nullptr;
@@ -50,6 +50,6 @@ void launch_fallback_setup(const float *ind, int ncells, double tol, int64_t M, 
 void launch_stage_update(const double *Q, const double *x, double *y, const double *qp, double a, int64_t n,
                          int mode, cudaStream_t st);
 void launch_indicator(const IndicatorTable &it, const Table &t, const float2 *F, const float2 *QN, int64_t eoff,
-                      int nslots, int nvalid, float *err2, float *den2, float *ind, cudaStream_t st);
+                      int nslots, int nvalid, float *err2, float *den2, float *ind, int *status, cudaStream_t st);
 
 }  // namespace bte
