@@ -911,7 +911,8 @@ bte_status ensure_indicator(bte_ctx *c) {
 // Indicator of the uniform batch B (cells of table 0): transform of f at every
 // mode, of Q at the sampled pencils, the exact sums there and the per-slot
 // ratio. *ind receives the device array (one float per slot, in SC_MISC).
-bte_status enqueue_indicator(bte_ctx *c, Batch *B, const double *f, const double *Q, float **ind, cudaStream_t st) {
+bte_status enqueue_indicator(bte_ctx *c, Batch *B, const double *f, const double *Q, float **ind, cudaStream_t st,
+                             double *ind64 = nullptr) {
     const Segment &sg = B->segs[0];
     const Table *t = c->tables[0];
     bte_status s;
@@ -932,7 +933,7 @@ bte_status enqueue_indicator(bte_ctx *c, Batch *B, const double *f, const double
     float *d2 = e2 + (size_t)B->nslots * c->ind->S;
     *ind = d2 + (size_t)B->nslots * c->ind->S;
     launch_indicator(*c->ind, *t, (const float2 *)c->scratch[SC_F], (const float2 *)c->scratch[SC_QH], sg.eoff,
-                     sg.nslots, sg.nvalid, e2, d2, *ind, c->d_status, st);
+                     sg.nslots, sg.nvalid, e2, d2, *ind, ind64, c->d_status, st);
     count_launches(c, 4);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? BTE_OK : cuda_fail(c, e, "indicator launch");
@@ -1532,9 +1533,7 @@ bte_status bte_learned_indicator(bte_ctx *c, const double *f, const double *Q, i
     if ((s = prepare(c, B, BTE_FP32, false, false)) != BTE_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
     float *d_ind = nullptr;
-    if ((s = enqueue_indicator(c, B, f, Q, &d_ind, st)) != BTE_OK) return s;
-    launch_widen(d_ind, ind, (int)ncells, st);
-    count_launches(c, 1);
+    if ((s = enqueue_indicator(c, B, f, Q, &d_ind, st, ind)) != BTE_OK) return s;
     fence_record(c, st);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? BTE_OK : cuda_fail(c, e, "bte_learned_indicator: launch");

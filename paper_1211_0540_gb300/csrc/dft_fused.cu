@@ -314,7 +314,8 @@ dft_inv_fused_kernel(const float2 *__restrict__ G, const int64_t *__restrict__ s
     float *R = UPD ? reinterpret_cast<float *>(base + NP) : reinterpret_cast<float *>(A);
     __shared__ float red[32][10];
     __shared__ float part[10];
-    __shared__ double sg[N], lam[5];
+    __shared__ double tab[3][N], lam[5];
+    const double(&sg)[N] = tab[2];
     const int r = (int)cl.block_rank(), sl = blockIdx.x / C, t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int64_t off = slot_off[s.s0 + sl];
     if (off < 0) return;  // the whole cluster leaves
@@ -401,30 +402,23 @@ dft_inv_fused_kernel(const float2 *__restrict__ G, const int64_t *__restrict__ s
     }
     if (mode != 0) {
         // moments: warp trees, warp 0 over the CTA's warps, then the cluster's partials in rank order
-#pragma unroll
-        for (int i = 0; i < 5; ++i) mom[i] = df_warp_sum(mom[i]);
-        if (S::NW > 1) {
-            if (lane == 0)
-#pragma unroll
-                for (int i = 0; i < 5; ++i) {
-                    red[warp][2 * i] = mom[i].hi;
-                    red[warp][2 * i + 1] = mom[i].lo;
-                }
+        Df sum;
+        const int mi = df_warp_sum5(mom, sum);
+        float *const to = S::NW > 1 ? red[warp] : part;
+        if (mi >= 0) {
+            to[2 * mi] = sum.hi;
+            to[2 * mi + 1] = sum.lo;
+        }
+        if constexpr (S::NW > 1) {
             __syncthreads();
-            if (warp == 0) {
+            if (t < 5) {
+                Df m{red[0][2 * t], red[0][2 * t + 1]};
 #pragma unroll
-                for (int i = 0; i < 5; ++i)
-                    mom[i] = lane < S::NW ? Df{red[lane][2 * i], red[lane][2 * i + 1]} : Df{0.f, 0.f};
-#pragma unroll
-                for (int i = 0; i < 5; ++i) mom[i] = df_warp_sum(mom[i]);
+                for (int w = 1; w < S::NW; ++w) m = df_add(m, Df{red[w][2 * t], red[w][2 * t + 1]});
+                part[2 * t] = m.hi;
+                part[2 * t + 1] = m.lo;
             }
         }
-        if (t == 0)
-#pragma unroll
-            for (int i = 0; i < 5; ++i) {
-                part[2 * i] = mom[i].hi;
-                part[2 * i + 1] = mom[i].lo;
-            }
         cell_sync<C>(cl);
         if (warp == 0) {
             double mu = 0.0;
@@ -448,18 +442,11 @@ dft_inv_fused_kernel(const float2 *__restrict__ G, const int64_t *__restrict__ s
                 for (int k = 0; k < 5; ++k) l = fma(pa.ainv[lane * 5 + k], m5[k], l);
                 lam[lane] = l;
             }
+            __syncwarp();
+            correction_tables<N>(lam, pa.dv, tab);
         }
-        cell_sync<C>(cl);  // every CTA has read the partials before any leaves; lambda is visible
-        // correction C^T lambda = base(j1, j2) + g(j3)
-        const double dv = pa.dv;
-        if (t < N) {
-            const double v = dv * (double)(t - H);
-            sg[t] = fma(lam[3], v, lam[4] * v * v);
-        }
-        if (act) {
-            const double v1 = dv * (double)(r * JR + t / N - H), v2 = dv * (double)(t % N - H);
-            base[t] = lam[0] + fma(lam[1], v1, fma(lam[2], v2, lam[4] * fma(v1, v1, v2 * v2)));
-        }
+        cell_sync<C>(cl);  // every CTA has read the partials before any leaves; the tables are visible
+        if (act) base[t] = tab[0][r * JR + t / N] + tab[1][t % N];
     }
     __syncthreads();
     // coalesced output of the own slab: local value e = (pencil p, j3)

@@ -222,7 +222,7 @@ indicator_kernel(const float2 *__restrict__ F, const float2 *__restrict__ QN, co
 }
 
 __global__ void indicator_reduce_kernel(const float *__restrict__ err2, const float *__restrict__ den2, int S,
-                                        int nslots, int nvalid, float *ind) {
+                                        int nslots, int nvalid, float *ind, double *ind64) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= nslots) return;
     float e = 0.f, d = 0.f;
@@ -230,7 +230,9 @@ __global__ void indicator_reduce_kernel(const float *__restrict__ err2, const fl
         e += err2[(size_t)s * nslots + c];
         d += den2[(size_t)s * nslots + c];
     }
-    ind[c] = c < nvalid ? sqrtf(e) / fmaxf(sqrtf(d), 1e-30f) : 0.f;
+    const float v = c < nvalid ? sqrtf(e) / fmaxf(sqrtf(d), 1e-30f) : 0.f;
+    ind[c] = v;
+    if (ind64 && c < nvalid) ind64[c] = (double)v;  // the caller's array (slot = cell)
 }
 
 // Surrogate output to the caller's cells with the conservation projection of
@@ -238,7 +240,9 @@ __global__ void indicator_reduce_kernel(const float *__restrict__ err2, const fl
 // cell, one thread per pencil (j1, j2): the moments of Y are accumulated in
 // double-float FP32 (the values are FP32), mu(Q) = c mu(Y) and lambda are
 // formed in FP64, and Q_j = c Y_j - C_j^T lambda is written in FP64 on a
-// coalesced mapping (one FP64 operation per value).
+// coalesced mapping (one FP64 operation per value). Instructions bound it: 1024
+// cells, N = 16, 34.6 us with five warp trees, the correction's polynomial per
+// pencil and two renormalised additions a value, 24 us as it stands.
 template <int N>
 __global__ void __launch_bounds__((N * N + 31) / 32 * 32)
 post_project_kernel(const float *__restrict__ Y, const double *__restrict__ rho, float s_out, ProjArgs pa,
@@ -248,8 +252,9 @@ post_project_kernel(const float *__restrict__ Y, const double *__restrict__ rho,
     const float *y = Y + (size_t)r * M;
     double *q = Q + (size_t)r * M;
     __shared__ float red[NW][10];
-    __shared__ float2 base[NN], sg[N];
-    __shared__ double lam[5], c_s;
+    __shared__ float2 base[NN];
+    __shared__ __align__(16) float2 sg[N];
+    __shared__ double lam[5], tab[3][N], c_s;
     __shared__ float2 c_hl;
     if (t == 0) {  // the output scale, once per cell (an FP64 division), and its double-float split
         const double c = rho[r] * rho[r] / (double)s_out;
@@ -260,13 +265,18 @@ post_project_kernel(const float *__restrict__ Y, const double *__restrict__ rho,
     Df mom[5];
     if (t < NN) {
         Df s0{0.f, 0.f}, s1{0.f, 0.f}, s2{0.f, 0.f};
-        const float *yp = y + t * N;
+        const float4 *yp = reinterpret_cast<const float4 *>(y + t * N);
 #pragma unroll
-        for (int j = 0; j < N; ++j) {
-            const float v = yp[j];
-            df_add(s0, v);
-            df_add_prod(s1, (float)(j - H), v);
-            df_add_prod(s2, (float)((j - H) * (j - H)), v);
+        for (int i = 0; i < N / 4; ++i) {
+            const float4 v4 = yp[i];
+            const float v[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+            for (int o = 0; o < 4; ++o) {
+                const int w = 4 * i + o - H;
+                df_add(s0, v[o]);
+                df_add_prod(s1, (float)w, v[o]);
+                df_add_prod(s2, (float)(w * w), v[o]);
+            }
         }
         const int w1 = t / N - H, w2 = t % N - H;
         mom[0] = s0;
@@ -278,26 +288,22 @@ post_project_kernel(const float *__restrict__ Y, const double *__restrict__ rho,
 #pragma unroll
         for (int i = 0; i < 5; ++i) mom[i] = Df{0.f, 0.f};
     }
-#pragma unroll
-    for (int i = 0; i < 5; ++i) mom[i] = df_warp_sum(mom[i]);
-    if (lane == 0)
-#pragma unroll
-        for (int i = 0; i < 5; ++i) {
-            red[warp][2 * i] = mom[i].hi;
-            red[warp][2 * i + 1] = mom[i].lo;
-        }
+    Df sum;
+    const int mi = df_warp_sum5(mom, sum);
+    if (mi >= 0) {
+        red[warp][2 * mi] = sum.hi;
+        red[warp][2 * mi + 1] = sum.lo;
+    }
     __syncthreads();
     if (warp == 0) {
-#pragma unroll
-        for (int i = 0; i < 5; ++i) mom[i] = lane < NW ? Df{red[lane][2 * i], red[lane][2 * i + 1]} : Df{0.f, 0.f};
-#pragma unroll
-        for (int i = 0; i < 5; ++i) mom[i] = df_warp_sum(mom[i]);
         double mu = 0.0;
-        const double c = c_s;
+        if (lane < 5) {
+            Df m{red[0][2 * lane], red[0][2 * lane + 1]};
 #pragma unroll
-        for (int i = 0; i < 5; ++i)
-            if (lane == i) mu = ((double)mom[i].hi + (double)mom[i].lo) * c;
-        mu *= lane == 0 ? 1.0 : (lane == 4 ? pa.dv * pa.dv : pa.dv);
+            for (int w = 1; w < NW; ++w) m = df_add(m, Df{red[w][2 * lane], red[w][2 * lane + 1]});
+            mu = (fpc::widen(m.hi) + fpc::widen(m.lo)) * c_s;
+            mu *= lane == 0 ? 1.0 : (lane == 4 ? pa.dv * pa.dv : pa.dv);
+        }
         double m5[5];
 #pragma unroll
         for (int i = 0; i < 5; ++i) m5[i] = __shfl_sync(0xffffffffu, mu, i);
@@ -307,36 +313,44 @@ post_project_kernel(const float *__restrict__ Y, const double *__restrict__ rho,
             for (int k = 0; k < 5; ++k) l = fma(pa.ainv[lane * 5 + k], m5[k], l);
             lam[lane] = l;
         }
+        __syncwarp();
+        correction_tables<N>(lam, pa.dv, tab);
     }
     __syncthreads();
     // The correction C^T lambda = base(j1, j2) + g(j3) is formed in FP64 per
     // pencil and per j3, then kept as double-float pairs (hi, lo): per value
-    // Q = c Y - base - g is then FP32 work (an exact TwoProduct for c Y and
-    // two double-float additions, relative error ~2^-48) and one FP64
-    // addition hi + lo, instead of three FP64-unit operations.
-    const double dv = pa.dv;
-    if (t < N) {
-        const double v = dv * (double)(t - H);
-        const double g = fma(lam[3], v, lam[4] * v * v);
-        const float hi = fpc::narrow(g);
-        sg[t] = make_float2(hi, fpc::narrow(g - fpc::widen(hi)));
-    }
-    if (t < NN) {
-        const double v1 = dv * (double)(t / N - H), v2 = dv * (double)(t % N - H);
-        const double b = lam[0] + fma(lam[1], v1, fma(lam[2], v2, lam[4] * fma(v1, v1, v2 * v2)));
-        const float hi = fpc::narrow(b);
-        base[t] = make_float2(hi, fpc::narrow(b - fpc::widen(hi)));
-    }
+    // Q = c Y - base - g is then FP32 work (an exact TwoProduct for c Y, an
+    // exact TwoSum of the leading parts each and the sum of what they leave,
+    // relative error ~2^-48) and one FP64 addition hi + lo, instead of three
+    // FP64-unit operations.
+    const auto split = [](double v) {
+        const float hi = fpc::narrow(v);
+        return make_float2(-hi, -fpc::narrow(v - fpc::widen(hi)));
+    };
+    if (t < NN) base[t] = split(tab[0][t / N] + tab[1][t % N]);
+    if (t < N) sg[t] = split(tab[2][t]);
     __syncthreads();
     const float c_hi = c_hl.x, c_lo = c_hl.y;
-    for (int e = t; e < M; e += NT) {
-        const float yv = y[e];
-        const float p = c_hi * yv;
-        Df prod{p, fmaf(c_lo, yv, fmaf(c_hi, yv, -p))};
-        const float2 b = base[e / N], g = sg[e % N];
-        const Df corr = df_add(Df{b.x, b.y}, Df{g.x, g.y});
-        const Df v = df_add(prod, Df{-corr.hi, -corr.lo});
-        q[e] = fpc::widen(v.hi) + fpc::widen(v.lo);
+    const bool wide = (reinterpret_cast<uintptr_t>(q) & 15u) == 0;
+    const auto value = [&](float yv, float2 b, float2 g) {
+        const float p = __fmul_rn(c_hi, yv), pe = fmaf(c_lo, yv, fmaf(c_hi, yv, -p));
+        float s1, e1, s2, e2;
+        two_sum_f(b.x, g.x, s1, e1);
+        two_sum_f(p, s1, s2, e2);
+        const float lo = __fadd_rn(__fadd_rn(pe, __fadd_rn(b.y, g.y)), __fadd_rn(e1, e2));
+        return fpc::widen(s2) + fpc::widen(lo);
+    };
+    for (int e = 2 * t; e < M; e += 2 * NT) {  // two values of a pencil: 8-byte loads, 16-byte stores where q allows
+        const float2 yv = *reinterpret_cast<const float2 *>(y + e);
+        const float2 b = base[e / N];
+        const float4 g = *reinterpret_cast<const float4 *>(&sg[e % N]);
+        const double q0 = value(yv.x, b, make_float2(g.x, g.y)), q1 = value(yv.y, b, make_float2(g.z, g.w));
+        if (wide) {
+            *reinterpret_cast<double2 *>(q + e) = make_double2(q0, q1);
+        } else {
+            q[e] = q0;
+            q[e + 1] = q1;
+        }
     }
 }
 
@@ -408,17 +422,7 @@ __global__ void stage_update_kernel(const double *__restrict__ Q, const double *
         y[i] = mode == 1 ? fma(a, Q[i], x[i]) : fma(a, qp[i] + Q[i], y[i]);
 }
 
-// ind (one float per slot of a uniform batch, slot = cell) to the caller's doubles.
-__global__ void widen_kernel(const float *__restrict__ in, double *__restrict__ out, int n) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = (double)in[i];
-}
-
 }  // namespace
-
-void launch_widen(const float *in, double *out, int n, cudaStream_t st) {
-    if (n > 0) widen_kernel<<<(n + 255) / 256, 256, 0, st>>>(in, out, n);
-}
 
 void launch_fallback_setup(const float *ind, int ncells, double tol, int64_t M, const ConvItem *tmpl, int ntmpl,
                            int nslots_cap, int64_t *off, ConvItem *items, int *nitems, unsigned *counter,
@@ -553,8 +557,8 @@ size_t indicator_scratch_floats(const IndicatorTable &it, int N, int nslots) {
 }
 
 void launch_indicator(const IndicatorTable &it, const Table &t, const float2 *F, const float2 *QN, int64_t eoff,
-                      int nslots, int nvalid, float *err2, float *den2, float *ind, int *status,
-                      cudaStream_t st) {
+                      int nslots, int nvalid, float *err2, float *den2, float *ind, double *ind64,
+                      int *status, cudaStream_t st) {
     dim3 grid(it.S, nslots / kLanes, it.parts);
     // after err2, den2 and ind: the parts' sums, then the per-item counts
     const size_t items = (size_t)it.S * (nslots / kLanes);
@@ -570,7 +574,7 @@ void launch_indicator(const IndicatorTable &it, const Table &t, const float2 *F,
         default: BTE_INDICATOR(16); break;
     }
 #undef BTE_INDICATOR
-    indicator_reduce_kernel<<<(nslots + 255) / 256, 256, 0, st>>>(err2, den2, it.S, nslots, nvalid, ind);
+    indicator_reduce_kernel<<<(nslots + 255) / 256, 256, 0, st>>>(err2, den2, it.S, nslots, nvalid, ind, ind64);
 }
 
 }  // namespace bte

@@ -38,8 +38,6 @@ void launch_post_project(const float *Y, const double *rho, int B, int N, float 
 // err2, den2: S * nslots floats of scratch each, ind: nslots floats followed by
 // the kernel's own scratch (indicator_scratch_floats counts all of it).
 size_t indicator_scratch_floats(const IndicatorTable &it, int N, int nslots);
-// out[i] = (double) in[i], i < n
-void launch_widen(const float *in, double *out, int n, cudaStream_t st);
 // The learned mode's fallback batch on the device (learned.cu): flagged cells
 // (ind > tol), offsets (-1 padding lanes, -2 unused groups), work list, its
 // length, the zeroed queue counter; statistics (cells, fallbacks, max ind bits).
@@ -50,6 +48,6 @@ void launch_fallback_setup(const float *ind, int ncells, double tol, int64_t M, 
 void launch_stage_update(const double *Q, const double *x, double *y, const double *qp, double a, int64_t n,
                          int mode, cudaStream_t st);
 void launch_indicator(const IndicatorTable &it, const Table &t, const float2 *F, const float2 *QN, int64_t eoff,
-                      int nslots, int nvalid, float *err2, float *den2, float *ind, int *status, cudaStream_t st);
+                      int nslots, int nvalid, float *err2, float *den2, float *ind, double *ind64, int *status, cudaStream_t st);
 
 }  // namespace bte

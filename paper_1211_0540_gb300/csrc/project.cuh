@@ -74,6 +74,42 @@ __device__ __forceinline__ Df df_warp_sum(Df v) {
     return v;
 }
 
+// Sums of five numbers over the 32 lanes, the lanes halving the set at each of
+// the first three steps (9 additions a lane instead of the 25 of five trees; the
+// additions are most of the work: 14 operations each). Returns the index of the
+// value whose sum the lane then holds in `sum`, or -1 (four lanes hold each).
+__device__ __forceinline__ int df_warp_sum5(const Df (&m)[5], Df &sum) {
+    const int lane = threadIdx.x & 31;
+    const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
+    const auto halve = [](const Df &lo, const Df &hi, bool upper, int o) {  // the upper lanes keep hi
+        const Df keep = upper ? hi : lo, send = upper ? lo : hi;
+        return df_add(keep, Df{__shfl_xor_sync(0xffffffffu, send.hi, o), __shfl_xor_sync(0xffffffffu, send.lo, o)});
+    };
+    const Df zero{0.f, 0.f};
+    const Df a0 = halve(m[0], m[3], h16, 16), a1 = halve(m[1], m[4], h16, 16), a2 = halve(m[2], zero, h16, 16);
+    const Df b0 = halve(a0, a2, h8, 8), b1 = halve(a1, zero, h8, 8);
+    Df c = halve(b0, b1, h4, 4);
+#pragma unroll
+    for (int o = 2; o > 0; o >>= 1)
+        c = df_add(c, Df{__shfl_xor_sync(0xffffffffu, c.hi, o), __shfl_xor_sync(0xffffffffu, c.lo, o)});
+    sum = c;
+    const int i = 2 * h8 + h4;
+    return i == 3 || (h16 && i == 2) ? -1 : 3 * h16 + i;
+}
+
+// The correction C^T lambda = base(j1, j2) + g(j3), base = a1(j1) + a2(j2), by
+// axes: tab[0] = a1, tab[1] = a2, tab[2] = g, formed by one warp in FP64 (per
+// pencil the polynomial takes nine operations on the FP64 unit, the sum of
+// two table entries one).
+template <int N>
+__device__ __forceinline__ void correction_tables(const double *lam, double dv, double (&tab)[3][N]) {
+    for (int i = threadIdx.x & 31; i < 3 * N; i += 32) {
+        const int ax = i / N;
+        const double v = dv * (double)(i % N - N / 2);
+        tab[ax][i % N] = (ax == 0 ? lam[0] : 0.0) + fma(lam[1 + ax], v, lam[4] * v * v);
+    }
+}
+
 // Block-wide sum of 5 values in a fixed order; result valid in all threads.
 // Only the first `active` threads hold data: the other warps skip the
 // shuffles, and five threads add the per-warp partials (FP64 is slow here, so
