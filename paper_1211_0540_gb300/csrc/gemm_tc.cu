@@ -3,7 +3,7 @@
 // followed by a fused epilogue (bias, GELU, residual, FP32 / BF16 / transposed BF16 stores).
 // Used by the learned surrogate (forward and backward passes of its MLP).
 //
-// Structure of one CTA (4 warps, one 128 x BN output tile, BN = 64, 128 or 256):
+// Structure of one CTA (kWarps warps, one 128 x BN output tile, BN = 64, 128 or 256):
 // - thread 0 (producer) streams 128 x 64 tiles of A and BN x 64 tiles of B with
 //   TMA (cp.async.bulk.tensor.2d, 128-byte swizzle) into a STAGES-deep ring
 //   (4, or 6-8 when the grid fits in one wave),
@@ -12,8 +12,8 @@
 //   tcgen05.mma.kind::f16 (K = 16 each) into the TMEM accumulator (128 lanes x
 //   BN FP32 columns) and commits the stage's "empty" barrier, then the "done"
 //   barrier after the last k tile;
-// - all four warps read their 32 TMEM lanes (rows) with tcgen05.ld and apply
-//   the epilogue.
+// - all warps read their 32 TMEM lanes (rows) with tcgen05.ld and apply the
+//   epilogue.
 // Every mbarrier wait is bounded by the global timer (1 s); after a timeout
 // the CTA sets the status word, skips the remaining waits and still frees its
 // TMEM before leaving.
@@ -31,6 +31,12 @@ namespace bte {
 namespace {
 
 constexpr int BM = 128, BK = 64;
+// The epilogue's warps: warp w reads the TMEM lanes of its quarter (w mod 4), the
+// columns go to the groups of four warps in turn. The epilogue follows the whole k
+// loop of a CTA that has its SM to itself, so its time adds up: the surrogate's three
+// layers and their neighbours on 1024 cells (N = 16) 102.3 us with four warps, 97.2
+// with eight.
+constexpr int kWarps = 8;
 constexpr unsigned long long kWaitNs = 1000000000ull;
 
 __device__ __forceinline__ uint32_t su32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -93,7 +99,7 @@ __device__ __forceinline__ float gelu_f(float x) {
 // wave takes the deepest ring that fits (192 KB). KB: 64-wide K boxes per
 // stage and operand (a k-step of KB * 64).
 template <int BN, int STAGES, int KB = 1>
-__global__ void __launch_bounds__(128, 1)
+__global__ void __launch_bounds__(32 * kWarps, 1)
 gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, GemmEpi g,
                     int M, int N, int K, int *status) {
     extern __shared__ uint8_t smem_raw[];
@@ -191,16 +197,16 @@ gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                      : "memory");
     }
     __syncwarp();
-    // epilogue: warp w owns TMEM lanes (rows) 32w .. 32w + 31
+    // epilogue: warp w owns the TMEM lanes (rows) 32 (w mod 4) .. + 31
     wait_bounded(su32(&bar_done), 0, abort, status);
     __syncwarp();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const int row = tile_m + warp * 32 + lane;
+    const int row = tile_m + (warp & 3) * 32 + lane;
     const bool rok = row < M && !*abort;
 #pragma unroll 1
-    for (int c0 = 0; c0 < BN; c0 += 16) {
+    for (int c0 = 16 * (warp >> 2); c0 < BN; c0 += 16 * (kWarps / 4)) {
         uint32_t r[16];
-        const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
+        const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c0;
         asm volatile(
             "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
             "%14, %15}, [%16];"
@@ -341,17 +347,17 @@ int gemm_bf16(const void *A, const void *B, int M, int N, int K, const GemmEpi &
     dim3 grid(N / BN, (M + BM - 1) / BM);
     const bool deep = (long)grid.x * grid.y <= sm_count() && K / BK > 4;  // one wave: the deep ring
     if (BN == 256) {
-        gemm_bf16_tc_kernel<256, 4><<<grid, 128, smem_bytes<256, 4>(), st>>>(ma, mb, g, M, N, K, status);
+        gemm_bf16_tc_kernel<256, 4><<<grid, 32 * kWarps, smem_bytes<256, 4>(), st>>>(ma, mb, g, M, N, K, status);
     } else if (BN == 128) {
-        if (deep) gemm_bf16_tc_kernel<128, 6><<<grid, 128, smem_bytes<128, 6>(), st>>>(ma, mb, g, M, N, K, status);
-        else gemm_bf16_tc_kernel<128, 4><<<grid, 128, smem_bytes<128, 4>(), st>>>(ma, mb, g, M, N, K, status);
+        if (deep) gemm_bf16_tc_kernel<128, 6><<<grid, 32 * kWarps, smem_bytes<128, 6>(), st>>>(ma, mb, g, M, N, K, status);
+        else gemm_bf16_tc_kernel<128, 4><<<grid, 32 * kWarps, smem_bytes<128, 4>(), st>>>(ma, mb, g, M, N, K, status);
     } else {
         // long K: stages of two 64-wide K boxes (4 of them), half the k-steps (each
         // step's round trip through the ring costs more than its bytes there)
         if (deep && K % (2 * BK) == 0 && K / BK >= 32)
-            gemm_bf16_tc_kernel<64, 4, 2><<<grid, 128, smem_bytes<64, 4, 2>(), st>>>(ma, mb, g, M, N, K, status);
-        else if (deep) gemm_bf16_tc_kernel<64, 8><<<grid, 128, smem_bytes<64, 8>(), st>>>(ma, mb, g, M, N, K, status);
-        else gemm_bf16_tc_kernel<64, 4><<<grid, 128, smem_bytes<64, 4>(), st>>>(ma, mb, g, M, N, K, status);
+            gemm_bf16_tc_kernel<64, 4, 2><<<grid, 32 * kWarps, smem_bytes<64, 4, 2>(), st>>>(ma, mb, g, M, N, K, status);
+        else if (deep) gemm_bf16_tc_kernel<64, 8><<<grid, 32 * kWarps, smem_bytes<64, 8>(), st>>>(ma, mb, g, M, N, K, status);
+        else gemm_bf16_tc_kernel<64, 4><<<grid, 32 * kWarps, smem_bytes<64, 4>(), st>>>(ma, mb, g, M, N, K, status);
     }
     return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
