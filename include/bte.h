@@ -57,7 +57,7 @@ typedef enum {
 } bte_status;
 
 typedef enum {
-    BTE_FP64_PLAIN = 0,   /* plain FP64 operator: direct sums, FP64 weights     */
+    BTE_FP64_PLAIN = 0,   /* FP64 throughout: FFTs, direct weighted sums        */
     BTE_FP32 = 1,         /* FP32 compensated convolution, FP64 projection      */
     BTE_LEARNED = 2       /* MLP surrogate + FP64 projection + exact fallback   */
 } bte_mode;
