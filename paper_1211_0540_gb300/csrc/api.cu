@@ -651,7 +651,7 @@ bte_status enqueue_collide(bte_ctx *c, Batch *B, const double *f, double *Q, int
                 count_launches(c, launch_dft_forward(f, B->d_slot_off, ds, sf, c->scratch[SC_T1], c->scratch[SC_F],
                                                      fp64 && by_cells64(sg), c->d_status, st));
             else {
-                launch_dft_forward_fused(f, B->d_slot_off, ds, t->d_root32, sf, (float2 *)c->scratch[SC_F], c->d_status,
+                launch_dft_forward_fused(f, B->d_slot_off, ds, sf, (float2 *)c->scratch[SC_F], c->d_status,
                                          st, cfg.split);
                 count_launches(c, 1);
             }
@@ -735,14 +735,14 @@ bte_status enqueue_collide(bte_ctx *c, Batch *B, const double *f, double *Q, int
         const double si = std::pow(2.0 * kPi, -1.5) * t->dz * t->dz * t->dz;
         if (fuse & FUSE_NEXT_FWD) {  // post == POST_STAGE1 (checked by the caller)
             const double sf = std::pow(2.0 * kPi, -1.5) * t->dv * t->dv * t->dv;
-            launch_dft_inverse_forward_fused((const float2 *)c->scratch[SC_QH], B->d_slot_off, ds, t->d_root32, si,
+            launch_dft_inverse_forward_fused((const float2 *)c->scratch[SC_QH], B->d_slot_off, ds, si,
                                              Q, proj_args(t), x, a, sf, (float2 *)c->scratch[SC_F], c->d_status, st,
                                              cfg.split);
             count_launches(c, 1);
             continue;
         }
         if (!fp64 && fused_dft_supported(t->N)) {
-            launch_dft_inverse_fused((const float2 *)c->scratch[SC_QH], B->d_slot_off, ds, t->d_root32, si, Q,
+            launch_dft_inverse_fused((const float2 *)c->scratch[SC_QH], B->d_slot_off, ds, si, Q,
                                      proj_args(t), post, x, y, qp, a, st, cfg.split);
             count_launches(c, 1);
             continue;
@@ -925,7 +925,7 @@ bte_status enqueue_indicator(bte_ctx *c, Batch *B, const double *f, const double
     // sector order; one CTA per cell once the cells fill the SMs (the fastest for
     // this transform alone), else the batch's tuned split
     const int split = B->nslots >= c->num_sms ? 1 : cfg_of(c, B).split;
-    launch_dft_forward_fused(f, B->d_slot_off, ds, t->d_root32, sf, (float2 *)c->scratch[SC_F], c->d_status, st,
+    launch_dft_forward_fused(f, B->d_slot_off, ds, sf, (float2 *)c->scratch[SC_F], c->d_status, st,
                              split, true);
     launch_dft_forward_pencils(Q, B->d_slot_off, ds, sf, c->ind->d_kk, c->ind->S, (float2 *)c->scratch[SC_QH],
                                c->d_status, st);  // only the sampled pencils are compared
@@ -1038,7 +1038,7 @@ bte_status enqueue_learned(bte_ctx *c, Batch *B, const double *f, double *Q, uns
     DftSeg ds{t->N, 0, B->nslots, 0};
     const double sf = std::pow(2.0 * kPi, -1.5) * t->dv * t->dv * t->dv;
     const double si = std::pow(2.0 * kPi, -1.5) * t->dz * t->dz * t->dz;
-    launch_dft_forward_fused(f, fa.off, ds, t->d_root32, sf, (float2 *)c->scratch[SC_F], c->d_status, st, cfg.split);
+    launch_dft_forward_fused(f, fa.off, ds, sf, (float2 *)c->scratch[SC_F], c->d_status, st, cfg.split);
     ConvLaunch L;
     cudaError_t e = conv32_configure(t->kinds_mask(), c->num_sms, cfg.warps, cfg.stages, cfg.impl, &L);
     if (e != cudaSuccess) return cuda_fail(c, e, "learned mode: convolution configuration");
@@ -1062,7 +1062,7 @@ bte_status enqueue_learned(bte_ctx *c, Batch *B, const double *f, double *Q, uns
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(c, e, "learned mode: launch");
     if ((e = conv32_launch(L, p, st)) != cudaSuccess) return cuda_fail(c, e, "learned mode: convolution launch");
-    launch_dft_inverse_fused((const float2 *)c->scratch[SC_QH], fa.off, ds, t->d_root32, si, Q, proj_args(t),
+    launch_dft_inverse_fused((const float2 *)c->scratch[SC_QH], fa.off, ds, si, Q, proj_args(t),
                              POST_PROJECT, nullptr, nullptr, nullptr, 0.0, st, cfg.split);
     count_launches(c, 4);
     e = cudaGetLastError();

@@ -160,7 +160,7 @@ __device__ __forceinline__ void load_pencil_f64(const double *__restrict__ fp, f
 template <int N, int C_, bool SECTOR = false>
 __global__ void __cluster_dims__(C_, 1, 1) __launch_bounds__(FusedShape<N, C_>::NT)
 dft_fwd_fused_kernel(const double *__restrict__ f, const int64_t *__restrict__ slot_off, DftSeg s,
-                     const float2 *__restrict__ root, float scale, float2 *__restrict__ G, int *status) {
+                     float scale, float2 *__restrict__ G, int *status) {
     using S = FusedShape<N, C_>;
     constexpr int M = S::M, NN = S::NN, P = S::P, JR = S::JR, C = S::C;
     cg::cluster_group cl = cg::this_cluster();
@@ -299,7 +299,7 @@ dft_fwd_pencils_kernel(const double *__restrict__ f, const int64_t *__restrict__
 template <int N, int C_, bool FWD = false, bool UPD = true>
 __global__ void __cluster_dims__(C_, 1, 1) __launch_bounds__(FusedShape<N, C_>::NT)
 dft_inv_fused_kernel(const float2 *__restrict__ G, const int64_t *__restrict__ slot_off, DftSeg s,
-                     const float2 *__restrict__ root, float scale, double *__restrict__ q, ProjArgs pa,
+                     float scale, double *__restrict__ q, ProjArgs pa,
                      int mode, const double *__restrict__ x, double *__restrict__ y,
                      const double *__restrict__ qp, double a, float2 *__restrict__ Gout = nullptr,
                      float fscale = 0.f, int *status = nullptr) {
@@ -541,38 +541,38 @@ namespace {
 // cell-major: the padding slots have nothing to write
 int grid_slots(const DftSeg &s) { return s.cells ? s.nvalid : s.nslots; }
 template <int N, int C>
-void fwd_launch(const double *f, const int64_t *slot_off, const DftSeg &s, const float2 *root, double scale,
+void fwd_launch(const double *f, const int64_t *slot_off, const DftSeg &s, double scale,
                 float2 *G, int *status, cudaStream_t st, bool sector) {
     using S = FusedShape<N, C>;
     if constexpr (N <= 16) {
         if (sector) {
-            dft_fwd_fused_kernel<N, C, true><<<s.nslots * C, S::NT, S::smem_fwd, st>>>(f, slot_off, s, root,
-                                                                                      (float)scale, G, status);
+            dft_fwd_fused_kernel<N, C, true><<<s.nslots * C, S::NT, S::smem_fwd, st>>>(f, slot_off, s, (float)scale, G,
+                                                                                      status);
             return;
         }
     }
-    dft_fwd_fused_kernel<N, C><<<grid_slots(s) * C, S::NT, S::smem_fwd, st>>>(f, slot_off, s, root, (float)scale, G,
+    dft_fwd_fused_kernel<N, C><<<grid_slots(s) * C, S::NT, S::smem_fwd, st>>>(f, slot_off, s, (float)scale, G,
                                                                         status);
 }
 template <int N, int C>
-void inv_launch(const float2 *G, const int64_t *slot_off, const DftSeg &s, const float2 *root, double scale,
+void inv_launch(const float2 *G, const int64_t *slot_off, const DftSeg &s, double scale,
                 double *q, const ProjArgs &pa, int mode, const double *x, double *y, const double *qp, double a,
                 cudaStream_t st) {
     using S = FusedShape<N, C>;
     if (mode >= 2)
-        dft_inv_fused_kernel<N, C><<<grid_slots(s) * C, S::NT, S::smem_inv, st>>>(G, slot_off, s, root, (float)scale, q,
+        dft_inv_fused_kernel<N, C><<<grid_slots(s) * C, S::NT, S::smem_inv, st>>>(G, slot_off, s, (float)scale, q,
                                                                                  pa, mode, x, y, qp, a);
     else
         dft_inv_fused_kernel<N, C, false, false><<<grid_slots(s) * C, S::NT, S::smem_inv_proj, st>>>(
-            G, slot_off, s, root, (float)scale, q, pa, mode, x, y, qp, a);
+            G, slot_off, s, (float)scale, q, pa, mode, x, y, qp, a);
 }
 template <int N, int C>
-void inv_fwd_launch(const float2 *G, const int64_t *slot_off, const DftSeg &s, const float2 *root, double scale,
+void inv_fwd_launch(const float2 *G, const int64_t *slot_off, const DftSeg &s, double scale,
                     double *q, const ProjArgs &pa, const double *x, double a, double fscale, float2 *Gout,
                     int *status, cudaStream_t st) {
     using S = FusedShape<N, C>;
     dft_inv_fused_kernel<N, C, true><<<grid_slots(s) * C, S::NT, S::smem_inv, st>>>(
-        G, slot_off, s, root, (float)scale, q, pa, 2, x, nullptr, nullptr, a, Gout, (float)fscale, status);
+        G, slot_off, s, (float)scale, q, pa, 2, x, nullptr, nullptr, a, Gout, (float)fscale, status);
 }
 template <int N, int C>
 void prepare_one() {
@@ -619,7 +619,7 @@ bool fused_dft_supported(int N) { return N == 8 || N == 12 || N == 16 || N == 24
 void fused_dft_prepare(int N) {
     // roots of unity (constant memory is per device) and shared-memory
     // attributes; must happen outside stream capture
-    static std::map<int, unsigned> done;  // device -> bit N of the uploaded root tables
+    static std::map<int, unsigned> done;  // device -> bit N of the uploaded roots
     static std::mutex mu;                   // contexts on several host threads share the map
     std::lock_guard<std::mutex> lock(mu);
     int dev = 0;
@@ -659,34 +659,34 @@ void launch_dft_forward_pencils(const double *f, const int64_t *slot_off, const 
     }
 }
 
-void launch_dft_forward_fused(const double *f, const int64_t *slot_off, const DftSeg &s, const float2 *root,
-                              double scale, float2 *G, int *status, cudaStream_t st, int split, bool sector) {
+void launch_dft_forward_fused(const double *f, const int64_t *slot_off, const DftSeg &s, double scale, float2 *G,
+                              int *status, cudaStream_t st, int split, bool sector) {
     switch (s.N) {
-        case 8: BTE_SPLIT_DISPATCH(fwd_launch, 8, f, slot_off, s, root, scale, G, status, st, sector) break;
-        case 12: BTE_SPLIT_DISPATCH(fwd_launch, 12, f, slot_off, s, root, scale, G, status, st, sector) break;
-        case 16: BTE_SPLIT_DISPATCH(fwd_launch, 16, f, slot_off, s, root, scale, G, status, st, sector) break;
-        case 24: fwd_launch<24, 4>(f, slot_off, s, root, scale, G, status, st, false); break;
-        case 32: fwd_launch<32, 8>(f, slot_off, s, root, scale, G, status, st, false); break;
+        case 8: BTE_SPLIT_DISPATCH(fwd_launch, 8, f, slot_off, s, scale, G, status, st, sector) break;
+        case 12: BTE_SPLIT_DISPATCH(fwd_launch, 12, f, slot_off, s, scale, G, status, st, sector) break;
+        case 16: BTE_SPLIT_DISPATCH(fwd_launch, 16, f, slot_off, s, scale, G, status, st, sector) break;
+        case 24: fwd_launch<24, 4>(f, slot_off, s, scale, G, status, st, false); break;
+        case 32: fwd_launch<32, 8>(f, slot_off, s, scale, G, status, st, false); break;
         default: break;
     }
 }
 
-void launch_dft_inverse_fused(const float2 *G, const int64_t *slot_off, const DftSeg &s, const float2 *root,
-                              double scale, double *q, const ProjArgs &pa, int mode, const double *x, double *y,
+void launch_dft_inverse_fused(const float2 *G, const int64_t *slot_off, const DftSeg &s, double scale, double *q,
+                              const ProjArgs &pa, int mode, const double *x, double *y,
                               const double *qp, double a, cudaStream_t st, int split) {
     switch (s.N) {
-        case 8: BTE_SPLIT_DISPATCH(inv_launch, 8, G, slot_off, s, root, scale, q, pa, mode, x, y, qp, a, st) break;
-        case 12: BTE_SPLIT_DISPATCH(inv_launch, 12, G, slot_off, s, root, scale, q, pa, mode, x, y, qp, a, st) break;
-        case 16: BTE_SPLIT_DISPATCH(inv_launch, 16, G, slot_off, s, root, scale, q, pa, mode, x, y, qp, a, st) break;
-        case 24: inv_launch<24, 4>(G, slot_off, s, root, scale, q, pa, mode, x, y, qp, a, st); break;
-        case 32: inv_launch<32, 8>(G, slot_off, s, root, scale, q, pa, mode, x, y, qp, a, st); break;
+        case 8: BTE_SPLIT_DISPATCH(inv_launch, 8, G, slot_off, s, scale, q, pa, mode, x, y, qp, a, st) break;
+        case 12: BTE_SPLIT_DISPATCH(inv_launch, 12, G, slot_off, s, scale, q, pa, mode, x, y, qp, a, st) break;
+        case 16: BTE_SPLIT_DISPATCH(inv_launch, 16, G, slot_off, s, scale, q, pa, mode, x, y, qp, a, st) break;
+        case 24: inv_launch<24, 4>(G, slot_off, s, scale, q, pa, mode, x, y, qp, a, st); break;
+        case 32: inv_launch<32, 8>(G, slot_off, s, scale, q, pa, mode, x, y, qp, a, st); break;
         default: break;
     }
 }
 bool inverse_forward_fused_supported(int N, int) { return fused_dft_supported(N); }
 
 void launch_dft_inverse_forward_fused(const float2 *G, const int64_t *slot_off, const DftSeg &s,
-                                      const float2 *root, double scale, double *q, const ProjArgs &pa,
+                                      double scale, double *q, const ProjArgs &pa,
                                       const double *x, double a, double fscale, float2 *Gout, int *status,
                                       cudaStream_t st, int split) {
     switch (s.N) {
@@ -695,24 +695,24 @@ void launch_dft_inverse_forward_fused(const float2 *G, const int64_t *slot_off, 
         case 16:
             switch (norm_split(split, s)) {
                 case 1:
-                    if (s.N == 8) inv_fwd_launch<8, 1>(G, slot_off, s, root, scale, q, pa, x, a, fscale, Gout, status, st);
-                    else if (s.N == 12) inv_fwd_launch<12, 1>(G, slot_off, s, root, scale, q, pa, x, a, fscale, Gout, status, st);
-                    else inv_fwd_launch<16, 1>(G, slot_off, s, root, scale, q, pa, x, a, fscale, Gout, status, st);
+                    if (s.N == 8) inv_fwd_launch<8, 1>(G, slot_off, s, scale, q, pa, x, a, fscale, Gout, status, st);
+                    else if (s.N == 12) inv_fwd_launch<12, 1>(G, slot_off, s, scale, q, pa, x, a, fscale, Gout, status, st);
+                    else inv_fwd_launch<16, 1>(G, slot_off, s, scale, q, pa, x, a, fscale, Gout, status, st);
                     break;
                 case 2:
-                    if (s.N == 8) inv_fwd_launch<8, 2>(G, slot_off, s, root, scale, q, pa, x, a, fscale, Gout, status, st);
-                    else if (s.N == 12) inv_fwd_launch<12, 2>(G, slot_off, s, root, scale, q, pa, x, a, fscale, Gout, status, st);
-                    else inv_fwd_launch<16, 2>(G, slot_off, s, root, scale, q, pa, x, a, fscale, Gout, status, st);
+                    if (s.N == 8) inv_fwd_launch<8, 2>(G, slot_off, s, scale, q, pa, x, a, fscale, Gout, status, st);
+                    else if (s.N == 12) inv_fwd_launch<12, 2>(G, slot_off, s, scale, q, pa, x, a, fscale, Gout, status, st);
+                    else inv_fwd_launch<16, 2>(G, slot_off, s, scale, q, pa, x, a, fscale, Gout, status, st);
                     break;
                 default:
-                    if (s.N == 8) inv_fwd_launch<8, 4>(G, slot_off, s, root, scale, q, pa, x, a, fscale, Gout, status, st);
-                    else if (s.N == 12) inv_fwd_launch<12, 4>(G, slot_off, s, root, scale, q, pa, x, a, fscale, Gout, status, st);
-                    else inv_fwd_launch<16, 4>(G, slot_off, s, root, scale, q, pa, x, a, fscale, Gout, status, st);
+                    if (s.N == 8) inv_fwd_launch<8, 4>(G, slot_off, s, scale, q, pa, x, a, fscale, Gout, status, st);
+                    else if (s.N == 12) inv_fwd_launch<12, 4>(G, slot_off, s, scale, q, pa, x, a, fscale, Gout, status, st);
+                    else inv_fwd_launch<16, 4>(G, slot_off, s, scale, q, pa, x, a, fscale, Gout, status, st);
                     break;
             }
             break;
-        case 24: inv_fwd_launch<24, 4>(G, slot_off, s, root, scale, q, pa, x, a, fscale, Gout, status, st); break;
-        case 32: inv_fwd_launch<32, 8>(G, slot_off, s, root, scale, q, pa, x, a, fscale, Gout, status, st); break;
+        case 24: inv_fwd_launch<24, 4>(G, slot_off, s, scale, q, pa, x, a, fscale, Gout, status, st); break;
+        case 32: inv_fwd_launch<32, 8>(G, slot_off, s, scale, q, pa, x, a, fscale, Gout, status, st); break;
         default: break;
     }
 }

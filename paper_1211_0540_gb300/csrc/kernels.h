@@ -130,11 +130,10 @@ __host__ __device__ __forceinline__ int64_t sector_index(int64_t e, int lane) {
 // instead of 4 where the cells alone fill the SMs);
 // sector: fhat in the sector order (N <= 16) instead of the convolution's
 // group layout
-void launch_dft_forward_fused(const double *f, const int64_t *slot_off, const DftSeg &s, const float2 *root,
-                              double scale, float2 *G, int *status, cudaStream_t st, int split = 4,
-                              bool sector = false);
-void launch_dft_inverse_fused(const float2 *G, const int64_t *slot_off, const DftSeg &s, const float2 *root,
-                              double scale, double *q, const ProjArgs &pa, int mode, const double *x, double *y,
+void launch_dft_forward_fused(const double *f, const int64_t *slot_off, const DftSeg &s, double scale, float2 *G,
+                              int *status, cudaStream_t st, int split = 4, bool sector = false);
+void launch_dft_inverse_fused(const float2 *G, const int64_t *slot_off, const DftSeg &s, double scale, double *q,
+                              const ProjArgs &pa, int mode, const double *x, double *y,
                               const double *qp, double a, cudaStream_t st, int split = 4);
 // The first Heun stage's inverse (mode 2: Q = P Qt into q) fused with the second
 // stage's forward transform: f* = x + a Q is not stored; fhat(f*) (times fscale)
@@ -142,7 +141,7 @@ void launch_dft_inverse_fused(const float2 *G, const int64_t *slot_off, const Df
 // by launch_dft_forward_fused on f*. Supported wherever the fused transforms are.
 bool inverse_forward_fused_supported(int N, int split);
 void launch_dft_inverse_forward_fused(const float2 *G, const int64_t *slot_off, const DftSeg &s,
-                                      const float2 *root, double scale, double *q, const ProjArgs &pa,
+                                      double scale, double *q, const ProjArgs &pa,
                                       const double *x, double a, double fscale, float2 *Gout, int *status,
                                       cudaStream_t st, int split = 4);
 

@@ -285,13 +285,6 @@ int build_table(Table &t, std::string &err) {
     for (int a = 0; a < 5; ++a)
         for (int b = 0; b < 5; ++b) t.ainv[a * 5 + b] = (a < nr && b < nr) ? Ai[a][b + nr] : 0.0;
 
-    // DFT roots exp(2 pi i t / N)
-    std::vector<float2> r32(N);
-    for (int s = 0; s < N; ++s) {
-        double c = std::cos(2.0 * kPi * s / N), sn = std::sin(2.0 * kPi * s / N);
-        r32[s] = make_float2((float)c, (float)sn);
-    }
-
     // one group's work items, costliest first (stable, so ties keep (tile, k1, k2) order)
     std::vector<ConvItem> tmpl;
     std::vector<uint64_t> tcost;
@@ -379,7 +372,6 @@ int build_table(Table &t, std::string &err) {
     if (e == cudaSuccess && ne) e = cudaMalloc(&t.d_ent, sizeof(uint16_t) * ent.size());
     if (e == cudaSuccess && ne) e = cudaMalloc(&t.d_rk, sizeof(int16_t) * rk.size());
     if (e == cudaSuccess) e = cudaMalloc(&t.d_desc, sizeof(uint32_t) * std::max<size_t>(t.n_desc, 1));
-    if (e == cudaSuccess) e = cudaMalloc(&t.d_root32, sizeof(float2) * N);
     if (e != cudaSuccess) {
         err = std::string("cudaMalloc (weight table): ") + cudaGetErrorString(e);
         free_table(t);
@@ -399,7 +391,6 @@ int build_table(Table &t, std::string &err) {
         e = cudaMemcpy(t.d_etab, etab.data(), sizeof(uint16_t) * etab.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = cudaMemcpy(t.d_desc, desc.data(), sizeof(uint32_t) * t.n_desc, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(t.d_root32, r32.data(), sizeof(float2) * N, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         err = std::string("cudaMemcpy (weight table): ") + cudaGetErrorString(e);
         free_table(t);
@@ -545,12 +536,10 @@ void free_table(Table &t) {
     cudaFree(t.d_desc);
     cudaFree(t.d_w64);
     cudaFree(t.d_zeta64);
-    cudaFree(t.d_root32);
     t.d_w32 = nullptr;
     t.d_desc = nullptr;
     t.d_w64 = nullptr;
     t.d_zeta64 = nullptr;
-    t.d_root32 = nullptr;
 }
 
 }  // namespace bte
