@@ -59,6 +59,26 @@ struct Kind {
             for (int t = 0; t < (v == i ? j : T); ++t) c += pair_visit(K0 + t, v, N, T);
         return c;
     }
+    static constexpr int first_visit(int j) {  // the visit that holds output j's first pair
+        int i = 0;
+        while (!pair_visit(K0 + j, i, N, T)) ++i;
+        return i;
+    }
+    // The most blocks that a plain sum runs over before a TwoSum merge (fewer if
+    // ConvParams::merge says so), and whether variants 4 and 5 sum every block by itself
+    // and add those instead. A mode and its mirror are one sum here, so their roundings
+    // do not average; the limits keep the operator's error within that of the full
+    // spectrum's sums merged every 16 blocks. Error relative to that one, merged every
+    // 16 / 8 / 4 / 2 / 1 blocks, 128 to 2048 cells: N = 8 1.07 / 1.06 / 1.05 / 1.03 / 0.99,
+    // N = 12 1.12 / 1.08 / 1.05 / 0.98, N = 16 1.08 / 1.05 / 1.01 / 0.95 / 0.89 (every 3:
+    // 0.96), N = 24 1.05 / 1.01 / 0.98, N = 32 1.06 / 1.02 / 0.97; with block sums 0.96, 0.91 and
+    // 0.92 at N = 12, 24, 32. Block sums cost 16 additions a block and registers: a collide of 1024
+    // cells N = 12 176 (every 16) -> 181 us (every 2: 191), 128 cells N = 24 869 -> 875 us
+    // and N = 32 4.39 -> 4.63 ms (every 4: 4.70). N = 16 has no registers left for them
+    // (1024 cells 638 -> 706 us; merges every 3 blocks 667), N = 8 needs a merge every block
+    // (2048 cells 73 -> 80 us). N = 48 is within the bound at 16.
+    static constexpr int merge_most = N == 8 ? 1 : N == 12 ? 2 : N == 16 ? 3 : N == 48 ? 1 << 20 : 4;
+    static constexpr bool block_sums = N == 12 || N == 24 || N == 32;
     static constexpr int cpad = (count() + 3) & ~3;
     static constexpr int row_bytes = N * kLanes * 8;
     static constexpr int stage_bytes = 2 * row_bytes + cpad * 4;
@@ -85,7 +105,8 @@ __device__ __forceinline__ void static_for(F &&f) {
 }
 
 // The pairs of a block in the order of its weights: begin(m3) at each visit,
-// then pair(j, n3, w) for every output j of the tile that has one. All indices
+// then pair(j, n3, w, first) for every output j of the tile that has one, first at the
+// output's first pair. All indices
 // are compile-time constants; the weights are read four at a time. Plain
 // unrolled loops where the tile holds every output (N <= 16); wider grids
 // unroll by recursion, since the compiler leaves loops of that size rolled
@@ -107,7 +128,7 @@ __device__ __forceinline__ void for_pairs(const float4 *W4, Begin &&begin, Pair 
                     if ((wi & 3) == 0) w4 = W4[wi >> 2];
                     const float w = (wi & 3) == 0 ? w4.x : (wi & 3) == 1 ? w4.y : (wi & 3) == 2 ? w4.z : w4.w;
                     ++wi;
-                    pair(j, pair_partner(j, m3, K::N), w);
+                    pair(j, pair_partner(j, m3, K::N), w, m3 == K::first_visit(j));
                 }
         }
     } else {
@@ -121,7 +142,8 @@ __device__ __forceinline__ void for_pairs(const float4 *W4, Begin &&begin, Pair 
                     constexpr int wi = K::rank(i, j);
                     if constexpr ((wi & 3) == 0) w4 = W4[wi >> 2];
                     pair(j, pair_partner(K::K0 + j, m3, K::N),
-                         (wi & 3) == 0 ? w4.x : (wi & 3) == 1 ? w4.y : (wi & 3) == 2 ? w4.z : w4.w);
+                         (wi & 3) == 0 ? w4.x : (wi & 3) == 1 ? w4.y : (wi & 3) == 2 ? w4.z : w4.w,
+                         i == K::first_visit(j));
                 }
             });
         });
@@ -136,7 +158,7 @@ __device__ __forceinline__ void conv_block(const char *st, int lane, float (&par
     float2 a;
     for_pairs<K>(
         reinterpret_cast<const float4 *>(B + K::N * kLanes), [&](int m3) { a = A[m3 * kLanes + lane]; },
-        [&](int j, int n3, float w) {
+        [&](int j, int n3, float w, bool) {
             const float2 b = B[n3 * kLanes + lane];
             const float tr = w * a.x, ti = w * a.y;
             part[2 * j] = fmaf(tr, b.x, part[2 * j]);
@@ -262,6 +284,7 @@ __device__ bool conv_item(WarpRing &r, const ConvItem &it, const ConvParams &p, 
     for (int i = 0; i < 2 * K::T; ++i) part[i] = hi[i] = lo[i] = 0.f;
 
     int since = 0;
+    const int merge = min(p.merge, K::merge_most);
     bool ok = true;
     int j = 0;
     for (; j < nb; ++j) {
@@ -275,7 +298,7 @@ __device__ bool conv_item(WarpRing &r, const ConvItem &it, const ConvParams &p, 
         }
         r.phase ^= (1u << s);
         conv_block<K>(r.base + s * r.stage_bytes, lane, part);
-        if (++since == p.merge || j == nb - 1) {
+        if (++since == merge || j == nb - 1) {
             since = 0;
 #pragma unroll
             for (int i = 0; i < 2 * K::T; ++i) {  // TwoSum(hi, part)
@@ -379,13 +402,24 @@ __device__ __forceinline__ uint64_t fmul2(uint64_t a, uint64_t b) {
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
+__device__ __forceinline__ uint64_t fadd2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t fsub2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
 __device__ __forceinline__ uint64_t ffma2(uint64_t a, uint64_t b, uint64_t c) {
     uint64_t d;
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
     return d;
 }
 
-template <class K>
+// FRESH: part becomes the block's sums; else they are added to it.
+template <class K, bool FRESH>
 __device__ __forceinline__ void conv_block_packed(const char *st, int lane, uint64_t (&part)[K::T]) {
     const float2 *A = reinterpret_cast<const float2 *>(st);
     const float2 *B = A + K::N * kLanes;
@@ -397,11 +431,11 @@ __device__ __forceinline__ void conv_block_packed(const char *st, int lane, uint
             aR = pk2(a.x, a.x);
             aI = pk2(a.y, a.y);
         },
-        [&](int j, int n3, float w) {
+        [&](int j, int n3, float w, bool first) {
             const float2 b = B[n3 * kLanes + lane];
             uint64_t pr = fmul2(aR, pk2(b.x, b.y));
             pr = ffma2(aI, pk2(-b.y, b.x), pr);
-            part[j] = ffma2(pk2(w, w), pr, part[j]);
+            part[j] = FRESH && first ? fmul2(pk2(w, w), pr) : ffma2(pk2(w, w), pr, part[j]);
         });
 }
 
@@ -434,6 +468,7 @@ __device__ bool coop_item(WarpRing &r, const ConvItem &it, const ConvParams &p, 
     for (int i = 0; i < T; ++i) pp[i] = 0ull;
 
     bool ok = true;
+    const int merge = min(p.merge, K::merge_most);
     int since = 0, i = 0;
     for (; i < mine; ++i) {
         const int s = i % S;
@@ -444,9 +479,9 @@ __device__ bool coop_item(WarpRing &r, const ConvItem &it, const ConvParams &p, 
             break;
         }
         r.phase ^= (1u << s);
-        if (PACKED) conv_block_packed<K>(r.base + s * r.stage_bytes, lane, pp);
+        if (PACKED) conv_block_packed<K, false>(r.base + s * r.stage_bytes, lane, pp);
         else conv_block<K>(r.base + s * r.stage_bytes, lane, part);
-        if (++since == p.merge || i == mine - 1) {
+        if (++since == merge || i == mine - 1) {
             since = 0;
             if (PACKED) {
 #pragma unroll
@@ -475,12 +510,12 @@ __device__ bool coop_item(WarpRing &r, const ConvItem &it, const ConvParams &p, 
         }
         __syncwarp();
     }
-    // partial sums of this warp into its own (drained) ring: [4T][32] floats
-    float *red = reinterpret_cast<float *>(r.base);
+    // partial sums of this warp into its own (drained) ring: (hi, lo)[T][32] (re, im)
+    float2 *red = reinterpret_cast<float2 *>(r.base);
 #pragma unroll
-    for (int q = 0; q < 2 * T; ++q) {
-        red[q * kLanes + lane] = hi[q];
-        red[(2 * T + q) * kLanes + lane] = lo[q];
+    for (int t = 0; t < T; ++t) {
+        red[t * kLanes + lane] = make_float2(hi[2 * t], hi[2 * t + 1]);
+        red[(T + t) * kLanes + lane] = make_float2(lo[2 * t], lo[2 * t + 1]);
     }
     return ok;
 }
@@ -494,11 +529,12 @@ __device__ __forceinline__ void coop_reduce(const ConvItem &it, const ConvParams
     for (int t = warp; t < T; t += nwarps) {
         float sr = 0.f, lr = 0.f, si = 0.f, li = 0.f;
         for (int w = 0; w < nwarps; ++w) {
-            const float *red = reinterpret_cast<const float *>(ring0 + (size_t)w * warp_smem + sums_off);
-            two_sum(sr, lr, red[(2 * t) * kLanes + lane]);
-            lr += red[(2 * T + 2 * t) * kLanes + lane];
-            two_sum(si, li, red[(2 * t + 1) * kLanes + lane]);
-            li += red[(2 * T + 2 * t + 1) * kLanes + lane];
+            const float2 *red = reinterpret_cast<const float2 *>(ring0 + (size_t)w * warp_smem + sums_off);
+            const float2 h = red[t * kLanes + lane], l = red[(T + t) * kLanes + lane];
+            two_sum(sr, lr, h.x);
+            lr += l.x;
+            two_sum(si, li, h.y);
+            li += l.y;
         }
         Q[t * kLanes] = make_float2(sr + lr, si + li);
     }
@@ -529,7 +565,7 @@ __device__ __forceinline__ bool coop_run(WarpRing &r, const ConvItem &it, const 
 // instructions and the (w, w) operand only. One-block rings keep 3 CTAs per
 // SM (4 warps x (one 8.75 KB stage + 8 KB of sums) at N = 16).
 // ---------------------------------------------------------------------------
-template <class K>
+template <class K, bool FRESH>
 __device__ __forceinline__ void conv_block_packed_h(const char *st, int lane, uint64_t (&part)[K::T]) {
     const float2 *A = reinterpret_cast<const float2 *>(st);
     const float2 *B = A + K::N * kLanes;
@@ -548,14 +584,14 @@ __device__ __forceinline__ void conv_block_packed_h(const char *st, int lane, ui
             aR = pk2(a.x, a.x);
             aI = pk2(a.y, a.y);
         },
-        [&](int j, int n3, float w) {
+        [&](int j, int n3, float w, bool first) {
             uint64_t pr = fmul2(aR, bb[n3]);
             pr = ffma2(aI, bs[n3], pr);
-            part[j] = ffma2(pk2(w, w), pr, part[j]);
+            part[j] = FRESH && first ? fmul2(pk2(w, w), pr) : ffma2(pk2(w, w), pr, part[j]);
         });
 }
 
-// Bytes of a warp's shared (hi, lo) sums: 4T x 32 floats with T <= 16.
+// Bytes of a warp's shared (hi, lo) sums, T x 32 packed (re, im) each, T <= 16.
 constexpr int kSumsBytes = 4 * 16 * kLanes * 4;
 
 // One item by all warps of the CTA, sums in shared memory at r.base + ring
@@ -577,11 +613,13 @@ __device__ bool coop_item_sm(WarpRing &r, const ConvItem &it, const ConvParams &
 #pragma unroll
     for (int q = 0; q < 4 * T; ++q) sums[q * kLanes + lane] = 0.f;
     __syncwarp();
-    uint64_t pp[T];
+    constexpr bool BS = K::block_sums;
+    uint64_t pp[T], bs[T];  // the sums since the last merge; block_sums: the block's own
 #pragma unroll
     for (int i = 0; i < T; ++i) pp[i] = 0ull;
 
     bool ok = true;
+    const int merge = BS ? p.merge : min(p.merge, K::merge_most);
     int since = 0, i = 0;
     for (; i < mine; ++i) {
         const int s = i % S;
@@ -592,21 +630,20 @@ __device__ bool coop_item_sm(WarpRing &r, const ConvItem &it, const ConvParams &
             break;
         }
         r.phase ^= (1u << s);
-        if (K::N <= 16) conv_block_packed_h<K>(r.base + s * r.stage_bytes, lane, pp);
-        else conv_block_packed<K>(r.base + s * r.stage_bytes, lane, pp);
-        if (++since == p.merge || i == mine - 1) {
+        if (K::N <= 16) conv_block_packed_h<K, BS>(r.base + s * r.stage_bytes, lane, BS ? bs : pp);
+        else conv_block_packed<K, BS>(r.base + s * r.stage_bytes, lane, BS ? bs : pp);
+        if (BS) {
+#pragma unroll
+            for (int t = 0; t < T; ++t) pp[t] = fadd2(pp[t], bs[t]);
+        }
+        if (++since == merge || i == mine - 1) {
             since = 0;
 #pragma unroll
             for (int t = 0; t < T; ++t) {
-                const float2 v = up2(pp[t]);
-                float *h = sums + (2 * t) * kLanes + lane, *l = sums + (2 * T + 2 * t) * kLanes + lane;
-                float hr = h[0], lr = l[0], hi = h[kLanes], li = l[kLanes];
-                two_sum(hr, lr, v.x);
-                two_sum(hi, li, v.y);
-                h[0] = hr;
-                l[0] = lr;
-                h[kLanes] = hi;
-                l[kLanes] = li;
+                uint64_t *h = reinterpret_cast<uint64_t *>(sums) + t * kLanes + lane, *l = h + T * kLanes;
+                const uint64_t hi = *h, sum = fadd2(hi, pp[t]), bp = fsub2(sum, hi);
+                *l = fadd2(*l, fadd2(fsub2(hi, fsub2(sum, bp)), fsub2(pp[t], bp)));
+                *h = sum;
                 pp[t] = 0ull;
             }
         }
@@ -641,11 +678,12 @@ __device__ __forceinline__ void coop_reduce_split(const ConvItem &it, const Conv
     for (int t = warp; t < T; t += nwarps) {
         float sr = 0.f, lr = 0.f, si = 0.f, li = 0.f;
         for (int w = 0; w < nwarps; ++w) {
-            const float *red = reinterpret_cast<const float *>(ring0 + (size_t)w * warp_smem + sums_off);
-            two_sum(sr, lr, red[(2 * t) * kLanes + lane]);
-            lr += red[(2 * T + 2 * t) * kLanes + lane];
-            two_sum(si, li, red[(2 * t + 1) * kLanes + lane]);
-            li += red[(2 * T + 2 * t + 1) * kLanes + lane];
+            const float2 *red = reinterpret_cast<const float2 *>(ring0 + (size_t)w * warp_smem + sums_off);
+            const float2 h = red[t * kLanes + lane], l = red[(T + t) * kLanes + lane];
+            two_sum(sr, lr, h.x);
+            lr += l.x;
+            two_sum(si, li, h.y);
+            li += l.y;
         }
         float *o = mine + (size_t)t * 4 * kLanes + lane;
         o[0] = sr;
@@ -686,11 +724,12 @@ __device__ __forceinline__ void coop_reduce_parts(const ConvItem &it, const Conv
     for (int t = warp; t < T; t += nwarps) {
         float sr = 0.f, lr = 0.f, si = 0.f, li = 0.f;
         for (int w = 0; w < nwarps; ++w) {
-            const float *red = reinterpret_cast<const float *>(ring0 + (size_t)w * warp_smem + sums_off);
-            two_sum(sr, lr, red[(2 * t) * kLanes + lane]);
-            lr += red[(2 * T + 2 * t) * kLanes + lane];
-            two_sum(si, li, red[(2 * t + 1) * kLanes + lane]);
-            li += red[(2 * T + 2 * t + 1) * kLanes + lane];
+            const float2 *red = reinterpret_cast<const float2 *>(ring0 + (size_t)w * warp_smem + sums_off);
+            const float2 h = red[t * kLanes + lane], l = red[(T + t) * kLanes + lane];
+            two_sum(sr, lr, h.x);
+            lr += l.x;
+            two_sum(si, li, h.y);
+            li += l.y;
         }
         if (sp < 0) {
             Q[t * kLanes] = make_float2(sr + lr, si + li);

@@ -126,6 +126,52 @@ __device__ __forceinline__ T *cell_smem(cg::cluster_group &cl, T *p, int rank) {
     else return cl.map_shared_rank(p, rank);
 }
 
+// N = 8 and 16: the register FFT (4 x 2 and 4 x 4) of conjugate symmetric or real data is
+// symmetric to the last bit.
+constexpr bool symmetric_fft(int N) { return N == 8 || N == 16; }
+
+// Where the passes are not symmetric, the CTAs of a cell take the k2 of the forward
+// transform's last pass in this order, mirror pairs side by side: with an even number
+// of them a CTA then holds both pencils of a pair.
+template <int N, int JR>
+__device__ __forceinline__ int last_k2(int i) {
+    if (symmetric_fft(N) || JR % 2) return i;
+    return i < 2 ? i * (N / 2) : (i & 1) ? N - i / 2 : i / 2;
+}
+
+// The cell's fhat made conjugate symmetric: y (index k1; k2 the thread's i-th of last_k2,
+// k3) becomes the mean of every mode and the conjugate of its mirror mode, which
+// another thread holds. The half-spectrum convolution takes fhat_m* for conj(fhat_m),
+// and the roundings of the passes are not symmetric: their antisymmetric part, which
+// the real part of a full spectrum's sum drops, would double there (error of the operator
+// against 64 bits, 1024 cells N = 12: 1.19 to 1.12 times that of the full spectrum's sums, before
+// the shorter merges of conv32_device.cuh). rows: the CTA's pencils, stride N + 1, free
+// at the call; for an odd number of k2 a CTA the pair's other pencil is in another
+// CTA of the cell, which the caller keeps until all have read.
+template <int N, int C, int JR>
+__device__ __forceinline__ void symmetrise(cg::cluster_group &cl, float2 *rows, bool act, int t, int r,
+                                           float2 (&y)[N]) {
+    if constexpr (!symmetric_fft(N)) {
+        constexpr int P = N + 1;
+        constexpr bool own = JR % 2 == 0;
+        if (act) {
+#pragma unroll
+            for (int k = 0; k < N; ++k) rows[t * P + k] = y[k];
+        }
+        cell_sync<own ? 1 : C>(cl);
+        if (act) {
+            const int i = r * JR + t / N, m3 = mode_mirror(t % N, N);
+            const int mi = own ? (i < 2 ? i : i ^ 1) : mode_mirror(i, N);
+            const float2 *o = cell_smem<own ? 1 : C>(cl, rows, mi / JR) + ((mi % JR) * N + m3) * P;
+#pragma unroll
+            for (int k = 0; k < N; ++k) {
+                const float2 m = o[mode_mirror(k, N)];
+                y[k] = make_float2(0.5f * (y[k].x + m.x), 0.5f * (y[k].y - m.y));
+            }
+        }
+    }
+}
+
 // The N consecutive FP64 values of a pencil, narrowed to FP32 (integer pipes),
 // with 16-byte loads when the pencil is 16-byte aligned; `bad` collects
 // non-finite inputs.
@@ -202,16 +248,20 @@ dft_fwd_fused_kernel(const double *__restrict__ f, const int64_t *__restrict__ s
         for (int k = 0; k < N; ++k) B[(jl * N + k) * N + k3] = y[k];
     }
     cell_sync<C>(cl);
-    if (act) {  // along j1, pencil (k2, k3), rows from every CTA of the cluster, into fhat's layout
-        const int k2 = r * JR + t / N, k3 = t % N;
+    float2 y[N];
+    if (act) {  // along j1, pencil (k2, k3), rows from every CTA of the cluster
+        const int k2 = last_k2<N, JR>(r * JR + t / N), k3 = t % N;
         const float2 *src[C];
 #pragma unroll
         for (int o = 0; o < C; ++o) src[o] = cell_smem<C>(cl, B, o);
-        float2 x[N], y[N];
+        float2 x[N];
 #pragma unroll
         for (int j = 0; j < N; ++j) x[j] = src[j / JR][((j % JR) * N + k2) * N + k3];
         pencil_cc<N, true>(x, y, rt);
-        const int pk = k2 * N + k3;
+    }
+    if constexpr (!SECTOR) symmetrise<N, C, JR>(cl, A, act, t, r, y);  // (the indicator sums over the full spectrum)
+    if (act) {  // into fhat's layout
+        const int pk = last_k2<N, JR>(r * JR + t / N) * N + t % N;
 #pragma unroll
         for (int k = 0; k < N; ++k) g[gi(k * NN + pk)] = make_float2(scale * y[k].x, scale * y[k].y);
     }
@@ -518,17 +568,21 @@ dft_inv_fused_kernel(const float2 *__restrict__ G, const int64_t *__restrict__ s
             for (int k = 0; k < N; ++k) Bf[(jl * N + k) * N + k3] = yy[k];
         }
         cell_sync<C>(cl);
-        if (act) {  // along j1, pencil (k2, k3), rows from every CTA of the cluster, into fhat's layout
-            const int k2 = r * JR + t / N, k3 = t % N;
+        float2 yy[N];
+        if (act) {  // along j1, pencil (k2, k3), rows from every CTA of the cluster
+            const int k2 = last_k2<N, JR>(r * JR + t / N), k3 = t % N;
             const float2 *src[C];
 #pragma unroll
             for (int o = 0; o < C; ++o) src[o] = cell_smem<C>(cl, Bf, o);
-            float2 xx[N], yy[N];
+            float2 xx[N];
 #pragma unroll
             for (int j = 0; j < N; ++j) xx[j] = src[j / JR][((j % JR) * N + k2) * N + k3];
             pencil_cc<N, true>(xx, yy, rt);
+        }
+        symmetrise<N, C, JR>(cl, Af, act, t, r, yy);
+        if (act) {  // into fhat's layout
             float2 *go = Gout + cell_base(s, sl, M);
-            const int pk = k2 * N + k3;
+            const int pk = last_k2<N, JR>(r * JR + t / N) * N + t % N;
 #pragma unroll
             for (int k = 0; k < N; ++k)
                 go[(int64_t)(k * NN + pk) * stride] = make_float2(fscale * yy[k].x, fscale * yy[k].y);
