@@ -313,8 +313,9 @@ bte_status bte_graph_count(const bte_ctx *ctx, int64_t *count);
  *                      transform (the intermediate state is not stored), bit
  *                      for bit the result of separate launches (0);
  *       "dft_split"   CTAs (one thread-block cluster) per cell in the fused
- *                      transforms of N <= 16: 1, 2 or 4 (default 4: four for
- *                      few cells, one where the cells alone fill the SMs);
+ *                      transforms of N <= 16: 1, 2 or 4 (3 is taken as 4), or 0
+ *                      (default): four for few cells, one where the cells alone
+ *                      fill the SMs;
  *       "debug_conv_stall" testing only: 1 makes every warp of the
  *                      cooperative convolution (conv_impl 1..4) skip the
  *                      copies of its first block, so that its bounded wait runs

@@ -1444,7 +1444,7 @@ bte_status bte_launch_count(const bte_ctx *c, int64_t *count) {
 
 static int *option_slot(bte_ctx *c, const char *name, int *lo, int *hi) {
     if (!std::strcmp(name, "conv_impl")) { *lo = 0; *hi = 5; return &c->conv_impl; }
-    if (!std::strcmp(name, "dft_split")) { *lo = 1; *hi = 4; return &c->dft_split; }
+    if (!std::strcmp(name, "dft_split")) { *lo = 0; *hi = 4; return &c->dft_split; }
     if (!std::strcmp(name, "debug_conv_stall")) { *lo = 0; *hi = 1; return &c->debug_conv_stall; }
     if (!std::strcmp(name, "profile_mask")) { *lo = 0; *hi = 63; return &c->prof_mask; }
     if (!std::strcmp(name, "conv_warps")) { *lo = 1; *hi = 8; return &c->conv_warps; }

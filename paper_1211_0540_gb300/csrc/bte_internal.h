@@ -169,7 +169,7 @@ struct GraphKey {
 // One configuration of the FP32 path (convolution variant and launch shape,
 // compensated-merge interval, CTAs per cell of the fused transforms).
 struct ConvCfg {
-    int impl = 4, warps = 4, stages = 0, merge = 16, split = 4;
+    int impl = 4, warps = 4, stages = 0, merge = 16, split = 0;
     int csplit = 1;   // variant 4: run the batch's split item list, or the few-cells kernel
     double ms = 0.0;  // measured time of one collide of the batch when tuned
 };
@@ -237,7 +237,7 @@ struct bte_ctx {
     int conv_merge = 16;       // blocks per compensated (TwoSum) merge
     int conv_impl = 4;         // 0 warp items, 1 CTA-cooperative, 2 cooperative + packed f32x2,
                                // 3 as 2 at 2 CTAs/SM, 4 as 2 with the compensated sums in shared memory
-    int dft_split = 4;         // CTAs per cell of the fused transforms (N <= 16)
+    int dft_split = 0;         // CTAs per cell of the fused transforms (N <= 16), 0: by the number of cells
     int conv_split = 1;        // variant 4: split items, few-cells kernel
     int dft_fuse_stages = 1;   // FP32 Heun step: stage 1's inverse transform also forms stage 2's forward
     int debug_conv_stall = 0;  // testing only: make the convolution's waits run out

@@ -647,15 +647,18 @@ void prepare_n() {
     prepare_one<N, 2>();
     prepare_one<N, 4>();
 }
-// CTAs per cell: 1 or 2 as asked; 4 (the default) while the cells are few, one
-// once they alone give about 5 warps per SM, from where it is the faster one
-// (forward + inverse, 4 against 1 CTAs per cell: N = 16, 56 cells 27.4 / 28.6 us, 128
-// 31.5 / 29.2, 1024 129.6 / 110.4; N = 12, 128 cells 25.1 / 23.1, 512 47.7 / 35.3;
+// CTAs per cell: as asked (1, 2, else 4), or with 0 (the default) four while the
+// cells are few and one once they alone give about 5 warps per SM, from where it is the
+// faster one (forward + inverse, 4 against 1 CTAs per cell: N = 16, 56 cells 27.4 / 28.6
+// us, 128 31.5 / 29.2, 1024 129.6 / 110.4; N = 12, 128 cells 25.1 / 23.1, 512 47.7 / 35.3;
 // N = 8, 256 cells 19.8 / 20.1, 1024 46.1 / 26.2).
-constexpr int kOneCtaWarps = 5 * 152;
+constexpr int kOneCtaWarps = 5;  // per SM
 int norm_split(int split, const DftSeg &s) {
-    if (split == 1 || split == 2) return split;
-    return (int64_t)grid_slots(s) * ((s.N * s.N + 31) / 32) >= kOneCtaWarps ? 1 : 4;
+    if (split != 0) return split == 1 || split == 2 ? split : 4;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return (int64_t)grid_slots(s) * ((s.N * s.N + 31) / 32) >= (int64_t)kOneCtaWarps * sms ? 1 : 4;
 }
 template <int N>
 void upload_roots(const float2 (&sym)[N]) {

@@ -126,15 +126,15 @@ void launch_dft_forward_pencils(const double *f, const int64_t *slot_off, const 
 __host__ __device__ __forceinline__ int64_t sector_index(int64_t e, int lane) {
     return ((e >> 2) << 7) + ((int64_t)lane << 2) + (e & 3);
 }
-// split: CTAs (a thread-block cluster) per cell, 1, 2 or 4 (other values: 4; one
-// instead of 4 where the cells alone fill the SMs);
+// split: CTAs (a thread-block cluster) per cell, 1, 2 or 4 (3: 4), or 0 for 4 or 1
+// by the number of cells (norm_split);
 // sector: fhat in the sector order (N <= 16) instead of the convolution's
 // group layout
 void launch_dft_forward_fused(const double *f, const int64_t *slot_off, const DftSeg &s, double scale, float2 *G,
-                              int *status, cudaStream_t st, int split = 4, bool sector = false);
+                              int *status, cudaStream_t st, int split = 0, bool sector = false);
 void launch_dft_inverse_fused(const float2 *G, const int64_t *slot_off, const DftSeg &s, double scale, double *q,
                               const ProjArgs &pa, int mode, const double *x, double *y,
-                              const double *qp, double a, cudaStream_t st, int split = 4);
+                              const double *qp, double a, cudaStream_t st, int split = 0);
 // The first Heun stage's inverse (mode 2: Q = P Qt into q) fused with the second
 // stage's forward transform: f* = x + a Q is not stored; fhat(f*) (times fscale)
 // goes to Gout in the group layout. Same results as the inverse (mode 2) followed
@@ -143,7 +143,7 @@ bool inverse_forward_fused_supported(int N, int split);
 void launch_dft_inverse_forward_fused(const float2 *G, const int64_t *slot_off, const DftSeg &s,
                                       double scale, double *q, const ProjArgs &pa,
                                       const double *x, double a, double fscale, float2 *Gout, int *status,
-                                      cudaStream_t st, int split = 4);
+                                      cudaStream_t st, int split = 0);
 
 // Transport (Sec. 3.4) on nx uniform cells of M values. mw_*: wall Maxwellians
 // per velocity (device, M doubles), den_*: sum over the incoming half of |v.n| M_w.
