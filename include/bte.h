@@ -355,7 +355,8 @@ bte_status bte_state_load(bte_ctx *ctx, const char *path, double *f, int64_t n, 
  * four CTAs per cell in the fused transforms -- times reps
  * repetitions with CUDA events on `stream`, and keeps the fastest as this
  * context's configuration for batches of the same shape (the same set of
- * grid sizes and number of 32-cell slots); it takes precedence over the
+ * grid sizes and number of 32-cell slots, and the same kernel for few cells or
+ * not); it takes precedence over the
  * options until any conv_* or dft_split option is set. f (DEVICE, read only) is
  * the input the timing runs on; results go to internal scratch. out_cfg (HOST,
  * 6 ints, optional) receives (conv_impl, conv_warps, conv_stages, conv_merge,

@@ -44,6 +44,7 @@ struct Batch {
     ConvItem *d_items_split = nullptr;
     int *d_halves = nullptr;   // the split codes as halves, when no item has more parts
     int nitems_split = 0, nsplit = 0;
+    bool few = false;          // few_cells()
     int *d_split = nullptr;
     float *d_part = nullptr;
     unsigned *d_counters = nullptr;
@@ -364,6 +365,20 @@ void plan_splits(const bte_ctx *c, const std::vector<ConvItem> &items, std::vect
     }
 }
 
+// The batch has so few cells that the FP32 convolution runs with pairs in lanes
+// (conv32_cells.cu). Its cost is proportional to the cells, one segment after the
+// other, and equals that of the kernels with cells in lanes at the limit: the shares of
+// the limit add up.
+bool few_cells(const bte_ctx *c, const Batch *B) {
+    double share = 0.0;
+    for (const Segment &sg : B->segs) {
+        const int limit = conv32_cells_limit(c->tables[sg.table]->N);
+        if (sg.nvalid > limit) return false;
+        share += (double)sg.nvalid / limit;
+    }
+    return share <= 1.0;
+}
+
 // Build (or fetch) the batch for an instance layout.
 bte_status get_batch(bte_ctx *c, const bte_instance *inst, int64_t ninst, Batch **out) {
     if (c->tables.empty()) return fail(c, BTE_ESTATE, "no weight tables: call bte_init_weights first");
@@ -450,6 +465,7 @@ bte_status get_batch(bte_ctx *c, const bte_instance *inst, int64_t ninst, Batch 
         B->n_celem += (int64_t)s.nslots * M;
         B->segs.push_back(s);
     }
+    B->few = few_cells(c, B);
     // convolution work items, costliest first
     std::vector<ConvItem> items;
     std::vector<uint64_t> cost;
@@ -530,9 +546,11 @@ bte_status get_batch(bte_ctx *c, const bte_instance *inst, int64_t ninst, Batch 
     return BTE_OK;
 }
 
-// Batch shape key of the tuning cache: the convolution kinds and the slots.
+// Batch shape key of the tuning cache: the convolution kinds and the slots, and
+// whether the cells are few, since 1 and 32 cells have as many slots but another
+// convolution kernel.
 std::string tune_key(const Batch *B) {
-    return "k" + std::to_string(B->kinds_mask) + ":s" + std::to_string(B->nslots);
+    return "k" + std::to_string(B->kinds_mask) + ":s" + std::to_string(B->nslots) + (B->few ? ":few" : "");
 }
 
 // The FP32 configuration of a batch: the autotuned one for its shape, else the options.
@@ -607,19 +625,9 @@ bte_status prepare(bte_ctx *c, Batch *B, int mode, bool step, bool transport) {
 // half full one by one (lanes over the sum instead of cells).
 bool by_cells64(const Segment &sg) { return 2 * sg.nvalid <= sg.nslots; }
 
-// The batch has so few cells that the FP32 convolution runs with pairs in lanes
-// (conv32_cells.cu), part of the split plan (conv_split 1) of variant 4. Its cost
-// is proportional to the cells, one segment after the other, and equals that of
-// the kernels with cells in lanes at the limit: the shares of the limit add up.
+// The convolution with pairs in lanes is part of the split plan (conv_split 1) of variant 4.
 bool by_cells32(const bte_ctx *c, const Batch *B, const ConvCfg &g) {
-    if (g.impl != 4 || !g.csplit || c->debug_conv_stall) return false;
-    double share = 0.0;
-    for (const Segment &sg : B->segs) {
-        const int limit = conv32_cells_limit(c->tables[sg.table]->N);
-        if (sg.nvalid > limit) return false;
-        share += (double)sg.nvalid / limit;
-    }
-    return share <= 1.0;
+    return B->few && g.impl == 4 && g.csplit && !c->debug_conv_stall;
 }
 
 // What happens after the inverse transform of a collide.
@@ -1590,6 +1598,8 @@ bte_status bte_autotune(bte_ctx *c, const double *f, const bte_instance *inst, i
                         for (int csplit : {1, 0}) {
                         if (!small_n && split != 4) continue;
                         if (csplit && (impl != 4 || (B->nsplit == 0 && !cells))) continue;
+                        // pairs in lanes: a kernel of its own, without these choices
+                        if (csplit && cells && (warps != 4 || stages != 1 || merge != 16)) continue;
                         // kinds of N = 48: variant 4, and 3 when they are the only kinds
                         if ((B->kinds_mask >> 7) && impl != 4 && !(impl == 3 && B->kinds_mask == (128u | 256u | 512u)))
                             continue;
