@@ -322,6 +322,12 @@ bte_status bte_graph_count(const bte_ctx *ctx, int64_t *count);
  *                      out: the call completes after about two seconds, the
  *                      next bte_sync_status returns BTE_ETIMEOUT and the
  *                      context stays usable (the test of the timeout path);
+ *       "debug_conv_parts" testing only: u > 0 cuts every item of variant 4 into
+ *                      block ranges of at most u blocks a warp instead of by
+ *                      the plan (drops the cached instance layouts);
+ *       "debug_conv_path" (read only) how the last FP32 collide's convolution ran:
+ *                      1 pairs in lanes (few cells), 2 items whole, 3 in
+ *                      halves, 4 in more parts, 0 none yet;
  *       "profile_mask" which kernels bte_profile_enable times, bit k for
  *                      conv32 (0), conv64 (1), collide (2), forward (3),
  *                      inverse (4), transport (5); default 63 (all).

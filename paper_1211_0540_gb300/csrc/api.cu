@@ -280,9 +280,8 @@ double queue_makespan(const std::vector<double> &cost, int S, int K, const doubl
 // one and no neighbour: fitted to measured launches of 12 values of u on 20 batch
 // shapes, where this choice loses 1 % to the best u on average. N = 16: 32 cells
 // 50.9 -> 35.4 us (u = 8), 56 cells 70.8 -> 52.7 (10), 96 cells 96.2 -> 68.0 (12), 128
-// cells 99.4 -> 86.4 (20), from 256 cells on every cut is slower; N = 12, 37 cells
-// 25.1 -> 22.3 (6). Small predicted gains are not taken (the wide kinds' first, where
-// 5 % predicted measured as 4 % lost).
+// cells 99.4 -> 86.4 (20), from 256 cells on every cut is slower. Small predicted gains are
+// not taken (the wide kinds' first, where 5 % predicted measured as 4 % lost).
 // out: the items in queue order; code[i]: ConvParams::split; *slots: parts' slots.
 void plan_splits(const bte_ctx *c, const std::vector<ConvItem> &items, std::vector<ConvItem> &out,
                  std::vector<int> &code, int *slots) {
@@ -295,10 +294,15 @@ void plan_splits(const bte_ctx *c, const std::vector<ConvItem> &items, std::vect
     const int K = wide ? 2 : 3, W = K * c->num_sms;
     static const double rate3[4] = {0.0, 1.5, 1.2, 1.0}, rate2[3] = {0.0, 1.25, 1.0};
     if (items.empty() || items.size() > (size_t)16 * W) return;  // long queues have no tail to cut
-    // N < 16: halves at most (37 cells N = 12, one collide: 45.9 us in halves, 47.0
-    // in three parts, for which the model predicts less)
+    // N < 16: halves at most; the model predicts more of three and more parts than they
+    // give, their blocks being short beside the reduction (a collide at N = 12, whole /
+    // halves / the best of 3 to 6 parts: 31 cells 43.0 / 36.8 / 35.9 us, 37 43.1 / 40.0 / 41.0,
+    // 64 43.1 / 40.7 / 41.1, 96 50.0 / 46.3 / 47.8, 128 52.0 / 51.0 / 53.2; N = 8, 57 to 160
+    // cells within 0.4 us)
+    const int forced = c->debug_conv_parts;
     auto parts_of = [&](const ConvItem &it, int u) {
-        const int per_warp = ((int)it.nblocks + 3) / 4, most = c->tables[it.table]->N < 16 ? 2 : (int)kMaxParts;
+        const int per_warp = ((int)it.nblocks + 3) / 4;
+        const int most = c->tables[it.table]->N < 16 && !forced ? 2 : (int)kMaxParts;
         return std::min((per_warp + u - 1) / u, most);
     };
     auto first_block = [](const ConvItem &it, int parts, int p) { return (uint32_t)((uint64_t)it.nblocks * p / parts); };
@@ -338,6 +342,7 @@ void plan_splits(const bte_ctx *c, const std::vector<ConvItem> &items, std::vect
             best_u = u;
         }
     }
+    if (forced) best_u = forced;
     if (best_u == whole) return;
     const std::vector<Piece> v = pieces(best_u);
     std::vector<int> first(items.size(), -1);
@@ -683,6 +688,7 @@ bte_status enqueue_collide(bte_ctx *c, Batch *B, const double *f, double *Q, int
         }
         prof_end(c, on, pe_conv, st);
     } else if (cells32) {
+        c->conv_path = CONV_FEW;
         const int on = prof_begin(c, PK_CONV32, st, &pe_conv);
         for (const Segment &sg : B->segs)
             launch_conv32_cells((const float2 *)c->scratch[SC_F], (float2 *)c->scratch[SC_QH], *c->tables[sg.table],
@@ -695,6 +701,7 @@ bte_status enqueue_collide(bte_ctx *c, Batch *B, const double *f, double *Q, int
         cudaError_t e = conv32_configure(B->kinds_mask, c->num_sms, cfg.warps, cfg.stages, cfg.impl, &L,
                                          parts_kernel(B, cfg));
         if (e != cudaSuccess) return cuda_fail(c, e, "convolution kernel configuration");
+        c->conv_path = !split ? CONV_WHOLE : B->d_halves && cfg.impl == 4 ? CONV_HALVES : CONV_PARTS;
         ConvParams p{};
         p.items = split ? B->d_items_split : B->d_items;
         p.nitems = split ? B->nitems_split : B->nitems;
@@ -1454,6 +1461,8 @@ static int *option_slot(bte_ctx *c, const char *name, int *lo, int *hi) {
     if (!std::strcmp(name, "conv_impl")) { *lo = 0; *hi = 5; return &c->conv_impl; }
     if (!std::strcmp(name, "dft_split")) { *lo = 0; *hi = 4; return &c->dft_split; }
     if (!std::strcmp(name, "debug_conv_stall")) { *lo = 0; *hi = 1; return &c->debug_conv_stall; }
+    if (!std::strcmp(name, "debug_conv_parts")) { *lo = 0; *hi = 1 << 20; return &c->debug_conv_parts; }
+    if (!std::strcmp(name, "debug_conv_path")) { *lo = 1; *hi = 0; return &c->conv_path; }  // read only
     if (!std::strcmp(name, "profile_mask")) { *lo = 0; *hi = 63; return &c->prof_mask; }
     if (!std::strcmp(name, "conv_warps")) { *lo = 1; *hi = 8; return &c->conv_warps; }
     if (!std::strcmp(name, "conv_stages")) { *lo = 0; *hi = 4; return &c->conv_stages; }
@@ -1473,8 +1482,12 @@ bte_status bte_set_option(bte_ctx *c, const char *name, int value) {
     if (!slot) return fail(c, BTE_EINVAL, std::string("unknown option ") + name);
     if (value < lo || value > hi) return fail(c, BTE_EINVAL, std::string("option out of range: ") + name);
     if (*slot != value) {
-        drop_graphs(c);
+        drop_graphs(c);  // waits for the context's work
         *slot = value;
+        if (slot == &c->debug_conv_parts) {  // the plans belong to the batches
+            for (auto &kv : c->batches) free_batch(kv.second);
+            c->batches.clear();
+        }
     }
     // an explicit choice of the FP32 path's configuration replaces the tuned ones
     if (!std::strncmp(name, "conv_", 5) || !std::strcmp(name, "dft_split")) {

@@ -166,6 +166,9 @@ struct GraphKey {
     bool operator<(const GraphKey &o) const;
 };
 
+// How a convolution ran: pairs in lanes, items whole, in halves, in more parts.
+enum ConvPath { CONV_NONE = 0, CONV_FEW, CONV_WHOLE, CONV_HALVES, CONV_PARTS };
+
 // One configuration of the FP32 path (convolution variant and launch shape,
 // compensated-merge interval, CTAs per cell of the fused transforms).
 struct ConvCfg {
@@ -241,6 +244,8 @@ struct bte_ctx {
     int conv_split = 1;        // variant 4: split items, few-cells kernel
     int dft_fuse_stages = 1;   // FP32 Heun step: stage 1's inverse transform also forms stage 2's forward
     int debug_conv_stall = 0;  // testing only: make the convolution's waits run out
+    int debug_conv_parts = 0;  // testing only: blocks a warp at which every item is cut (0: by the plan)
+    int conv_path = 0;         // how the last FP32 collide's convolution ran (ConvPath)
     std::string gpu_name;      // device name (key of saved tuning caches)
     std::map<std::string, bte::ConvCfg> tuned;  // autotuned configuration per batch shape
     bte::Mlp *mlp = nullptr;   // learned surrogate (bte_mlp_init)
