@@ -2,8 +2,8 @@
 // over the pairs of a block instead of over cells.
 //
 // The kernels of conv32_device.cuh give every cell a lane, so one cell costs as
-// much as 32 (N = 16: 43 us for 1 to 32 cells, 130 pencils of up to 128 blocks
-// for 456 CTAs). Here one CTA takes a (cell, pencil, k3 tile): its warps take the
+// much as 32 (a collide at N = 16: 55 us for 1 to 32 cells, 26 us for one cell here:
+// 130 pencils of up to 128 blocks for 456 CTAs). Here one CTA takes a (cell, pencil, k3 tile): its warps take the
 // pencil's (m1, m2) blocks in turn, and lane l the pairs l, l + 32, ... of a
 // block in the order of the weight table (for_pairs), so that weights are read
 // coalesced and a lane's pair t belongs to the same (m3, k3) in every block: it
@@ -176,17 +176,20 @@ int conv32_cells_entries(int N) {
     }
 }
 
-// Cells at which the two kernels take as long (measured per collide: N = 8, 64
-// cells 26.7 against 26.1 us; N = 12, 32 cells 41.9 / 42.0; N = 16, 16 cells 71.9 /
-// 67.8, 8 cells 48.7 / 67.6, 1 cell 29.7 / 69.7; N = 24, 8 cells 225 / 269; N = 32,
-// 8 cells 948 / 1157).
+// Up to this many cells no call is slower with pairs in lanes than with cells in lanes and
+// the items cut by their plan (us, pairs / cells in lanes, a collide and a Heun step:
+// N = 8, 56 cells 24.6 / 26.5 and 36.3 / 43.0, 64 cells 26.6 / 26.6 and 38.3 / 43.1; N = 12, 20
+// cells 33.8 / 36.0 and 57.4 / 61.7, 24 cells 36.0 / 36.3 and 63.6 / 61.5; N = 16, 1 cell 26 / 55,
+// 8 cells 47.1 / 55.5, 11 cells 55.3 / 55.5 and 100.3 / 104.8, 12 cells 59.3 / 55.2 and 105.7 /
+// 105.6; N = 24, 9 cells 246 / 266 and 501 / 549, 10 cells 269 / 266 and 547 / 547; N = 32, 10 cells
+// 1168 / 1234 and 2349 / 2474, 12 cells 1390 / 1226 and 2793 / 2473).
 int conv32_cells_limit(int N) {
     switch (N) {
         case 8: return 56;
-        case 12: return 30;
-        case 16: return 14;
+        case 12: return 22;
+        case 16: return 11;
         case 24: return 9;
-        case 32: return 9;
+        case 32: return 10;
         default: return 0;
     }
 }

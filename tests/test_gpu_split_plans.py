@@ -85,3 +85,20 @@ def test_fp64_single_cell_matches_oracle(bte, N, lam):
     c.sync_status()
     c.close()
     assert error(N, lam, f, Q) <= TOL64
+
+
+@pytest.mark.parametrize("N,few", [(8, 56), (12, 22), (16, 11), (24, 9), (32, 10)])
+def test_where_few_cells_end(bte, N, few):
+    """The last batch with pairs in lanes and the first with cells in lanes, where a call takes as long
+    either way (measured with the items cut by their plan); within the bar of one another."""
+    f = torch.from_numpy(inputs.precision_sweep_cells(N, L, few + 1, seed=5)).cuda()
+    c = bte.Context(0)
+    c.init_weights([(N, L, 1.0)])
+    Q = c.collide(f[:few], mode=bte.FP32)
+    assert c.get_option("debug_conv_path") == FEW
+    P = c.collide(f, mode=bte.FP32)
+    assert c.get_option("debug_conv_path") != FEW
+    c.sync_status()
+    c.close()
+    Qm = oracle.collide(N, L, 1.0, f[:1].cpu().numpy(), part=1, project=False)
+    assert float((P[0] - Q[0]).norm()) <= 2 * TOL32 * np.linalg.norm(Qm)
