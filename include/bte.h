@@ -305,7 +305,9 @@ bte_status bte_graph_count(const bte_ctx *ctx, int64_t *count);
  *                      resident CTAs); the part that finishes last adds all
  *                      parts' sums in a fixed order (deterministic), and
  *                      batches of few cells run a convolution with pairs
- *                      instead of cells in the lanes;
+ *                      instead of cells in the lanes; the parts' sums take up to
+ *                      58 MB of the context's scratch (8 KB a part, at most
+ *                      16 parts for every resident CTA);
  *                      0 runs every pencil whole;
  *       "learned_tol_ppm" fallback threshold of the learned mode in 1e-6 units;
  *       "dft_fuse_stages" 1 (default): in an FP32 Heun step the first stage's

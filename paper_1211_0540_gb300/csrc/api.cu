@@ -39,14 +39,13 @@ struct Batch {
     ConvItem *d_items = nullptr;
     int nitems = 0;
     // the same work with items split into block ranges (convolution variants 4, 5):
-    // items, split codes, the parts' sums (nsplit slots), counters ([0] the queue,
-    // [1 + first slot] the finished parts of a split item)
+    // items, split codes, counters ([0] the queue, [1 + first slot] the finished parts
+    // of a split item); the parts' sums (nsplit slots) go to the context's SC_PART
     ConvItem *d_items_split = nullptr;
     int *d_halves = nullptr;   // the split codes as halves, when no item has more parts
     int nitems_split = 0, nsplit = 0;
     bool few = false;          // few_cells()
     int *d_split = nullptr;
-    float *d_part = nullptr;
     unsigned *d_counters = nullptr;
     uint64_t last_use = 0;  // context tick of the latest lookup (least recently used is evicted first)
     unsigned kinds_mask = 0;
@@ -65,7 +64,7 @@ using namespace bte;
 
 namespace {
 
-enum ScratchId { SC_T1 = 0, SC_T2, SC_F, SC_QH, SC_FS, SC_Q1, SC_Q2, SC_MISC, SC_FB };
+enum ScratchId { SC_T1 = 0, SC_T2, SC_F, SC_QH, SC_FS, SC_Q1, SC_Q2, SC_MISC, SC_FB, SC_PART };
 
 // NVTX range over a host-side stage (enqueue of its launches; inside stream
 // capture it marks the capture, not the replays). A no-op without a profiler.
@@ -229,7 +228,6 @@ void free_batch(Batch *B) {
     cudaFree(B->d_items_split);
     cudaFree(B->d_split);
     cudaFree(B->d_halves);
-    cudaFree(B->d_part);
     cudaFree(B->d_counters);
     delete B;
 }
@@ -521,7 +519,6 @@ bte_status get_batch(bte_ctx *c, const bte_instance *inst, int64_t ninst, Batch 
         e = cudaMalloc(&B->d_items_split, sizeof(ConvItem) * split_items.size());
         if (e == cudaSuccess) e = cudaMalloc(&B->d_split, sizeof(int) * split_code.size());
         if (e == cudaSuccess && !halves.empty()) e = cudaMalloc(&B->d_halves, sizeof(int) * halves.size());
-        if (e == cudaSuccess) e = cudaMalloc(&B->d_part, sizeof(float) * kSplitFloats * (size_t)B->nsplit);
     }
     if (e == cudaSuccess) e = cudaMalloc(&B->d_counters, sizeof(unsigned) * (1 + (size_t)B->nsplit));
     if (e != cudaSuccess) {
@@ -585,6 +582,16 @@ bool parts_kernel(const Batch *B, const ConvCfg &g) {
     return g.impl == 4 && g.csplit && B->nsplit > 0 && !B->d_halves;
 }
 
+// The convolution with pairs in lanes is part of the split plan (conv_split 1) of variant 4.
+bool by_cells32(const bte_ctx *c, const Batch *B, const ConvCfg &g) {
+    return B->few && g.impl == 4 && g.csplit && !c->debug_conv_stall;
+}
+
+// Whether the convolution runs the batch's split item list.
+bool split_list(const bte_ctx *c, const Batch *B, const ConvCfg &g) {
+    return g.impl >= 4 && g.csplit && B->nsplit > 0 && !by_cells32(c, B, g);
+}
+
 // Allocate everything a collide/step on this batch needs (never inside capture).
 bte_status prepare(bte_ctx *c, Batch *B, int mode, bool step, bool transport) {
     bte_status s;
@@ -620,6 +627,9 @@ bte_status prepare(bte_ctx *c, Batch *B, int mode, bool step, bool transport) {
                 if (r != BTE_OK) return (bte_status)r;
             }
         }
+        if (split_list(c, B, g) &&
+            (s = ensure_scratch(c, SC_PART, sizeof(float) * kSplitFloats * (size_t)B->nsplit)) != BTE_OK)
+            return s;
         cudaError_t e = conv32_configure(B->kinds_mask, c->num_sms, g.warps, g.stages, g.impl, &L, parts_kernel(B, g));
         if (e != cudaSuccess) return cuda_fail(c, e, "convolution kernel configuration");
     }
@@ -630,10 +640,6 @@ bte_status prepare(bte_ctx *c, Batch *B, int mode, bool step, bool transport) {
 // half full one by one (lanes over the sum instead of cells).
 bool by_cells64(const Segment &sg) { return 2 * sg.nvalid <= sg.nslots; }
 
-// The convolution with pairs in lanes is part of the split plan (conv_split 1) of variant 4.
-bool by_cells32(const bte_ctx *c, const Batch *B, const ConvCfg &g) {
-    return B->few && g.impl == 4 && g.csplit && !c->debug_conv_stall;
-}
 
 // What happens after the inverse transform of a collide.
 enum Post { POST_RAW = 0, POST_PROJECT = 1, POST_STAGE1 = 2, POST_STAGE2 = 3 };
@@ -697,7 +703,7 @@ bte_status enqueue_collide(bte_ctx *c, Batch *B, const double *f, double *Q, int
         count_launches(c, (int)B->segs.size());
     } else {
         ConvLaunch L;
-        const bool split = cfg.impl >= 4 && cfg.csplit && B->nsplit > 0;
+        const bool split = split_list(c, B, cfg);
         cudaError_t e = conv32_configure(B->kinds_mask, c->num_sms, cfg.warps, cfg.stages, cfg.impl, &L,
                                          parts_kernel(B, cfg));
         if (e != cudaSuccess) return cuda_fail(c, e, "convolution kernel configuration");
@@ -709,7 +715,7 @@ bte_status enqueue_collide(bte_ctx *c, Batch *B, const double *f, double *Q, int
         if (split) {
             p.split = B->d_split;
             p.halves = B->d_halves;
-            p.part = B->d_part;
+            p.part = (float *)c->scratch[SC_PART];
             p.split_cnt = B->d_counters + 1;
         }
         p.F = (const float2 *)c->scratch[SC_F];
