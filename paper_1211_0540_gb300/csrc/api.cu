@@ -64,7 +64,7 @@ using namespace bte;
 
 namespace {
 
-enum ScratchId { SC_T1 = 0, SC_T2, SC_F, SC_QH, SC_FS, SC_Q1, SC_Q2, SC_MISC, SC_FB, SC_PART };
+enum ScratchId { SC_T1 = 0, SC_MOM, SC_F, SC_QH, SC_FS, SC_Q1, SC_Q2, SC_MISC, SC_FB, SC_PART };
 
 // NVTX range over a host-side stage (enqueue of its launches; inside stream
 // capture it marks the capture, not the replays). A no-op without a profiler.
@@ -597,8 +597,18 @@ bte_status prepare(bte_ctx *c, Batch *B, int mode, bool step, bool transport) {
     bte_status s;
     const size_t ce = (size_t)B->n_celem;
     const size_t csz = mode == BTE_FP64_PLAIN ? sizeof(double2) : sizeof(float2);
-    for (int id : {SC_T1, SC_T2, SC_F, SC_QH})
+    for (int id : {SC_F, SC_QH})
         if ((s = ensure_scratch(c, id, ce * csz)) != BTE_OK) return s;
+    // the transforms of dft.cu: a pass's result, and the planes' moment sums of one segment
+    // at a time (the segments follow one another on the stream)
+    size_t mom = 0;
+    for (const Segment &sg : B->segs) {
+        const int N = c->tables[sg.table]->N;
+        if (mode == BTE_FP64_PLAIN || !fused_dft_supported(N))
+            mom = std::max(mom, sizeof(double) * 5 * N * (size_t)sg.nslots);
+    }
+    if (mom && ((s = ensure_scratch(c, SC_T1, ce * csz)) != BTE_OK || (s = ensure_scratch(c, SC_MOM, mom)) != BTE_OK))
+        return s;
     if (step || transport) {
         for (int id : {SC_FS, SC_Q1, SC_Q2})
             if ((s = ensure_scratch(c, id, sizeof(double) * (size_t)B->extent)) != BTE_OK) return s;
@@ -769,9 +779,8 @@ bte_status enqueue_collide(bte_ctx *c, Batch *B, const double *f, double *Q, int
             continue;
         }
         // post - 1: the projection's mode (ProjArgs), -1 for the raw Qt
-        double *mom = fp64 ? (double *)((double2 *)c->scratch[SC_T2] + sg.eoff)
-                           : (double *)((float2 *)c->scratch[SC_T2] + sg.eoff);
-        count_launches(c, launch_dft_inverse(c->scratch[SC_QH], B->d_slot_off, ds, si, c->scratch[SC_T1], mom, Q,
+        count_launches(c, launch_dft_inverse(c->scratch[SC_QH], B->d_slot_off, ds, si, c->scratch[SC_T1],
+                                             (double *)c->scratch[SC_MOM], Q,
                                              fp64 && by_cells64(sg), proj_args(t), post - 1, x, y, qp, a, st));
     }
     prof_end(c, on_inv, pe_inv, st);

@@ -51,3 +51,20 @@ def test_calls_that_read_no_parts_hold_none(bte):
         c.project(f[:n])
     assert held(free0) <= 16 * MB
     c.close()
+
+
+@pytest.mark.parametrize("mode,N,cells,arrays", [("FP32", 16, 1024, 2), ("FP64_PLAIN", 16, 512, 3)])
+def test_transforms_hold_what_they_use(bte, mode, N, cells, arrays):
+    """Beside the state, fhat and Qhat (one complex value a grid point), in FP64 one pass's result."""
+    c = bte.Context(0)
+    c.init_weights([(N, L, 1.0)])
+    f = torch.from_numpy(inputs.precision_sweep_cells(N, L, 1, seed=1)).cuda()
+    c.collide(f, mode=getattr(bte, mode))  # weight tables
+    g = f.repeat(cells, 1)
+    Q = torch.empty_like(g)
+    free0 = torch.cuda.mem_get_info()[0]
+    c.collide(g, Q, mode=getattr(bte, mode))
+    c.sync_status()
+    each = cells * N ** 3 * (8 if mode == "FP32" else 16)
+    assert held(free0) <= arrays * each + 20 * MB
+    c.close()
