@@ -49,22 +49,16 @@ PROFILES = os.path.join(ROOT, "profiles")
 
 
 def conv_pairs_per_cell(n):
-    """Unordered (zeta, {xi, zeta - xi}) pairs the FP32 kernel evaluates per cell: one pencil
-    (k1, k2) of each mirror pair, blocks (m1, m2) <= (n1, n2) of the pencil's and its mirror's box,
-    partner indices mod n."""
+    """Unordered (zeta, {xi, zeta - xi}) pairs of the FP32 convolution per cell: those with a weight, and the
+    entries of weight 0 that the kernel visits besides. One pencil (k1, k2) of each mirror pair,
+    blocks (m1, m2) <= (n1, n2) of the pencil's and its mirror's box, partner indices mod n; a block of
+    one of the two boxes alone has weights only where that one holds (k3, m3)."""
     h = n // 2
-
-    def mirror(i):
-        return (n - i) % n
-
-    def on(k, m):
-        return 0 <= k - m + h < n
-
-    def onm(k, m):
-        return on(mirror(k), mirror(m))
-
-    row = sum(on(k, m) or onm(k, m) for k in range(n) for m in range(n))
-    blocks = 0
+    on = [[0 <= k - m + h < n for m in range(n)] for k in range(n)]
+    onm = [[on[(n - k) % n][(n - m) % n] for m in range(n)] for k in range(n)]
+    row = sum(map(sum, on))          # (k3, m3) of one box; its mirror holds as many
+    union = sum(on[k][m] or onm[k][m] for k in range(n) for m in range(n))
+    both = one = 0
     for k1 in range(n):
         for k2 in range(n):
             if not (k1 > h or (k1 in (0, h) and (k2 == 0 or k2 >= h))):
@@ -76,8 +70,11 @@ def conv_pairs_per_cell(n):
                 for m2 in range(n):
                     if m1 == n1 and m2 > (k2 - m2 + h) % n:
                         continue
-                    blocks += (on(k1, m1) and on(k2, m2)) or (onm(k1, m1) and onm(k2, m2))
-    return blocks * row
+                    a, b = on[k1][m1] and on[k2][m2], onm[k1][m1] and onm[k2][m2]
+                    both += a and b
+                    one += a != b
+    pairs = both * union + one * row
+    return pairs, (both + one) * union - pairs
 
 
 def parse():
@@ -406,7 +403,7 @@ def main():
                            "cells_checked": pick, "norm": "||Q - Q_oracle|| / ||Q_loss_oracle||",
                            "fp32_max_abs_moment": float(np.abs(mom).max())}
 
-    conv_pairs = conv_pairs_per_cell(N)
+    conv_pairs, zero_pairs = conv_pairs_per_cell(N)
     flops_per_launch = 10.0 * conv_pairs * NX
     conv_avg_ms = conv_ms / max(conv_n, 1)
     achieved = flops_per_launch / (conv_avg_ms * 1e-3) / 1e12
@@ -429,7 +426,8 @@ def main():
                      "peak_basis": _peak_basis(clk, fma), "measured_fma": fma,
                      "frac_of_measured_ffma2": achieved / fma["fp32_ffma2_tflops"],
                      "flops_per_launch": flops_per_launch,
-                     "flop_unit": "10 flops per evaluated (zeta, {xi, zeta-xi}) pair per cell",
+                     "flop_unit": "10 flops per (zeta, {xi, zeta-xi}) pair with a weight per cell",
+                     "zero_weight_flops_per_launch": 10.0 * zero_pairs * NX,
                      "conv_ms_per_launch": conv_avg_ms, "conv_launches_timed": conv_n},
         "stage_ms_per_step": dict({k: v / args.steps for k, v in part_ms.items()},
                                   note="separate pass with events around every stage (each figure includes "
@@ -639,7 +637,7 @@ def run_sweep32(args, ctx, torch, bte, inputs, oracle, stream, flush, sampler, n
     relp = np.linalg.norm(Qg[pick] - Qo, axis=1) / np.linalg.norm(Qo, axis=1)
     peak, clk = _alu_peak(clocks)
     fma = _measured_fma(ctx, stream)
-    pairs = conv_pairs_per_cell(n)
+    pairs, _ = conv_pairs_per_cell(n)
     conv_ms = conv[0] / max(conv[1], 1)
     achieved = 10.0 * pairs * nc / (conv_ms * 1e-3) / 1e12
     wl = ("precision sweep: %d bi-Maxwellian cells (means ~ U(-1.5,1.5)^3, T ~ U(0.5,2), seed 3), "
@@ -697,7 +695,7 @@ def run_uneven(args, ctx, torch, bte, inputs, oracle, stream, flush, sampler):
     tot = float(sum(ms))
     evals = 2 * len(items)
     value = evals * args.steps / (tot * 1e-3)
-    flops_step = sum(2 * 10.0 * conv_pairs_per_cell(n) for (n, _, _) in items)
+    flops_step = sum(2 * 10.0 * conv_pairs_per_cell(n)[0] for (n, _, _) in items)
     conv_ms = t / max(k, 1)
     peak, clk = _alu_peak(clocks)
     fma = _measured_fma(ctx, stream)

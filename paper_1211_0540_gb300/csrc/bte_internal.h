@@ -43,8 +43,9 @@ inline ConvKind conv_kind(int id) {
 // modes of index 0, whose mirror is themselves). The convolutions evaluate
 // one pencil (k1, k2) of each mirror pair with these weights; the inverse
 // transforms take the other pencil as 0. Pencils that are their own mirror
-// carry half the weight at every k3. At N = 16: 130 of 256 pencils, 2.46 instead
-// of 3.56 million pairs per cell.
+// carry half the weight at every k3. At N = 16: 130 of 256 pencils, 2.34 instead
+// of 3.55 million pairs per cell (and 0.08 million entries of weight 0, of blocks
+// that only one of the two sums holds).
 // ----------------------------------------------------------------------------
 constexpr int mode_mirror(int i, int N) { return i == 0 ? 0 : N - i; }
 // n = k - m + N/2 on the grid, and its index mod N

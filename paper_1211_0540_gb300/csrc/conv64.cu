@@ -4,7 +4,7 @@
 // at the modes of the stored pencils (half spectrum, bte_internal.h). The FP64
 // units bound it (two FMAs per SM and clock against 128 in FP32), six
 // operations a pair, so what counts is the number of pairs: 2.42 M per cell at
-// N = 16 instead of the 7.08 M terms of the plain sum over m (128 cells: 10.09
+// N = 16 (0.08 M with weight 0) instead of the 7.08 M terms of the plain sum over m (128 cells: 10.09
 // -> 3.2 ms; six warp instructions of 16 clocks a pair on 152 SMs are 2.95 ms).
 // A zeta point's terms are listed block by block ((m1, m2) of its pencil), its
 // m_count values of m3 from m_first on (mod N), with the weights in that order;
