@@ -407,7 +407,8 @@ bte_status bte_tc_gemm(bte_ctx *ctx, const void *A, const void *B, float *D, int
  *   decay to lr/20, weight decay). *final_loss: mean square error of the last batch.
  * bte_mlp_grads: one forward/backward on the first n pairs without an update;
  *   copies the gradient (nparams floats) to host_grads and the loss to *loss.
- * bte_mlp_infer: Q_nn for n cells (device FP64; no projection).
+ * bte_mlp_infer: Q_nn for n cells (device FP64; no projection). Asynchronous; refused
+ *   (BTE_ECUDA) on a stream that is being captured.
  * bte_mlp_get/set_params: host FP32 vector of nparams values.
  * The surrogate is used by bte_collide and bte_step with mode BTE_LEARNED
  * (projection and fallback there). Errors: BTE_EINVAL, BTE_ESTATE (no surrogate), BTE_ENOMEM, BTE_ECUDA. */

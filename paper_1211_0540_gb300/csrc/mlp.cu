@@ -779,6 +779,12 @@ bte_status bte_mlp_infer(bte_ctx *c, const double *f, double *Q, int64_t n, void
     if (!f || !Q || n <= 0 || n > 65536) return mlp_fail(c, BTE_EINVAL, "bte_mlp_infer: bad arguments");
     cudaSetDevice(c->device);
     cudaStream_t st = (cudaStream_t)stream;
+    // a graph would keep the activations, which a larger batch later frees
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return mlp_fail(c, BTE_ECUDA, "bte_mlp_infer: the stream is being captured");
+    }
     if (!m->ensure_batch((int)n)) return mlp_fail(c, BTE_ENOMEM, "bte_mlp_infer: activations");
     if (m->run(f, nullptr, (int)n, false, c->d_status, st, m->rowuni)) return mlp_fail(c, BTE_ECUDA, "bte_mlp_infer: launch");
     launch_mlp_post(m->Y, m->rho, m->rowuni, (int)n, m->M, m->s_out, Q, st);
