@@ -525,18 +525,17 @@ bte_status get_batch(bte_ctx *c, const bte_instance *inst, int64_t ninst, Batch 
         free_batch(B);
         return fail(c, BTE_ENOMEM, std::string("batch allocation: ") + cudaGetErrorString(e));
     }
-    e = cudaMemcpy(B->d_slot_off, slot_off.data(), sizeof(int64_t) * slot_off.size(), cudaMemcpyHostToDevice);
+    e = upload(B->d_slot_off, slot_off.data(), sizeof(int64_t) * slot_off.size());
     if (e == cudaSuccess)
-        e = cudaMemcpy(B->d_slot_out, slot_out.data(), sizeof(int64_t) * slot_out.size(), cudaMemcpyHostToDevice);
+        e = upload(B->d_slot_out, slot_out.data(), sizeof(int64_t) * slot_out.size());
     if (e == cudaSuccess && !sorted.empty())
-        e = cudaMemcpy(B->d_items, sorted.data(), sizeof(ConvItem) * sorted.size(), cudaMemcpyHostToDevice);
+        e = upload(B->d_items, sorted.data(), sizeof(ConvItem) * sorted.size());
     if (e == cudaSuccess && B->nsplit > 0) {
-        e = cudaMemcpy(B->d_items_split, split_items.data(), sizeof(ConvItem) * split_items.size(),
-                       cudaMemcpyHostToDevice);
+        e = upload(B->d_items_split, split_items.data(), sizeof(ConvItem) * split_items.size());
         if (e == cudaSuccess)
-            e = cudaMemcpy(B->d_split, split_code.data(), sizeof(int) * split_code.size(), cudaMemcpyHostToDevice);
+            e = upload(B->d_split, split_code.data(), sizeof(int) * split_code.size());
         if (e == cudaSuccess && !halves.empty())
-            e = cudaMemcpy(B->d_halves, halves.data(), sizeof(int) * halves.size(), cudaMemcpyHostToDevice);
+            e = upload(B->d_halves, halves.data(), sizeof(int) * halves.size());
     }
     if (e != cudaSuccess) {
         free_batch(B);
@@ -841,7 +840,7 @@ bte_status wall_table(bte_ctx *c, const Table *t, double Tw, int side, const dou
         double *d = nullptr;
         cudaError_t e = cudaMalloc(&d, sizeof(double) * M);
         if (e != cudaSuccess) return cuda_fail(c, e, "wall table allocation");
-        e = cudaMemcpy(d, mw.data(), sizeof(double) * M, cudaMemcpyHostToDevice);
+        e = upload(d, mw.data(), sizeof(double) * M);
         if (e != cudaSuccess) {
             cudaFree(d);
             return cuda_fail(c, e, "wall table upload");
@@ -901,7 +900,7 @@ bte_status grid_coefficients(bte_ctx *c, const double *dx, int nx, TransportArgs
         double *d = nullptr;
         cudaError_t e = cudaMalloc(&d, sizeof(double) * h.size());
         if (e != cudaSuccess) return cuda_fail(c, e, "transport grid allocation");
-        e = cudaMemcpy(d, h.data(), sizeof(double) * h.size(), cudaMemcpyHostToDevice);
+        e = upload(d, h.data(), sizeof(double) * h.size());
         if (e != cudaSuccess) {
             cudaFree(d);
             return cuda_fail(c, e, "transport grid upload");

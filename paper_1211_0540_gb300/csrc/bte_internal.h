@@ -74,6 +74,14 @@ constexpr bool pencil_self_mirrored(int k1, int k2, int N) {
     return (k1 == 0 || k1 == N / 2) && (k2 == 0 || k2 == N / 2);
 }
 
+// Host to device, complete on return: cudaMemcpy from pageable memory may return while
+// its last part is still on the way, in the legacy stream, for which callers'
+// (non-blocking) streams do not wait.
+inline cudaError_t upload(void *dst, const void *src, size_t bytes) {
+    const cudaError_t e = cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice);
+    return e == cudaSuccess ? cudaStreamSynchronize(cudaStreamLegacy) : e;
+}
+
 int first_kind_for_N(int N);  // -1 if unsupported
 int tiles_for_N(int N);
 constexpr int kMaxTiles = 3;

@@ -283,7 +283,7 @@ void upload_root(const V (&sym)[N]) {
         r[t].x = (decltype(r[t].x))std::cos(th);
         r[t].y = (decltype(r[t].y))std::sin(th);
     }
-    cudaMemcpyToSymbol(sym, r, sizeof(r));
+    upload_symbol(sym, r);
 }
 
 template <int N, class V>

@@ -667,7 +667,7 @@ void upload_roots(const float2 (&sym)[N]) {
         const double th = 2.0 * 3.14159265358979323846 * t / N;
         h[t] = make_float2((float)std::cos(th), (float)std::sin(th));
     }
-    cudaMemcpyToSymbol(sym, h, sizeof(h));
+    upload_symbol(sym, h);
 }
 }  // namespace
 

@@ -18,6 +18,13 @@ struct DftSeg {
     bool cells = false;
 };
 
+// As upload (bte_internal.h), into a __constant__ array.
+template <class V, size_t N>
+cudaError_t upload_symbol(const V (&sym)[N], const V (&src)[N]) {
+    const cudaError_t e = cudaMemcpyToSymbol(sym, src, sizeof(src));
+    return e == cudaSuccess ? cudaStreamSynchronize(cudaStreamLegacy) : e;
+}
+
 // Projection (Sec. 3.3), optionally fused with the RK2 update:
 // mode 0: Q <- P Q;  mode 1: Q <- P Q, Y <- X + a Q;  mode 2: Q <- P Q, Y <- Y + a (Qp + Q).
 struct ProjArgs {

@@ -513,12 +513,12 @@ int build_indicator_table(const Table &t, int modes, uint64_t seed, IndicatorTab
     cudaError_t e = cudaMalloc(&out.d_w, sizeof(float) * std::max<size_t>(w.size(), 4));
     if (e == cudaSuccess) e = cudaMalloc(&out.d_desc, sizeof(uint32_t) * std::max<size_t>(desc.size(), 1));
     if (e == cudaSuccess)
-        e = cudaMemcpy(out.d_desc, desc.data(), sizeof(uint32_t) * desc.size(), cudaMemcpyHostToDevice);
+        e = upload(out.d_desc, desc.data(), sizeof(uint32_t) * desc.size());
     if (e == cudaSuccess) e = cudaMalloc(&out.d_pen, sizeof(IndPencil) * S);
-    if (e == cudaSuccess) e = cudaMemcpy(out.d_w, w.data(), sizeof(float) * w.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(out.d_pen, pens.data(), sizeof(IndPencil) * S, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = upload(out.d_w, w.data(), sizeof(float) * w.size());
+    if (e == cudaSuccess) e = upload(out.d_pen, pens.data(), sizeof(IndPencil) * S);
     if (e == cudaSuccess) e = cudaMalloc(&out.d_kk, sizeof(int) * S);
-    if (e == cudaSuccess) e = cudaMemcpy(out.d_kk, kks.data(), sizeof(int) * S, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = upload(out.d_kk, kks.data(), sizeof(int) * S);
     // shared memory of the cross-warp reduction (set outside any stream capture)
     if (e == cudaSuccess) e = cudaFuncSetAttribute(indicator_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ind_smem<8>());
     if (e == cudaSuccess) e = cudaFuncSetAttribute(indicator_kernel<12>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ind_smem<12>());

@@ -337,8 +337,7 @@ bool Mlp::ensure_batch(int B) {
               A((void **)&dH2, 4 * bh) && A((void **)&dH1, 4 * bh) && A((void **)&dZf, 4 * bh) &&
               A((void **)&rho, 8 * (size_t)Bp) && A((void **)&loss_rows, 8 * (size_t)Bp) &&
               A((void **)&rowuni, 8 * (size_t)Bp) &&
-              cudaMemcpy(rowuni, uni.data(), 8 * (size_t)Bp, cudaMemcpyHostToDevice) == cudaSuccess &&
-              cudaStreamSynchronize(nullptr) == cudaSuccess;  // callers' streams do not wait for the legacy stream
+              upload(rowuni, uni.data(), 8 * (size_t)Bp) == cudaSuccess;  // waits for the memsets too
     if (ok) bcap = Bp;
     return ok;
 }
@@ -611,7 +610,7 @@ bte_status bte_mlp_init(bte_ctx *c, int table, int width, uint64_t seed) {
     fill(m->off_W1(), m->H, m->M, std::sqrt(2.0f / m->M));
     fill(m->off_W2(), m->H, m->H, std::sqrt(1.0f / m->H));
     fill(m->off_W3(), m->M, m->H, 0.5f * std::sqrt(1.0f / m->H));
-    if (cudaMemcpy(m->params, h.data(), 4 * P, cudaMemcpyHostToDevice) != cudaSuccess ||
+    if (upload(m->params, h.data(), 4 * P) != cudaSuccess ||
         cudaMemset(m->adam_m, 0, 4 * P) != cudaSuccess || cudaMemset(m->adam_v, 0, 4 * P) != cudaSuccess ||
         cudaMemset(m->grads, 0, 4 * P) != cudaSuccess) {
         delete m;
@@ -687,7 +686,7 @@ bte_status bte_mlp_set_params(bte_ctx *c, const float *host, int64_t n) {
     if (s != BTE_OK) return s;
     if (!host || n != (int64_t)c->mlp->nparams()) return mlp_fail(c, BTE_EINVAL, "bte_mlp_set_params: size");
     cudaSetDevice(c->device);
-    if (cudaMemcpy(c->mlp->params, host, 4 * (size_t)n, cudaMemcpyHostToDevice) != cudaSuccess)
+    if (upload(c->mlp->params, host, 4 * (size_t)n) != cudaSuccess)
         return mlp_fail(c, BTE_ECUDA, "bte_mlp_set_params: copy");
     c->mlp->refresh_bf16(0);
     if (cudaDeviceSynchronize() != cudaSuccess) return mlp_fail(c, BTE_ECUDA, "bte_mlp_set_params: cast");

@@ -378,19 +378,19 @@ int build_table(Table &t, std::string &err) {
         return BTE_ENOMEM;
     }
     if (e == cudaSuccess && !tmpl.empty())
-        e = cudaMemcpy(t.d_tmpl, tmpl.data(), sizeof(ConvItem) * tmpl.size(), cudaMemcpyHostToDevice);
+        e = upload(t.d_tmpl, tmpl.data(), sizeof(ConvItem) * tmpl.size());
     if (e == cudaSuccess && !I32.empty())
-        e = cudaMemcpy(t.d_I32, I32.data(), sizeof(float) * I32.size(), cudaMemcpyHostToDevice);
+        e = upload(t.d_I32, I32.data(), sizeof(float) * I32.size());
     if (e == cudaSuccess && !J32.empty())
-        e = cudaMemcpy(t.d_J32, J32.data(), sizeof(float) * J32.size(), cudaMemcpyHostToDevice);
+        e = upload(t.d_J32, J32.data(), sizeof(float) * J32.size());
     if (e == cudaSuccess && ne)
-        e = cudaMemcpy(t.d_ent, ent.data(), sizeof(uint16_t) * ent.size(), cudaMemcpyHostToDevice);
+        e = upload(t.d_ent, ent.data(), sizeof(uint16_t) * ent.size());
     if (e == cudaSuccess && ne)
-        e = cudaMemcpy(t.d_rk, rk.data(), sizeof(int16_t) * rk.size(), cudaMemcpyHostToDevice);
+        e = upload(t.d_rk, rk.data(), sizeof(int16_t) * rk.size());
     if (e == cudaSuccess && !etab.empty())
-        e = cudaMemcpy(t.d_etab, etab.data(), sizeof(uint16_t) * etab.size(), cudaMemcpyHostToDevice);
+        e = upload(t.d_etab, etab.data(), sizeof(uint16_t) * etab.size());
     if (e == cudaSuccess)
-        e = cudaMemcpy(t.d_desc, desc.data(), sizeof(uint32_t) * t.n_desc, cudaMemcpyHostToDevice);
+        e = upload(t.d_desc, desc.data(), sizeof(uint32_t) * t.n_desc);
     if (e != cudaSuccess) {
         err = std::string("cudaMemcpy (weight table): ") + cudaGetErrorString(e);
         free_table(t);
@@ -442,7 +442,7 @@ int build_table_fp32(Table &t, std::string &err) {
         err = std::string("cudaMalloc (FP32 weight table): ") + cudaGetErrorString(e);
         return BTE_ENOMEM;
     }
-    e = cudaMemcpy(t.d_w32, w32.data(), sizeof(float) * t.n_w32, cudaMemcpyHostToDevice);
+    e = upload(t.d_w32, w32.data(), sizeof(float) * t.n_w32);
     if (e != cudaSuccess) {
         err = std::string("cudaMemcpy (FP32 weight table): ") + cudaGetErrorString(e);
         return BTE_ECUDA;
@@ -511,8 +511,8 @@ int build_table_fp64(Table &t, std::string &err) {
         t.d_zeta64 = nullptr;
         return BTE_ENOMEM;
     }
-    e = cudaMemcpy(t.d_w64, w.data(), sizeof(double) * t.n_w64, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(t.d_zeta64, z.data(), sizeof(Zeta64) * z.size(), cudaMemcpyHostToDevice);
+    e = upload(t.d_w64, w.data(), sizeof(double) * t.n_w64);
+    if (e == cudaSuccess) e = upload(t.d_zeta64, z.data(), sizeof(Zeta64) * z.size());
     if (e != cudaSuccess) {
         err = std::string("cudaMemcpy (FP64 weight table): ") + cudaGetErrorString(e);
         return BTE_ECUDA;
