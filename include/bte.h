@@ -407,6 +407,9 @@ bte_status bte_tc_gemm(bte_ctx *ctx, const void *A, const void *B, float *D, int
  *   decay to lr/20, weight decay). *final_loss: mean square error of the last batch.
  * bte_mlp_grads: one forward/backward on the first n pairs without an update;
  *   copies the gradient (nparams floats) to host_grads and the loss to *loss.
+ *   A host_grads of 4 MB or more whose pages are not all mapped yet is filled by up
+ *   to 12 host threads through 24 MB of pinned memory, which the first such
+ *   call allocates and the surrogate keeps (a plain copy where that fails).
  * bte_mlp_infer: Q_nn for n cells (device FP64; no projection). Asynchronous; refused
  *   (BTE_ECUDA) on a stream that is being captured.
  * bte_mlp_get/set_params: host FP32 vector of nparams values.

@@ -492,13 +492,18 @@ bte_status need_mlp(bte_ctx *c) {
     return BTE_OK;
 }
 
-// Whether every page of a host buffer is mapped (false also where it cannot be told).
+// Whether every page of a host buffer is mapped (true also where it cannot be told:
+// not plain memory, which cudaMemcpy knows).
 bool pages_mapped(const void *p, size_t bytes) {
-    const uintptr_t page = (uintptr_t)sysconf(_SC_PAGESIZE), a = (uintptr_t)p / page * page;
-    std::vector<unsigned char> in(((uintptr_t)p + bytes - a + page - 1) / page);
-    if (mincore((void *)a, (uintptr_t)p + bytes - a, in.data()) != 0) return true;  // not plain memory: cudaMemcpy
-    for (unsigned char c : in)
-        if (!(c & 1)) return false;
+    constexpr size_t kPages = 512;
+    unsigned char in[kPages];
+    const uintptr_t page = (uintptr_t)sysconf(_SC_PAGESIZE), end = (uintptr_t)p + bytes;
+    for (uintptr_t a = (uintptr_t)p / page * page; a < end; a += kPages * page) {
+        const size_t len = std::min<size_t>(end - a, kPages * page);
+        if (mincore((void *)a, len, in) != 0) return true;
+        for (size_t i = 0; i < (len + page - 1) / page; ++i)
+            if (!(in[i] & 1)) return false;
+    }
     return true;
 }
 
