@@ -147,7 +147,6 @@ struct Table {
     // output j), [tile][pair_visits][T], -1 if none
     uint16_t *d_ent = nullptr;
     int16_t *d_rk = nullptr;
-    // DFT roots exp(2 pi i t / N), t in [0, N)
     // Projection: (C C^T)^{-1}, row-major 5x5 (C without the dv^3 factor folded in)
     double ainv[25];
     // Host FP64 radial tables on integer invariants (kept for the lazy FP64 table)

@@ -12,7 +12,7 @@ struct DftSeg {
     int s0;        // first slot of the segment (global slot index)
     int nslots;    // slots in the segment (multiple of 32)
     int64_t eoff;  // complex-element offset of slot s0 in scratch / group buffers
-    int nvalid = 0;  // slots that hold a cell, the first ones (read by the transforms of dft.cu only)
+    int nvalid = 0;  // slots that hold a cell, the first ones (read by the transforms of dft.cu and with cells)
     // FP32 fhat and Qhat cell-major ([slot][m], the convolution with pairs in
     // lanes) instead of the group layout
     bool cells = false;
