@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "../../include/bte.h"
+#include "radial.h"
 
 namespace bte {
 
@@ -162,7 +163,7 @@ struct Table {
     double ghat(int k1, int k2, int k3, int m1, int m2, int m3) const;  // FP64, no dz^3
     // Gv(k, m) + Gv(k*, m*), halved on self-mirrored pencils (half-spectrum convolution); no dz^3
     double half_weight(int k1, int k2, int k3, int m1, int m2, int m3) const;
-    double gain_inelastic(double a, double b) const;                    // I(a, b) off the lattice
+    double gain_inelastic(radial::Dd s, radial::Dd t) const;            // I(hz s, hz t) off the lattice
 };
 
 struct GraphKey {

@@ -16,6 +16,8 @@ namespace radial {
 
 constexpr double kPi = 3.14159265358979323846;
 
+// The closed forms as they are printed, at any arguments (what the host check of the
+// quadrature compares with; the tables take Lattice below).
 struct Radial {
     double L, lam;
     double C(double k) const {
@@ -36,6 +38,68 @@ struct Radial {
         if (b == 0.0) return J(a);
         return (C(a - b) - C(a + b)) / (2.0 * a * b);
     }
+};
+
+// A number as the sum of two doubles.
+struct Dd {
+    double hi, lo;
+};
+inline Dd dd_sum(Dd a, Dd b) {  // TwoSum (Knuth) of the leading parts, then the parts normalised
+    const double s = a.hi + b.hi, t = s - a.hi, e = ((a.hi - (s - t)) + (b.hi - t)) + (a.lo + b.lo), h = s + e;
+    return {h, e - (h - s)};
+}
+inline Dd dd_mul(Dd a, Dd b) {
+    const double p = a.hi * b.hi;
+    return {p, std::fma(a.hi, b.hi, -p) + (a.hi * b.lo + a.lo * b.hi)};
+}
+inline Dd dd_sqrt(Dd x) {
+    const double h = std::sqrt(x.hi);
+    return {h, h != 0.0 ? (std::fma(-h, h, x.hi) + x.lo) / (2.0 * h) : 0.0};
+}
+inline Dd dd_sqrt(int n) { return dd_sqrt(Dd{(double)n, 0.0}); }
+
+// The closed forms at a = hz s, b = hz t with hz L = pi / 2 (s = sqrt p, t = sqrt q on the
+// grid's lattice): the phases (a +- b) L = (pi / 2)(s +- t) are reduced from two
+// doubles, so that the sines are those of the arguments themselves. (Phases formed in
+// one double are off by up to 1e-16 of their own size, which was the largest part of
+// the FP64 operator's error: one cell N = 16 lambda = 1 2.6e-15 of Q, now 2.0e-15.)
+struct Lattice {
+    double L, lam, hz;
+    // sin and cos of (pi / 2) t
+    static void sincos(Dd t, double &s, double &c) {
+        const double q = std::nearbyint(t.hi), x = 0.5 * kPi * ((t.hi - q) + t.lo);
+        const double sx = std::sin(x), cx = std::cos(x);
+        switch ((int)std::fmod(q, 4.0) & 3) {
+            case 0: s = sx; c = cx; break;
+            case 1: s = cx; c = -sx; break;
+            case 2: s = -sx; c = -cx; break;
+            default: s = -cx; c = sx; break;
+        }
+    }
+    double C(Dd t) const {  // k = hz t
+        if (t.hi == 0.0) return lam == 0.0 ? L : 0.5 * L * L;
+        const double k = hz * t.hi;
+        double s, c, h;
+        sincos(t, s, c);
+        if (lam == 0.0) return s / k;
+        sincos({0.5 * t.hi, 0.5 * t.lo}, h, c);
+        return L * s / k - 2.0 * h * h / (k * k);
+    }
+    double J(Dd t) const {  // J(hz t)
+        if (t.hi == 0.0) return std::pow(L, lam + 3.0) / (lam + 3.0);
+        const double x = 0.5 * kPi * t.hi, k = hz * t.hi;
+        double s, c;
+        sincos(t, s, c);
+        if (lam == 0.0) return (s - x * c) / (k * k * k);
+        return (2.0 * x * s - (x * x - 2.0) * c - 2.0) / (k * k * k * k);
+    }
+    double I(Dd s, Dd t) const {  // I(hz s, hz t)
+        if (s.hi == 0.0) return J(t);
+        if (t.hi == 0.0) return J(s);
+        return (C(dd_sum(s, {-t.hi, -t.lo})) - C(dd_sum(s, t))) / (2.0 * hz * hz * s.hi * t.hi);
+    }
+    double J(int n) const { return J(dd_sqrt(n)); }  // J(hz sqrt n)
+    double I(int p, int q) const { return I(dd_sqrt(p), dd_sqrt(q)); }
 };
 
 // Plain panel rule: composite Clenshaw-Curtis on [0, L], uniform panels of at

@@ -42,14 +42,12 @@
 #include <vector>
 
 #include "bte_internal.h"
-#include "radial.h"
 
 namespace bte {
 
 namespace {
 
 using radial::kPi;
-using radial::Radial;
 using radial::sinc;
 
 // I[p][q] = int_0^L r^(lam+2) sinc(a_p r) sinc(b_q r) dr and J[s] = I[0][4s]
@@ -59,6 +57,9 @@ using radial::sinc;
 // on [h, L] sum_i A_p[i] sinc(b_q r_i), A_p[i] = w_i sinc(a_p r_i). J is read
 // off the same sums, so Ghat(xi, 0) = I(0, |xi|) - J(|xi|) is exactly 0.
 void quadrature_tables(Table &t, double hz) {
+    // hz + hzl = pi / (2 L) (kPiLo: pi - kPi)
+    constexpr double kPiLo = 1.2246467991473532e-16;
+    const double hzl = 0.5 * (std::fma(-t.dz, t.L, kPi) + kPiLo) / t.L;
     using radial::kSeriesTerms;
     constexpr int K = kSeriesTerms;
     const int nrow = std::max(t.nq, 4 * (t.ns - 1) + 1);
@@ -69,7 +70,13 @@ void quadrature_tables(Table &t, double hz) {
 #pragma omp parallel for schedule(static)
     for (int q = 0; q < nrow; ++q) {
         const double b = hz * std::sqrt((double)q);
-        for (size_t i = 0; i < nn; ++i) S[(size_t)q * nn + i] = sinc(b * R.r[i]);
+        // b r from two doubles: the rounding of b is the same at every node, so it adds up
+        const radial::Dd sq = radial::dd_sqrt(q);
+        const double bl = std::fma(hz, sq.hi, -b) + hz * sq.lo + hzl * sq.hi;
+        for (size_t i = 0; i < nn; ++i) {
+            const double x = b * R.r[i], xl = std::fma(b, R.r[i], -x) + bl * R.r[i];
+            S[(size_t)q * nn + i] = x == 0.0 ? 1.0 : (std::sin(x) + xl * (std::cos(x) - std::sin(x) / x)) / x;
+        }
         double c[K];
         radial::series_coeffs(b, R.h, c);
         for (int j = 0; j < K; ++j) C[(size_t)q * K + j] = c[j];
@@ -87,7 +94,11 @@ void quadrature_tables(Table &t, double hz) {
     auto value = [&](int p, int q) {
         const double *a = &A[(size_t)p * nn], *b = &S[(size_t)q * nn];
         double rest = 0.0;
-        for (size_t i = 0; i < nn; ++i) rest += a[i] * b[i];
+        for (size_t i0 = 0; i0 < nn; i0 += 25) {  // panel by panel: the rule's many terms round less that way
+            double panel = 0.0;
+            for (size_t i = i0; i < std::min(i0 + 25, nn); ++i) panel += a[i] * b[i];
+            rest += panel;
+        }
         const double *wp = &W[(size_t)p * K], *cq = &C[(size_t)q * K];
         double first = 0.0;
         for (int j = K - 1; j >= 0; --j) first += wp[j] * cq[j];
@@ -126,14 +137,14 @@ double Table::ghat(int k1, int k2, int k3, int m1, int m2, int m3) const {
     }
     if (beta == 1.0) return std::sqrt(2.0 / kPi) * (I[(size_t)p * nq + q] - J[s]);
     // inelastic: gain arguments a = beta |zeta| / 2, b = |xi - beta zeta / 2| (Eq. GHat_calc)
-    const double hz = 0.5 * dz;
-    double b2 = 0.0;
+    using radial::Dd;
+    const Dd bt{beta, 0.0};
+    Dd b2{0.0, 0.0};
     for (int d = 0; d < 3; ++d) {
-        const double c = 2.0 * m[d] - beta * k[d];
-        b2 += c * c;
+        const Dd bk = radial::dd_mul(bt, {(double)k[d], 0.0}), c = radial::dd_sum({2.0 * m[d], 0.0}, {-bk.hi, -bk.lo});
+        b2 = radial::dd_sum(b2, radial::dd_mul(c, c));
     }
-    const double a = beta * hz * std::sqrt((double)p), b = hz * std::sqrt(b2);
-    return std::sqrt(2.0 / kPi) * (gain_inelastic(a, b) - J[s]);
+    return std::sqrt(2.0 / kPi) * (gain_inelastic(radial::dd_mul(bt, radial::dd_sqrt(p)), radial::dd_sqrt(b2)) - J[s]);
 }
 
 // Where both sums hold the pair, their weights are equal: the two lifts of an
@@ -152,9 +163,10 @@ double Table::half_weight(int k1, int k2, int k3, int m1, int m2, int m3) const 
 // The closed form loses digits when a b L^2 is small (C(a - b) and C(a + b)
 // nearly cancel); such pairs (|xi - beta zeta / 2| near 0, which the elastic
 // lattice never produces) take the quadrature rule instead.
-double Table::gain_inelastic(double a, double b) const {
-    Radial R{L, lam};
-    if (a == 0.0 || b == 0.0 || b * L >= 0.25) return R.I(a, b);
+double Table::gain_inelastic(radial::Dd s, radial::Dd t) const {
+    const radial::Lattice R{L, lam, 0.5 * dz};
+    const double a = R.hz * s.hi, b = R.hz * t.hi;
+    if (a == 0.0 || b == 0.0 || b * L >= 0.25) return R.I(s, t);
     return radial::I_quad(lam, L, a, b);
 }
 
@@ -196,17 +208,11 @@ int build_table(Table &t, std::string &err) {
     t.I.assign((size_t)t.np * t.nq, 0.0);
     t.J.assign(t.ns, 0.0);
     if (integer_lam) {
-        Radial R{t.L, t.lam};
+        const radial::Lattice R{t.L, t.lam, hz};
 #pragma omp parallel for schedule(dynamic, 4)
-        for (int p = 0; p < t.np; ++p) {
-            double a = hz * std::sqrt((double)p);
-            for (int q = 0; q < t.nq; ++q) {
-                if ((p - q) % 2 != 0) continue;  // q = |2m'-k'|^2 has the parity of |k'|^2
-                double b = hz * std::sqrt((double)q);
-                t.I[(size_t)p * t.nq + q] = R.I(a, b);
-            }
-        }
-        for (int s = 0; s < t.ns; ++s) t.J[s] = R.J(hz * std::sqrt((double)(4 * s)));
+        for (int p = 0; p < t.np; ++p)
+            for (int q = (p & 1); q < t.nq; q += 2) t.I[(size_t)p * t.nq + q] = R.I(p, q);  // q has the parity of p
+        for (int s = 0; s < t.ns; ++s) t.J[s] = R.J(4 * s);
     } else {
         quadrature_tables(t, hz);
     }
