@@ -291,10 +291,10 @@ bte_status bte_graph_count(const bte_ctx *ctx, int64_t *count);
  *                      resident CTAs per SM of a one-block ring);
  *       "conv_merge"  blocks accumulated in plain FP32 between compensated
  *                      (TwoSum) merges (>= 1, default 16), an upper bound: the
- *                      kernels merge every block at N = 8 and every third at N = 16,
- *                      and at N = 12, 24 and 32 the blocks are summed one by one
- *                      first (variants 4 and 5; the others merge at least every 2
- *                      blocks at N = 12, every 4 at N = 24 and 32);
+ *                      kernels merge every block at N = 8, at least every third
+ *                      at N = 16 and every sixth at N = 32, and at N = 12 and 24 the
+ *                      blocks are summed one by one first (variants 4 and 5; the
+ *                      others merge at least every 2 and every 4 blocks there);
  *       "batch_cache" instance layouts kept (2..2^20, default 64; see
  *                      bte_batch_count);
  *       "graph_cache" captured step graphs kept (1..2^20, default 32; see

@@ -71,14 +71,15 @@ struct Kind {
     // spectrum's sums merged every 16 blocks. Error relative to that one, merged every
     // 16 / 8 / 4 / 2 / 1 blocks, 128 to 2048 cells: N = 8 1.07 / 1.06 / 1.05 / 1.03 / 0.99,
     // N = 12 1.12 / 1.08 / 1.05 / 0.98, N = 16 1.08 / 1.05 / 1.01 / 0.95 / 0.89 (every 3:
-    // 0.96), N = 24 1.05 / 1.01 / 0.98, N = 32 1.06 / 1.02 / 0.97; with block sums 0.96, 0.91 and
-    // 0.92 at N = 12, 24, 32. Block sums cost 16 additions a block and registers: a collide of 1024
-    // cells N = 12 176 (every 16) -> 181 us (every 2: 191), 128 cells N = 24 869 -> 875 us
-    // and N = 32 4.39 -> 4.63 ms (every 4: 4.70). N = 16 has no registers left for them
-    // (1024 cells 638 -> 706 us; merges every 3 blocks 667), N = 8 needs a merge every block
-    // (2048 cells 73 -> 80 us). N = 48 is within the bound at 16.
-    static constexpr int merge_most = N == 8 ? 1 : N == 12 ? 2 : N == 16 ? 3 : N == 48 ? 1 << 20 : 4;
-    static constexpr bool block_sums = N == 12 || N == 24 || N == 32;
+    // 0.96), N = 24 1.05 / 1.01 / 0.98, N = 32 1.06 / 1.02 / 0.97 (every 6: 0.98); with block sums
+    // 0.96 and 0.91 at N = 12 and 24. Block sums cost T additions a block and registers: a
+    // collide of 1024 cells N = 12 176 (every 16) -> 181 us (every 2: 191), 512 cells N = 24
+    // 3.28 -> 3.30 ms (every 4: 3.40). N = 32 and 16 have no registers left for them (256 cells
+    // N = 32 8.68 -> 9.06 ms, merges every 6 blocks 8.81; 1024 cells N = 16 638 -> 706 us,
+    // every 3 blocks 667), N = 8 needs a merge every block (2048 cells 73 -> 80 us). N = 48
+    // is within the bound at 16.
+    static constexpr int merge_most = N == 8 ? 1 : N == 12 ? 2 : N == 16 ? 3 : N == 24 ? 4 : N == 32 ? 6 : 1 << 20;
+    static constexpr bool block_sums = N == 12 || N == 24;
     static constexpr int cpad = (count() + 3) & ~3;
     static constexpr int row_bytes = N * kLanes * 8;
     static constexpr int stage_bytes = 2 * row_bytes + cpad * 4;
