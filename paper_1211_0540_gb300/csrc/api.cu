@@ -95,9 +95,14 @@ bool owned_by_graph(const bte_ctx *c, cudaEvent_t ev) {
     return false;
 }
 
-// Record the context's fence on `st` after the work a call enqueued there.
+// Record the context's fence on `st` after the work a call enqueued there. Not on a stream
+// that is being captured, by the context or by the caller: an event recorded there
+// cannot be waited for, so that the next quiesce would fail.
 void fence_record(bte_ctx *c, cudaStream_t st) {
     if (c->capturing) return;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cudaGetLastError();
+    if (cap != cudaStreamCaptureStatusNone) return;
     auto it = c->fence.find(st);
     if (it == c->fence.end()) {
         if (c->fence.size() >= 64) {  // many streams: wait for all and start over
