@@ -281,9 +281,9 @@ double queue_makespan(const std::vector<double> &cost, int S, int K, const doubl
 // the SM) a block costs its entries + 40, an item 300 (first copies, reduction), a
 // part 450 (its sums go through L2), and a CTA runs 1.2 and 1.5 times as fast with
 // one and no neighbour: fitted to measured launches of 12 values of u on 20 batch
-// shapes, where this choice loses 1 % to the best u on average. N = 16: 32 cells
-// 50.9 -> 35.4 us (u = 8), 56 cells 70.8 -> 52.7 (10), 96 cells 96.2 -> 68.0 (12), 128
-// cells 99.4 -> 86.4 (20), from 256 cells on every cut is slower. Small predicted gains are
+// shapes, where this choice loses 1 % to the best u on average. A collide at N = 16, whole
+// against cut: 32 cells 66.2 -> 51.7 us (u = 8), 56 cells 89.9 -> 73.0 (10), 96 cells 116.4 ->
+// 91.4 (12), 128 cells 121.3 -> 107.2 (20), from 256 cells on every cut is slower. Small predicted gains are
 // not taken (the wide kinds' first, where 5 % predicted measured as 4 % lost).
 // out: the items in queue order; code[i]: ConvParams::split; *slots: parts' slots.
 void plan_splits(const bte_ctx *c, const std::vector<ConvItem> &items, std::vector<ConvItem> &out,

@@ -648,17 +648,18 @@ void prepare_n() {
     prepare_one<N, 4>();
 }
 // CTAs per cell: as asked (1, 2, else 4), or with 0 (the default) four while the
-// cells are few and one once they alone give about 5 warps per SM, from where it is the
-// faster one (forward + inverse, 4 against 1 CTAs per cell: N = 16, 56 cells 27.4 / 28.6
-// us, 128 31.5 / 29.2, 1024 129.6 / 110.4; N = 12, 128 cells 25.1 / 23.1, 512 47.7 / 35.3;
-// N = 8, 256 cells 19.8 / 20.1, 1024 46.1 / 26.2).
-constexpr int kOneCtaWarps = 5;  // per SM
+// cells are few and one once they alone give 5 warps per SM (N = 16) or 2 (N = 8, 12),
+// from where it is the faster one (a collide in us, 4 / 1 CTAs per cell: N = 16, 64 cells
+// 72.9 / 75.0, 96 90.6 / 91.2, 128 108.6 / 106.6, 1024 687 / 664; N = 12, 32 cells 30.9 / 31.0,
+// 64 36.3 / 35.1, 128 47.6 / 43.8, 512 120.3 / 101.3; N = 8, 64 cells 20.7 / 20.8, 128 22.8 /
+// 21.8, 192 24.8 / 23.5, 320 34.1 / 26.9, 1024 62.2 / 44.1).
+constexpr int one_cta_warps(int N) { return N < 16 ? 2 : 5; }  // per SM
 int norm_split(int split, const DftSeg &s) {
     if (split != 0) return split == 1 || split == 2 ? split : 4;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return (int64_t)grid_slots(s) * ((s.N * s.N + 31) / 32) >= (int64_t)kOneCtaWarps * sms ? 1 : 4;
+    return (int64_t)grid_slots(s) * ((s.N * s.N + 31) / 32) >= (int64_t)one_cta_warps(s.N) * sms ? 1 : 4;
 }
 template <int N>
 void upload_roots(const float2 (&sym)[N]) {
